@@ -636,9 +636,10 @@ __global__ void __launch_bounds__(kRedThreads) k_totals_part(const S* __restrict
   double acc[5] = {0, 0, 0, 0, 0};
   for (unsigned long long i = blockIdx.x * (unsigned long long)kRedThreads + threadIdx.x; i < nodes;
        i += (unsigned long long)kRedBlocks * kRedThreads) {
-    NodeMacro m;
-    stored_moments<S, Q>(lat, nodes, i, m);
-    acc[0] += m.N0; acc[1] += m.T00; acc[2] += m.Mx; acc[3] += m.My; acc[4] += m.Mz;
+    double t[5];
+    stored_totals<S, Q>(lat, nodes, i, t);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) acc[c] += t[c];
   }
   __shared__ double sh[5][kRedThreads];
 #pragma unroll

@@ -25,6 +25,7 @@
 
 #include "../../include/rlb.h"
 #include "rlb_internal.h"
+#include "rlb_io.cuh"
 #include "rlb_node.cuh"
 
 using namespace rlb;
@@ -53,16 +54,10 @@ __global__ void __launch_bounds__(kThreads) k_part(const S* __restrict__ lat, un
   const unsigned long long hi = lo + kNodesPerBlock < nodes ? lo + kNodesPerBlock : nodes;
   double acc[5] = {0, 0, 0, 0, 0};
   for (unsigned long long i = lo + threadIdx.x; i < hi; i += kThreads) {
-    S f[19], g[19];
+    double t[5];
+    stored_totals<S>(lat, nodes, i, t);
 #pragma unroll
-    for (int a = 0; a < 19; ++a) {
-      f[a] = lat[(unsigned long long)a * nodes + i];
-      g[a] = lat[(19ull + a) * nodes + i];
-    }
-    double sp[9], dp[9], Sa, Sd;
-    NodeMacro m;
-    node_moments<S>(f, g, sp, dp, Sa, Sd, m);
-    acc[0] += m.N0; acc[1] += m.T00; acc[2] += m.Mx; acc[3] += m.My; acc[4] += m.Mz;
+    for (int c = 0; c < 5; ++c) acc[c] += t[c];
   }
   __shared__ double sh[5][kThreads];
 #pragma unroll

@@ -547,6 +547,11 @@ constexpr unsigned long long kSixth = 0x2AAAAAAAAAAAAAABull;       // ceil(2^64 
 constexpr unsigned long long kTwoThirds = 0xAAAAAAAAAAAAAAABull;   // ceil(2^65 / 3)
 constexpr unsigned long long kEighteenth = 0x0E38E38E38E38E39ull;  // ceil(2^64 / 18)
 constexpr unsigned long long kSignBit = 0x8000000000000000ull;
+// D2Q9 weights
+constexpr unsigned long long kFourNinths = 0x71C71C71C71C71C8ull;  // ceil(2^66 / 9)
+constexpr unsigned long long kNinth = 0x1C71C71C71C71C72ull;       // ceil(2^64 / 9)
+constexpr unsigned long long kTwelfth = 0x1555555555555556ull;     // ceil(2^64 / 12)
+constexpr unsigned long long k36th = 0x071C71C71C71C71Dull;        // ceil(2^64 / 36)
 
 // floor(a b / 2^64) for unsigned a, b without the low partial products: low by at most 2.
 __device__ __forceinline__ unsigned long long mulhi(unsigned long long a, unsigned long long b) {
@@ -756,10 +761,121 @@ __device__ __forceinline__ void relax_links_store(const long long (&X)[19], cons
     }
   }
 }
+
+// ---- stored populations of either precision on a node's grid (field output, totals)
+
+// Unit of the integer grid: a value is X 2^(E - bias) with E the largest biased exponent
+// of its distribution, |X| < 2^57; in_range: exponents for which the FP64 form's T00^2 (and
+// with it what that form accepts) and every result stay normal.
+template <typename S> struct FxUnit;
+template <> struct FxUnit<double> {
+  static constexpr int bias = 1079;
+  static __device__ __forceinline__ bool in_range(int E) { return E >= 543 && E <= 1503; }
+};
+template <> struct FxUnit<float> {
+  static constexpr int bias = 183;
+  static __device__ __forceinline__ bool in_range(int E) { return E >= 1 && E <= 254; }
+};
+// Largest biased exponent of a distribution, and whether every value is positive, finite
+// and within 2^24 of the largest (the short conversion then applies).
+template <int N>
+__device__ __forceinline__ int max_exponent(const double (&v)[N], bool& fast) {
+  int hi = __double2hiint(v[0]), lo = hi;
+#pragma unroll
+  for (int a = 1; a < N; ++a) {
+    hi = max(hi, __double2hiint(v[a]));
+    lo = min(lo, __double2hiint(v[a]));
+  }
+  fast = lo > 0 && hi < 0x7ff00000 && lo >= (((hi >> 20) - 24) << 20);
+  if (fast) return hi >> 20;
+  unsigned m = 0;
+#pragma unroll
+  for (int a = 0; a < N; ++a) m = max(m, (unsigned)__double2hiint(v[a]) & 0x7fffffffu);
+  return (int)(m >> 20);
+}
+template <int N>
+__device__ __forceinline__ int max_exponent(const float (&v)[N]) {
+  unsigned m = 0;
+#pragma unroll
+  for (int a = 0; a < N; ++a) m = max(m, __float_as_uint(v[a]) & 0x7fffffffu);
+  return (int)(m >> 23);
+}
+__device__ __forceinline__ long long grid_value(double x, int E) { return to_fixed(x, E + 7); }
+// 24-bit significand at 2^33 times the value's distance from the grid's top exponent
+__device__ __forceinline__ long long grid_value(float x, int E) {
+  const unsigned b = __float_as_uint(x);
+  const int ex = (int)((b >> 23) & 0xffu);
+  const unsigned m = (b & 0x7fffffu) | (ex ? 0x800000u : 0u);
+  const int sh = min(E - max(ex, 1), 63);
+  return with_sign(((unsigned long long)m << 33) >> sh, b >> 31);
+}
+
+// ---- square root and reciprocals of 1 - u^2 (as w = (1 - u^2) 2^62, 0 < w <= 2^62)
+
+// rho = (a 2^-64)^(-1/2) as rho 2^61 for a in [2^60, 2^64): FP32 seed, two Newton steps
+__device__ __forceinline__ unsigned long long rsqrt_fixed(unsigned long long a) {
+  unsigned long long Y = fixed_from_float<61>(rsqrt_approx(top_float(a)));
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const unsigned long long q = mulhi(a, mulhi(Y, Y));
+    Y = mulhi(Y, (3ull << 62) - (q << 4)) << 1;
+  }
+  return Y;
+}
+// 2^126 / h for h in (1.5 2^62, 2^64): FP32 seed, two Newton steps
+__device__ __forceinline__ unsigned long long rcp_fixed(unsigned long long h) {
+  unsigned long long R = fixed_from_float<62>(rcp_approx(top_float(h)));
+#pragma unroll
+  for (int it = 0; it < 2; ++it) R = mulhi(R, (1ull << 63) - mulhi(h, R)) << 2;
+  return R;
+}
+// even shift that brings w into [2^61, 2^63)
+__device__ __forceinline__ int even_shift(unsigned long long w) { return (__clzll((long long)w) - 1) & ~1; }
+// sqrt(1 - u^2) = Sq 2^(-63 - h)
+__device__ __forceinline__ unsigned long long sqrt_one_minus(unsigned long long w, int& h) {
+  const int sh = even_shift(w);
+  const unsigned long long a = w << sh;
+  h = sh >> 1;
+  return mulhi(a, rsqrt_fixed(a)) << 3;
+}
+
+// K * 2^U rounded to the nearest float (ties to even); the result must be in the normal
+// range.  `near` is set where |K| is within tol (a power of two, at most 2^22) of a
+// rounding tie, or below 2^32 tol: there a value off by less than tol units may round the
+// other way (and the result is not used).
+__device__ __forceinline__ float fixed_to_f32(long long K, int U, unsigned tol, bool& near) {
+  const unsigned neg = (unsigned)((unsigned long long)K >> 63);
+  const unsigned long long a = (unsigned long long)with_sign((unsigned long long)K, neg);
+  const unsigned kh = (unsigned)(a >> 32), kl = (unsigned)a;
+  const int lz = __clz(kh);
+  const unsigned top = __funnelshift_l(kl, kh, lz), low = kl << lz;   // |K| 2^lz, bit 63 set
+  // the 40 bits below the 24-bit significand against their half, at 2^8 per unit
+  const unsigned t = (tol << lz) >> 8;
+  near |= (__funnelshift_l(low, top, 24) - 0x80000000u + t) <= 2u * t || kh < tol;
+  const unsigned r = __float_as_uint(__uint2float_rn(top | (low != 0u ? 1u : 0u))) + ((unsigned)(U + 32 - lz) << 23);
+  return __uint_as_float(r | (neg << 31));
+}
 }  // namespace fx
 
 using fx::EqPieces;
 using fx::UFix;
+
+// D2Q9 class constants of a distribution on its grid (weights 4/9, 1/9, 1/36; Eqs. 7,
+// 32-33), with X_i, Y_ij, Z_i of eq_pieces and SX = D u^2 / 4:
+//   rest r;  axis i: ev = KA + 2 X_i, od = 2 Z_i;  diagonal: ev = KD +- Y, od = (Z_x +- Z_y)/2.
+struct Eq9 {
+  long long r, KA, KD;
+};
+template <bool G>
+__device__ __forceinline__ void eq9_pieces(unsigned long long D, long long Pf, long long SX, Eq9& w) {
+  using namespace fx;
+  const unsigned long long P = (unsigned long long)Pf;
+  const long long s3 = (long long)mulhi((unsigned long long)SX, kThird);
+  const long long s83 = 2 * SX + (long long)mulhi((unsigned long long)SX, kTwoThirds);   // (2/3) D u^2
+  w.r = (G ? (long long)D - 2 * Pf - (long long)mulhi(P, kTwoThirds) : (long long)mulhi(D, kFourNinths)) - s83;
+  w.KA = (G ? (long long)mulhi(P, kThird) : (long long)mulhi(D, kNinth)) - 2 * s3;
+  w.KD = (G ? (long long)mulhi(P, kTwelfth) : (long long)mulhi(D, k36th)) + s3;
+}
 
 // Velocity on the fixed grid: |u_i| 2^63 and sign bits, and the six products
 // u_i^2 2^62, |u_i u_j| 2^62 the equilibria need.
@@ -799,18 +915,11 @@ __device__ __forceinline__ unsigned long long fx_recover(long long T00, long lon
   const unsigned long long a = t2 - 3ull * (badr ? 0ull : m2q);  // (A/4) 2^(2 nsh - 64), in (2^60, 2^64)
   // rho = (a 2^-64)^(-1/2) in (1, 4) as Y = rho 2^61 (< 2^63 even for a seed of 4):
   // Y <- Y (3 - a Y^2) / 2
-  unsigned long long Y = fixed_from_float<61>(rsqrt_approx(top_float(a)));
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const unsigned long long q = mulhi(a, mulhi(Y, Y));          // a rho^2 2^58
-    Y = mulhi(Y, (3ull << 62) - (q << 4)) << 1;
-  }
+  const unsigned long long Y = rsqrt_fixed(a);                 // a rho^2 2^58 per Newton step
   const unsigned long long Sq = mulhi(a, Y) << 3;              // sqrt(A/4) 2^nsh, in (2^62, 2^64)
   const unsigned long long h = (Tn >> 1) + (Sq >> 1);          // H 2^(nsh - 1), in (1.5 2^62, 2^64)
   // R = 2^126 / h: R <- R (2 - h R 2^-126)
-  unsigned long long R = fixed_from_float<62>(rcp_approx(top_float(h)));
-#pragma unroll
-  for (int it = 0; it < 2; ++it) R = mulhi(R, (1ull << 63) - mulhi(h, R)) << 2;
+  const unsigned long long R = rcp_fixed(h);
   // |u_i| 2^63 = (3/4)(|M_i| 2^nsh / h) 2^63 = (3/2) mulhi(|M_i| 2^nsh, R)
   const unsigned long long ux = mulhi(mxn, R), uy = mulhi(myn, R), uz = mulhi(mzn, R);
   u.ax = ux + (ux >> 1);
@@ -1571,6 +1680,109 @@ __device__ __forceinline__ void node_equilibrium_d2q9(double e, double ux, doubl
     g[2 * p + 1] = ge + go;
     g[2 * p + 2] = ge - go;
   }
+}
+
+// ---------------------------------------------------------------------------
+// Equilibrium of given FP64 fields on integers (the same sums as node_equilibrium):
+// gamma^2 and gamma from 1 - u^2 by fixed-point Newton steps, sigma = (4/3) e gamma^2 and
+// N0 = n gamma with their top bit at 2^60-2^62, so a unit is at most 2^-60 of them (FP64
+// rounding of each of the ~8 operations per link is 2^-53 of its terms).  g is
+// value 2^Ug, f is value 2^Uf.
+struct FxEquilibrium {
+  UFix u;
+  unsigned long long sig, N0;
+  long long Pf;
+  int Ug, Uf;
+  unsigned tol;   // units the FP64 form may be off by (FP32 results): 2^15 gamma^2
+};
+// False where e, n or |u| leave the range of this form (or are invalid): e and n normal
+// and, NARROW (FP32 results), within 2^60 of 1; 1 - u^2 >= 2^-32 (NARROW: 2^-7).
+template <bool NARROW>
+__device__ __forceinline__ bool fx_equilibrium_of(double e, double ux, double uy, double uz, double n,
+                                                  FxEquilibrium& q) {
+  using namespace fx;
+  const int eh = __double2hiint(e), nh = __double2hiint(n);
+  const int xh = __double2hiint(ux) & 0x7fffffff, yh = __double2hiint(uy) & 0x7fffffff,
+            zh = __double2hiint(uz) & 0x7fffffff;
+  constexpr int lo = NARROW ? 963 : 128, hi = NARROW ? 1083 : 1900;
+  bool ok = eh >= (lo << 20) && eh < (hi << 20) && nh >= (lo << 20) && nh < (hi << 20) && max(xh, max(yh, zh)) < 0x3ff00000;
+  q.u.ax = to_fixed_abs(ux, 1023);
+  q.u.ay = to_fixed_abs(uy, 1023);
+  q.u.az = to_fixed_abs(uz, 1023);
+  q.u.sx = (unsigned)__double2hiint(ux) >> 31;
+  q.u.sy = (unsigned)__double2hiint(uy) >> 31;
+  q.u.sz = (unsigned)__double2hiint(uz) >> 31;
+  ufix_products(q.u);
+  const unsigned long long s = q.u.xx + q.u.yy + q.u.zz;         // u^2 2^62
+  ok = ok && s < (1ull << 62) - (1ull << 30);
+  const unsigned long long w = ok ? (1ull << 62) - s : 1ull << 62;
+  const unsigned long long me = ((unsigned long long)(((unsigned)__double2hiint(e) & 0xfffffu) | 0x100000u) << 43) |
+                                ((unsigned long long)(unsigned)__double2loint(e) << 11);
+  const unsigned long long mn = ((unsigned long long)(((unsigned)__double2hiint(n) & 0xfffffu) | 0x100000u) << 43) |
+                                ((unsigned long long)(unsigned)__double2loint(n) << 11);
+  const int ee = (eh >> 20) & 0x7ff, en = (nh >> 20) & 0x7ff;
+  const int lzw = __clzll((long long)w);
+  const unsigned long long R = rcp_fixed(w << lzw);              // gamma^2 2^(64 - lzw)
+  q.sig = mulhi(mulhi(me, R), kTwoThirds);                       // sigma / 2 2^(1086 - ee - lzw)
+  q.Ug = ee + lzw - 1085;
+  q.Pf = (long long)(mulhi(me, kThird) >> (1 + lzw));            // P = e / 3
+  const int sh = even_shift(w);
+  q.N0 = mulhi(mn, rsqrt_fixed(w << sh));                        // n gamma 2^(1084 - en - sh / 2)
+  q.Uf = en - 1084 + (sh >> 1);
+  q.tol = NARROW ? (1u << 14) << min(lzw, 8) : 0u;
+  return ok && !(NARROW && lzw > 8);
+}
+// One distribution (G: g) written to out[a * stride].  FP32 results: true where one of them
+// lies so near a rounding tie that the FP64 form may round it the other way (about one
+// node in 2^13); the caller then takes that form, so that the stored FP32 state is the
+// FP64 equilibrium rounded once, bit for bit.
+template <typename S, bool INT>
+__device__ __forceinline__ S fx_round(long long K, int U, unsigned tol, bool& near) {
+  if constexpr (sizeof(S) == 4) return fx::fixed_to_f32(K, U, tol, near);
+  else if constexpr (INT) return fx::from_fixed_pos(K, U + 1079);
+  else return fx::from_fixed_dp(K, U + 1079);
+}
+template <typename S, int Q, bool G>
+__device__ __forceinline__ bool fx_equilibrium_store(const FxEquilibrium& e, S* __restrict__ out,
+                                                     unsigned long long stride) {
+  using namespace fx;
+  const unsigned long long D = G ? e.sig : e.N0;
+  const int U = G ? e.Ug : e.Uf;
+  EqPieces q;
+  eq_pieces(D, e.u, q);
+  const long long SX = q.Xx + q.Xy + q.Xz;
+  constexpr bool INT = !G;
+  bool near = false;
+  if constexpr (Q == 19) {
+    const long long w = G ? (long long)mulhi((unsigned long long)e.Pf, kSixth) : (long long)mulhi(D, kEighteenth);
+    const long long KA = w - (long long)mulhi((unsigned long long)SX, kThird), KD = KA >> 1;
+    const long long r = G ? (long long)D - 3 * e.Pf - 2 * SX : (long long)mulhi(D, kThird) - 2 * SX;
+    out[0] = fx_round<S, INT>(r, U, e.tol, near);
+    const long long ev[9] = {KA + q.Xx, KA + q.Xy, KA + q.Xz,
+                             KD + ((q.Xx + q.Xy) >> 1) + q.Yxy, KD + ((q.Xx + q.Xy) >> 1) - q.Yxy,
+                             KD + ((q.Xx + q.Xz) >> 1) + q.Yxz, KD + ((q.Xx + q.Xz) >> 1) - q.Yxz,
+                             KD + ((q.Xy + q.Xz) >> 1) + q.Yyz, KD + ((q.Xy + q.Xz) >> 1) - q.Yyz};
+    const long long od[9] = {q.Zx, q.Zy, q.Zz,
+                             (q.Zx + q.Zy) >> 1, (q.Zx - q.Zy) >> 1, (q.Zx + q.Zz) >> 1, (q.Zx - q.Zz) >> 1,
+                             (q.Zy + q.Zz) >> 1, (q.Zy - q.Zz) >> 1};
+#pragma unroll
+    for (int p = 0; p < 9; ++p) {
+      out[(unsigned long long)(2 * p + 1) * stride] = fx_round<S, INT>(ev[p] + od[p], U, e.tol, near);
+      out[(unsigned long long)(2 * p + 2) * stride] = fx_round<S, INT>(ev[p] - od[p], U, e.tol, near);
+    }
+  } else {
+    Eq9 w;
+    eq9_pieces<G>(D, e.Pf, SX, w);
+    out[0] = fx_round<S, INT>(w.r, U, e.tol, near);
+    const long long ev[4] = {w.KA + 2 * q.Xx, w.KA + 2 * q.Xy, w.KD + q.Yxy, w.KD - q.Yxy};
+    const long long od[4] = {2 * q.Zx, 2 * q.Zy, (q.Zx + q.Zy) >> 1, (q.Zx - q.Zy) >> 1};
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      out[(unsigned long long)(2 * p + 1) * stride] = fx_round<S, INT>(ev[p] + od[p], U, e.tol, near);
+      out[(unsigned long long)(2 * p + 2) * stride] = fx_round<S, INT>(ev[p] - od[p], U, e.tol, near);
+    }
+  }
+  return near;
 }
 
 }  // namespace rlb
