@@ -12,8 +12,8 @@
 //     and f warps (f update) of the same nodes, u handed over in shared memory;
 //   FP32 storage, and FP64 with per-node relaxation times (k_step): one thread
 //     per node;
-//   D2Q9 (k_step_d2q9): one thread per node, with k_macro_d2q9 first when the
-//     C7 correction needs gradients of the macroscopic fields.
+//   D2Q9 (k_step_d2q9): one thread per node on the same integers, with k_macro_d2q9 first
+//     when the C7 correction needs gradients of the macroscopic fields.
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -59,6 +59,7 @@ struct Geo {
   int nx, ny, nz;
   int bcx, bcy, bcz;   // 1 = zero-gradient
   unsigned long long plane;   // nodes
+  unsigned long long inv_nx;  // floor(2^64 / nx) + 1: high half of its product with i < 2^32 is i / nx
 };
 
 __device__ __forceinline__ int src_minus(int i, int n, int zg) {  // source of a pull with c = +1
@@ -539,84 +540,84 @@ __global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ 
   }
 }
 
-// D2Q9 pull of the 9 f and 9 g arriving at node (x, y).
-__device__ __forceinline__ unsigned pull_d2q9(const double* __restrict__ src, const Geo& geo, int x, int y,
-                                              double (&f)[9], double (&g)[9]) {
-  const int xs[3] = {src_minus(x, geo.nx, geo.bcx), x, src_plus(x, geo.nx, geo.bcx)};
-  const unsigned row[3] = {(unsigned)src_minus(y, geo.ny, geo.bcy) * (unsigned)geo.nx, (unsigned)y * (unsigned)geo.nx,
-                           (unsigned)src_plus(y, geo.ny, geo.bcy) * (unsigned)geo.nx};
+// ---- D2Q9: nodes are numbered along the rows one after the other (thread i of the grid
+// takes node i), so rows of any length fill their warps: the paper's 4 x 800 tube, whose
+// rows have 4 nodes, keeps 32 of 32 lanes busy instead of 4.
+struct NodeXY {
+  unsigned node;
+  int x, y;
+};
+__device__ __forceinline__ bool node_xy(const Geo& geo, NodeXY& n) {
+  n.node = blockIdx.x * blockDim.x + threadIdx.x;
+  n.y = (int)(geo.inv_nx ? (unsigned)__umul64hi(n.node, geo.inv_nx) : n.node);   // 0: nx = 1
+  n.x = (int)(n.node - (unsigned)n.y * (unsigned)geo.nx);
+  return n.node < geo.plane;
+}
+// Index offsets to the node's neighbours: a pull with c = +1 / -1 along each axis.
+struct Nbr {
+  int xm, xp, ym, yp;
+};
+__device__ __forceinline__ Nbr neighbours(const Geo& geo, const NodeXY& n) {
+  Nbr b;
+  b.xm = n.x > 0 ? -1 : (geo.bcx ? 0 : geo.nx - 1);
+  b.xp = n.x < geo.nx - 1 ? 1 : (geo.bcx ? 0 : 1 - geo.nx);
+  b.ym = n.y > 0 ? -geo.nx : (geo.bcy ? 0 : (int)geo.plane - geo.nx);
+  b.yp = n.y < geo.ny - 1 ? geo.nx : (geo.bcy ? 0 : geo.nx - (int)geo.plane);
+  return b;
+}
+__device__ __forceinline__ void pull9(const double* __restrict__ base, const Geo& geo, unsigned node, const Nbr& b,
+                                      double (&v)[9]) {
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
-    const unsigned idx = row[1 - d2_cy(a)] + (unsigned)xs[1 - d2_cx(a)];
-    f[a] = __ldg(src + (unsigned long long)a * geo.plane + idx);
-    g[a] = __ldg(src + (9ull + a) * geo.plane + idx);
+    const int cx = d2_cx(a), cy = d2_cy(a);
+    const unsigned i = node + (unsigned)((cx > 0 ? b.xm : cx < 0 ? b.xp : 0) + (cy > 0 ? b.ym : cy < 0 ? b.yp : 0));
+    v[a] = ldg_nc(base + (unsigned long long)a * geo.plane + i);
   }
-  return row[1] + (unsigned)x;
 }
 
-// Fields of the pulled D2Q9 state for the C_7 gradients (Eq. 38): per node
-// c_s^2 sigma - P, gamma, sigma u_x^2, sigma u_x, sigma u_y^2, sigma u_y.
-constexpr int kMacroD2Q9 = 6;
-__global__ void __launch_bounds__(kBlockX) k_macro_d2q9(const double* __restrict__ src, double* __restrict__ q,
-                                                        Geo geo) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= geo.nx) return;
+// The FP64 forms of the two kernels below, for nodes outside the integer grid's exponent
+// range (and a negative number density, which the FP64 step lets pass).
+__device__ __noinline__ void macro_d2q9_general(const double* __restrict__ src, double* __restrict__ q, const Geo& geo,
+                                                const NodeXY& nd) {
+  const Nbr b = neighbours(geo, nd);
   double f[9], g[9], dp[4], Sa, Sd;
-  const unsigned node = pull_d2q9(src, geo, x, blockIdx.y, f, g);
+  pull9(src, geo, nd.node, b, f);
+  pull9(src + 9ull * geo.plane, geo, nd.node, b, g);
   NodeMacro m;
   node_moments_d2q9<double>(f, g, dp, Sa, Sd, m);
   node_recover_fast(m);
-  const double sux = m.sigma * m.ux, suy = m.sigma * m.uy;
-  q[node] = fma(1.0 / 3.0, m.sigma, -m.P);
-  q[geo.plane + node] = 1.0 / sqrt(1.0 - m.u2);
-  q[2 * geo.plane + node] = sux * m.ux;
-  q[3 * geo.plane + node] = sux;
-  q[4 * geo.plane + node] = suy * m.uy;
-  q[5 * geo.plane + node] = suy;
+  const double a = fma(1.0 / 3.0, m.sigma, -m.P), sux = m.sigma * m.ux, suy = m.sigma * m.uy;
+  double* o = q + nd.node;
+  o[0] = fma(-sux, m.ux, a);
+  o[geo.plane] = fma(-suy, m.uy, a);
+  o[2 * geo.plane] = sux;
+  o[3 * geo.plane] = suy;
+  o[4 * geo.plane] = 1.0 / sqrt(1.0 - m.u2);
 }
-
-// One axis of the C_7 term (Eq. 38 for a flow along that axis): neighbours im, ip
-// of the node along the axis, u its velocity component, qa = q + 2 plane (x) or
-// q + 4 plane (y) the sigma u^2 / sigma u fields of that component.
-__device__ __forceinline__ double c7_axis(const double* __restrict__ q, const double* __restrict__ qa,
-                                          unsigned long long P, unsigned im, unsigned ip, double u, double sigma,
-                                          double gam, double theta, double kth) {
-  const double d1 = 0.5 * (q[ip] - q[im]);              // d(c_s^2 sigma - P)
-  const double d2 = 0.5 * (q[P + ip] - q[P + im]);      // d(gamma)
-  const double d3 = 0.5 * (qa[ip] - qa[im]);            // d(sigma u^2)
-  const double d4 = 0.5 * (qa[P + ip] - qa[P + im]);    // d(sigma u)
-  return 2.0 * (u * d1 - (sigma * (1.0 / 3.0)) * (u / gam) * d2 - u * d3) + kth * (u * u * theta * d4);
+// C_7 = E_x - E_y of Eq. 38 from the neighbours' macroscopic fields (below), with the
+// node's u, sigma / (3 gamma) and (k / 2) theta.  The neighbours are the pulls' sources: a
+// zero-gradient end reuses the edge node.
+__device__ __forceinline__ double c7_of(const double* __restrict__ qn, unsigned long long P, const Nbr& b, double ux,
+                                        double uy, double sg, double kth) {
+  const double dgx = qn[4 * P + b.xp] - qn[4 * P + b.xm], dgy = qn[4 * P + b.yp] - qn[4 * P + b.ym];
+  const double ex = fma(kth * ux, qn[2 * P + b.xp] - qn[2 * P + b.xm], fma(-sg, dgx, qn[b.xp] - qn[b.xm]));
+  const double ey = fma(kth * uy, qn[3 * P + b.yp] - qn[3 * P + b.ym], fma(-sg, dgy, qn[P + b.yp] - qn[P + b.ym]));
+  return fma(ux, ex, -uy * ey);
 }
-
-// D2Q9 (FP64): node (x, y) pulls link a from (x - c_x, y - c_y).  With CORR the
-// C_7 term of Eqs. 37-38, C_7 = E_x - E_y, is added to the m_7 = p_xx moment of the
-// result.
-template <bool MRT, bool QSEP, bool CORR, bool ETA = false>
-__global__ void __launch_bounds__(kBlockX) k_step_d2q9(const double* __restrict__ src, double* __restrict__ dst,
-                                                       Geo geo, StepConst k, unsigned long long* __restrict__ bad,
-                                                       const double* __restrict__ q) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= geo.nx) return;
-  const int y = blockIdx.y;
+template <bool MRT, bool QSEP, bool CORR>
+__device__ __noinline__ void step_d2q9_general(const double* __restrict__ src, double* __restrict__ dst, const Geo& geo,
+                                               const StepConst& k, unsigned long long* __restrict__ bad,
+                                               const double* __restrict__ q, const NodeXY& nd) {
+  const Nbr b = neighbours(geo, nd);
   double f[9], g[9];
-  const unsigned node = pull_d2q9(src, geo, x, y, f, g);
+  pull9(src, geo, nd.node, b, f);
+  pull9(src + 9ull * geo.plane, geo, nd.node, b, g);
   NodeMacro m;
-  const bool b = node_collide_d2q9_f64<MRT, QSEP, ETA>(f, g, k, m);
-  if (b) atomicMin(bad, (unsigned long long)node);
+  if (node_collide_d2q9_f64<MRT, QSEP, false>(f, g, k, m)) atomicMin(bad, (unsigned long long)nd.node);
   if (CORR) {
-    // neighbours: a zero-gradient end reuses the edge node, a periodic axis wraps
-    const unsigned nx = (unsigned)geo.nx, rowy = (unsigned)y * nx;
-    const unsigned xm = rowy + (unsigned)(x > 0 ? x - 1 : (geo.bcx ? 0 : geo.nx - 1));
-    const unsigned xp = rowy + (unsigned)(x < geo.nx - 1 ? x + 1 : (geo.bcx ? geo.nx - 1 : 0));
-    const unsigned ym = (unsigned)(y > 0 ? y - 1 : (geo.bcy ? 0 : geo.ny - 1)) * nx + (unsigned)x;
-    const unsigned yp = (unsigned)(y < geo.ny - 1 ? y + 1 : (geo.bcy ? geo.ny - 1 : 0)) * nx + (unsigned)x;
-    const unsigned long long P = geo.plane;
-    const double gam = q[P + node];
-    const double theta = 1.0 + 1.0 / fma(4.0 * gam, gam, -1.0);   // e / P = 3
-    const double c7 = c7_axis(q, q + 2 * P, P, xm, xp, m.ux, m.sigma, gam, theta, k.c7_theta) -
-                      c7_axis(q, q + 4 * P, P, ym, yp, m.uy, m.sigma, gam, theta, k.c7_theta);
-    // m_7 = p_xx (row c_x^2 - c_y^2, norm 4): (1 - s_7/2) C_7 spread over the axis links
-    const double dq = 0.25 * (1.0 - 0.5 * k.omv) * c7;
+    const double sg = m.sigma * (1.0 / 3.0) / q[4 * geo.plane + nd.node];
+    const double dq = (0.25 * (1.0 - 0.5 * k.omv)) *
+                      c7_of(q + nd.node, geo.plane, b, m.ux, m.uy, sg, 0.5 * k.c7_theta * (4.0 / (3.0 + m.u2)));
     g[1] += dq;
     g[2] += dq;
     g[3] -= dq;
@@ -624,8 +625,124 @@ __global__ void __launch_bounds__(kBlockX) k_step_d2q9(const double* __restrict_
   }
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
-    dst[(unsigned long long)a * geo.plane + node] = f[a];
-    dst[(9ull + a) * geo.plane + node] = g[a];
+    dst[(unsigned long long)a * geo.plane + nd.node] = f[a];
+    dst[(9ull + a) * geo.plane + nd.node] = g[a];
+  }
+}
+
+// Fields of the pulled D2Q9 state for the C_7 gradients (Eq. 38): per node
+// c_s^2 sigma - P - sigma u_x^2, the same with u_y, sigma u_x, sigma u_y and gamma.  From
+// the node's integers: c_s^2 sigma - P = T00 - (2/3) sigma and sigma u = M, one FP64
+// rounding each.
+constexpr int kMacroD2Q9 = 5;
+__global__ void __launch_bounds__(kBlockX) k_macro_d2q9(const double* __restrict__ src, double* __restrict__ q,
+                                                        const __grid_constant__ Geo geo) {
+  NodeXY nd;
+  if (!node_xy(geo, nd)) return;
+  double v[9];
+  pull9(src + 9ull * geo.plane, geo, nd.node, neighbours(geo, nd), v);
+  D9State s;
+  d9_load(v, s);
+  if (s.out) {
+    macro_d2q9_general(src, q, geo, nd);
+    return;
+  }
+  UFix u;
+  bool br;
+  const unsigned long long sig = fx_recover(s.T00, s.Mx, s.My, 0, u, br);
+  const unsigned long long xx = fx::mulhi(u.ax, u.ax), yy = fx::mulhi(u.ay, u.ay);   // u_i^2 2^62
+  const long long a = s.T00 - (long long)fx::mulhi(sig, fx::kTwoThirds);
+  const unsigned long long u2 = min(xx + yy, (1ull << 62) - 1);   // a non-physical node is flagged by the step
+  const unsigned long long w = (1ull << 62) - u2;
+  const int sh = fx::even_shift(w), U = s.E - 1079;
+  const unsigned long long Y = fx::rsqrt_fixed(w << sh);          // gamma 2^(62 - sh / 2)
+  double* o = q + nd.node;
+  o[0] = scale_pow2(__ll2double_rn(a - 4 * (long long)fx::mulhi(sig, xx)), U);
+  o[geo.plane] = scale_pow2(__ll2double_rn(a - 4 * (long long)fx::mulhi(sig, yy)), U);
+  o[2 * geo.plane] = scale_pow2(__ll2double_rn(s.Mx), U);
+  o[3 * geo.plane] = scale_pow2(__ll2double_rn(s.My), U);
+  o[4 * geo.plane] = scale_pow2(__ll2double_rn((long long)Y), (sh >> 1) - 62);
+}
+
+// D2Q9 (FP64): node (x, y) pulls link a from (x - c_x, y - c_y).  With CORR the
+// C_7 term of Eqs. 37-38, C_7 = E_x - E_y, is added to the m_7 = p_xx moment of the
+// result: with differences D over the two neighbours along axis a,
+//   E_a = u_a [D(c_s^2 sigma - P - sigma u_a^2) - (sigma / (3 gamma)) D gamma
+//              + (k/2) theta u_a D(sigma u_a)],   theta = 4 / (3 + u^2).
+// f is rounded on the integer pipe and g on the FP64 pipe, 9 FP64-pipe instructions per
+// node (31 with C_7), and f is pulled only when g is stored, which lets 8 blocks per SM
+// hold the launch's latency (64 registers; 5 blocks at 96 registers: 145 us with C_7).
+// 1200 x 900: 295 -> 70 us per step, with C_7 561 -> 126 (of that k_macro_d2q9 138 -> 30).
+template <bool MRT, bool QSEP, bool CORR>
+__global__ void __launch_bounds__(kBlockX, 8) k_step_d2q9(const double* __restrict__ src, double* __restrict__ dst,
+                                                       const __grid_constant__ Geo geo, const __grid_constant__ StepConst k,
+                                                       unsigned long long* __restrict__ bad,
+                                                       const double* __restrict__ q) {
+  NodeXY nd;
+  if (!node_xy(geo, nd)) return;
+  const unsigned node = nd.node;
+  const Nbr b = neighbours(geo, nd);
+  double v[9];
+  pull9(src + 9ull * geo.plane, geo, node, b, v);
+  D9State g;
+  d9_load(v, g);
+  UFix u;
+  bool br;
+  const unsigned long long sig = fx_recover(g.T00, g.Mx, g.My, 0, u, br);
+  const long long Pf = (long long)sig - g.T00;
+  u.xx = fx::mulhi(u.ax, u.ax);
+  u.yy = fx::mulhi(u.ay, u.ay);
+  u.xy = fx::mulhi(u.ax, u.ay);
+  const unsigned long long u2 = u.xx + u.yy;
+  const bool phys = !(br | (Pf <= 0) | (u2 >= (1ull << 62)));
+  const Rates r = constant_rates_d2q9(k);
+  d9_relax<true, MRT, QSEP, false>(g, sig, Pf, u, r, v);
+  if (CORR) {
+    // sigma / (3 gamma) on the grid of g, theta = R 2^-62, u_i 2^-63
+    int h;
+    const unsigned long long Sq = fx::sqrt_one_minus((1ull << 62) - (phys ? u2 : 0ull), h);
+    const double sg = scale_pow2(__ll2double_rn((long long)(fx::mulhi(fx::mulhi(sig, fx::kThird), Sq) << 1 >> h)), g.E - 1079);
+    const double th = scale_pow2(__ll2double_rn((long long)fx::rcp_fixed((3ull << 62) + (phys ? u2 : 0ull))), -62);
+    const double ux = scale_pow2(__ll2double_rn(fx::with_sign(u.ax, u.sx)), -63);
+    const double uy = scale_pow2(__ll2double_rn(fx::with_sign(u.ay, u.sy)), -63);
+    // m_7 = p_xx (row c_x^2 - c_y^2, norm 4): (1 - s_7/2) C_7 spread over the axis links
+    const double dq = (0.25 * (1.0 - 0.5 * k.omv)) * c7_of(q + node, geo.plane, b, ux, uy, sg, 0.5 * k.c7_theta * th);
+    v[1] += dq;
+    v[2] += dq;
+    v[3] -= dq;
+    v[4] -= dq;
+  }
+#pragma unroll
+  for (int a = 0; a < 9; ++a) dst[(9ull + a) * geo.plane + node] = v[a];
+  pull9(src, geo, node, b, v);
+  D9State f;
+  d9_load(v, f);
+  if (g.out | f.out | (f.T00 < 0)) {
+    step_d2q9_general<MRT, QSEP, CORR>(src, dst, geo, k, bad, q, nd);
+    return;
+  }
+  if (!phys) atomicMin(bad, (unsigned long long)node);
+  d9_relax<false, false, false, true>(f, (unsigned long long)f.T00, 0, u, r, v);
+#pragma unroll
+  for (int a = 0; a < 9; ++a) dst[(unsigned long long)a * geo.plane + node] = v[a];
+}
+
+// D2Q9 with relaxation times per node from a fixed eta/s, in FP64 arithmetic.
+template <bool MRT, bool QSEP>
+__global__ void __launch_bounds__(kBlockX) k_step_d2q9_eta(const double* __restrict__ src, double* __restrict__ dst,
+                                                           Geo geo, StepConst k, unsigned long long* __restrict__ bad) {
+  NodeXY nd;
+  if (!node_xy(geo, nd)) return;
+  const Nbr b = neighbours(geo, nd);
+  double f[9], g[9];
+  pull9(src, geo, nd.node, b, f);
+  pull9(src + 9ull * geo.plane, geo, nd.node, b, g);
+  NodeMacro m;
+  if (node_collide_d2q9_f64<MRT, QSEP, true>(f, g, k, m)) atomicMin(bad, (unsigned long long)nd.node);
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    dst[(unsigned long long)a * geo.plane + nd.node] = f[a];
+    dst[(9ull + a) * geo.plane + nd.node] = g[a];
   }
 }
 
@@ -679,6 +796,7 @@ Geo make_geo(const rlb_handle* h) {
   g.bcy = h->cfg.bc[1] == RLB_ZERO_GRADIENT;
   g.bcz = h->cfg.bc[2] == RLB_ZERO_GRADIENT;
   g.plane = h->nodes;
+  g.inv_nx = g.nx > 1 ? ~0ull / (unsigned long long)g.nx + 1 : 0;
   return g;
 }
 
@@ -709,25 +827,26 @@ template <typename S>
 cudaError_t launch_step(rlb_handle* h, const void* src, void* dst, cudaStream_t st) {
   const Geo geo = make_geo(h);
   if (h->Q == 9) {
+    // small planes spread over more SMs with one warp per block
     const int bx = h->nodes <= 152ull * 128ull * 2ull ? 32 : kBlockX;
-    dim3 grid2((geo.nx + bx - 1) / bx, geo.ny, 1);
+    const unsigned gr = (unsigned)((h->nodes + bx - 1) / bx);
     const bool mrt2 = h->cfg.collision == RLB_MRT, q2 = qsep(h->cfg);
     const double* s2 = (const double*)src;
     double* d2 = (double*)dst;
     if (h->cfg.eta_over_s > 0) {
-      if (!mrt2) k_step_d2q9<false, false, false, true><<<grid2, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
-      else if (!q2) k_step_d2q9<true, false, false, true><<<grid2, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
-      else k_step_d2q9<true, true, false, true><<<grid2, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
+      if (!mrt2) k_step_d2q9_eta<false, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad);
+      else if (!q2) k_step_d2q9_eta<true, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad);
+      else k_step_d2q9_eta<true, true><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad);
     } else if (h->cfg.correction != RLB_CORR_NONE) {
-      k_macro_d2q9<<<grid2, bx, 0, st>>>(s2, h->d_macro, geo);
-      if (!q2) k_step_d2q9<true, false, true><<<grid2, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, h->d_macro);
-      else k_step_d2q9<true, true, true><<<grid2, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, h->d_macro);
+      k_macro_d2q9<<<gr, bx, 0, st>>>(s2, h->d_macro, geo);
+      if (!q2) k_step_d2q9<true, false, true><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, h->d_macro);
+      else k_step_d2q9<true, true, true><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, h->d_macro);
     } else if (!mrt2) {
-      k_step_d2q9<false, false, false><<<grid2, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
+      k_step_d2q9<false, false, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
     } else if (!q2) {
-      k_step_d2q9<true, false, false><<<grid2, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
+      k_step_d2q9<true, false, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
     } else {
-      k_step_d2q9<true, true, false><<<grid2, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
+      k_step_d2q9<true, true, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
     }
     return cudaGetLastError();
   }

@@ -41,7 +41,9 @@
 //     mode, whose relaxation times vary per node;
 //   node_collide_f32s: FP32 population storage, exact sums, recovery by one FP64
 //     Newton step on sigma's quadratic from an FP32 seed, FP32 per-link work;
-//   node_collide_d2q9_f64: the D2Q9 model of Sec. V.A.
+//   d9_load / d9_relax: the D2Q9 model of Sec. V.A, on the same integers;
+//     node_collide_d2q9_f64 is its FP64 form (fixed eta/s, and exponents outside the
+//     integers' range).
 #pragma once
 #include <cmath>
 #include <cstdint>
@@ -93,6 +95,8 @@ struct StepConst {
   unsigned long long Om2_f, Om2_v;
   int r_f, r_v;
   long long CE, CP, CQ;
+  // the D2Q9 row constants: ce * 2^67, cp * 2^67, cq * 2^65 (norms 36, 36, 12)
+  long long CE9, CP9, CQ9;
   // coefficient of the theta term of the C_7 correction (Eq. 38): 1 (Eq. A17) or 2 (as printed)
   double c7_theta;
 };
@@ -142,9 +146,15 @@ inline StepConst make_step_const(double tau_f, double tau_v, double tau_e, doubl
   k.r_v = k.omv >= 1.0 ? 2 : 1;
   k.Om2_f = (unsigned long long)std::ldexp(k.r_f == 2 ? k.omf - 1.0 : k.omf, 64) & ~1ull;
   k.Om2_v = (unsigned long long)std::ldexp(k.r_v == 2 ? k.omv - 1.0 : k.omv, 64) & ~1ull;
-  k.CE = std::llround(std::ldexp(k.ce, 73));
-  k.CP = std::llround(std::ldexp(k.cp, 69));
-  k.CQ = std::llround(std::ldexp(k.cq, 67));
+  if (d2) {
+    k.CE9 = std::llround(std::ldexp(k.ce, 67));
+    k.CP9 = std::llround(std::ldexp(k.cp, 67));
+    k.CQ9 = std::llround(std::ldexp(k.cq, 65));
+  } else {
+    k.CE = std::llround(std::ldexp(k.ce, 73));
+    k.CP = std::llround(std::ldexp(k.cp, 69));
+    k.CQ = std::llround(std::ldexp(k.cq, 67));
+  }
   return k;
 }
 
@@ -548,7 +558,6 @@ constexpr unsigned long long kTwoThirds = 0xAAAAAAAAAAAAAAABull;   // ceil(2^65 
 constexpr unsigned long long kEighteenth = 0x0E38E38E38E38E39ull;  // ceil(2^64 / 18)
 constexpr unsigned long long kSignBit = 0x8000000000000000ull;
 // D2Q9 weights
-constexpr unsigned long long kFourNinths = 0x71C71C71C71C71C8ull;  // ceil(2^66 / 9)
 constexpr unsigned long long kNinth = 0x1C71C71C71C71C72ull;       // ceil(2^64 / 9)
 constexpr unsigned long long kTwelfth = 0x1555555555555556ull;     // ceil(2^64 / 12)
 constexpr unsigned long long k36th = 0x071C71C71C71C71Dull;        // ceil(2^64 / 36)
@@ -862,17 +871,16 @@ using fx::UFix;
 
 // D2Q9 class constants of a distribution on its grid (weights 4/9, 1/9, 1/36; Eqs. 7,
 // 32-33), with X_i, Y_ij, Z_i of eq_pieces and SX = D u^2 / 4:
-//   rest r;  axis i: ev = KA + 2 X_i, od = 2 Z_i;  diagonal: ev = KD +- Y, od = (Z_x +- Z_y)/2.
+//   axis i: ev = KA + 2 X_i, od = 2 Z_i;  diagonal: ev = KD +- Y, od = (Z_x +- Z_y)/2;
+//   rest: the density less the moving links, total - 4 (KA + KD + SX).
 struct Eq9 {
-  long long r, KA, KD;
+  long long KA, KD;
 };
 template <bool G>
 __device__ __forceinline__ void eq9_pieces(unsigned long long D, long long Pf, long long SX, Eq9& w) {
   using namespace fx;
   const unsigned long long P = (unsigned long long)Pf;
   const long long s3 = (long long)mulhi((unsigned long long)SX, kThird);
-  const long long s83 = 2 * SX + (long long)mulhi((unsigned long long)SX, kTwoThirds);   // (2/3) D u^2
-  w.r = (G ? (long long)D - 2 * Pf - (long long)mulhi(P, kTwoThirds) : (long long)mulhi(D, kFourNinths)) - s83;
   w.KA = (G ? (long long)mulhi(P, kThird) : (long long)mulhi(D, kNinth)) - 2 * s3;
   w.KD = (G ? (long long)mulhi(P, kTwelfth) : (long long)mulhi(D, k36th)) + s3;
 }
@@ -1683,6 +1691,110 @@ __device__ __forceinline__ void node_equilibrium_d2q9(double e, double ux, doubl
 }
 
 // ---------------------------------------------------------------------------
+// D2Q9 collide in 64-bit block fixed point, as the D3Q19 one: the FP64 form
+// (node_collide_d2q9_f64) issues about 140 FP64-pipe instructions per node, this one the
+// roundings of the outputs only.
+struct D9State {
+  long long X[9];
+  long long Sa, Sd, T00, Mx, My;     // of g
+  int E;
+  bool out;                          // exponent outside the grid's range: the FP64 form is used
+};
+// One distribution on its grid, with its class sums and moments (N0 in T00 for f).
+__device__ __forceinline__ void d9_load(const double (&v)[9], D9State& s) {
+  using namespace fx;
+  bool fast;
+  s.E = max_exponent(v, fast);
+  s.out = !FxUnit<double>::in_range(s.E);
+  if (fast) {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) s.X[a] = to_fixed_pos(v[a], s.E + 7);
+  } else {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) s.X[a] = to_fixed(v[a], s.E + 7);
+  }
+  s.Sa = (s.X[1] + s.X[2]) + (s.X[3] + s.X[4]);
+  s.Sd = (s.X[5] + s.X[6]) + (s.X[7] + s.X[8]);
+  s.T00 = s.X[0] + s.Sa + s.Sd;
+  const long long d2 = s.X[5] - s.X[6], d3 = s.X[7] - s.X[8];
+  s.Mx = (s.X[1] - s.X[2]) + d2 + d3;
+  s.My = (s.X[3] - s.X[4]) + d2 - d3;
+}
+// Rates of one node on integers: omega 2^63 (even) and the MRT row constants.
+struct Rates {
+  unsigned long long Omf, Omv;
+  long long CE, CP, CQ;
+};
+__device__ __forceinline__ Rates constant_rates_d2q9(const StepConst& k) {
+  return Rates{k.Om_f, k.Om_v, k.CE9, k.CP9, k.CQ9};
+}
+// Relaxed populations of one distribution (Eqs. 5-6, 30-35), rounded to FP64: G selects
+// g (density D = sigma, pressure Pf) or f (D = N0).  INT: the rounding runs on the integer
+// pipe instead of the FP64 pipe.
+template <bool G, bool MRT, bool QSEP, bool INT>
+__device__ __forceinline__ void d9_relax(const D9State& s, unsigned long long D, long long Pf, const UFix& u,
+                                         const Rates& r, double (&out)[9]) {
+  using namespace fx;
+  const long long Xx = (long long)mulhi(D, u.xx), Xy = (long long)mulhi(D, u.yy);
+  const long long Y = with_sign(mulhi(D, u.xy), u.sx ^ u.sy);
+  const unsigned long long D3 = mulhi(D, kThird);
+  const long long Zx = with_sign(mulhi(D3, u.ax), u.sx), Zy = with_sign(mulhi(D3, u.ay), u.sy);
+  const long long SX = Xx + Xy;
+  Eq9 w;
+  eq9_pieces<G>(D, Pf, SX, w);
+  // The conserved sums of the equilibrium are those of the populations to the unit (rest
+  // link, and for g the axis links' odd part from M), and 2 units (3 on the diagonals of f)
+  // come off each relaxed link against the truncation of its product and, for g, the
+  // conversion's set low bit.  Without these a run of 40 steps drifted by five times the
+  // FP64 form's error; with them the errors against 64 bits are below that form's
+  // (1200 x 900, 40 steps: e 8.5e-16 -> 6.1e-16, u 3.6e-15 -> 3.0e-15, n 1.5e-15 -> 5.5e-16).
+  const long long rest = s.T00 - 4 * (w.KA + w.KD + SX);
+  const unsigned long long Om = G ? r.Omv : r.Omf;
+  long long c0 = (long long)(Om >> 1) - 2, cA = c0, cD = c0 - (INT ? 1 : 0), dq[4] = {0, 0, 0, 0};
+  if (MRT && G) {
+    // class sums of g - g^eq (axis (4/3) P + sigma u^2 / 3, diagonal P / 3 + sigma u^2 / 3)
+    const long long s3 = 2 * (long long)mulhi((unsigned long long)SX, kTwoThirds);
+    const long long P23 = (long long)mulhi((unsigned long long)Pf, kTwoThirds);
+    const long long n0 = (s.X[0] - rest) >> 3;
+    const long long nA = (s.Sa - 2 * P23 - s3) >> 3;
+    const long long nD = (s.Sd - (P23 >> 1) - s3) >> 3;
+    const long long ae = __mul64hi(2 * nD - 4 * n0 - nA, r.CE);
+    const long long ap = __mul64hi(nD + 4 * n0 - 2 * nA, r.CP);
+    c0 += 4 * (ae - ap);
+    cA += 2 * ap + ae;
+    cD -= 2 * ae + ap;
+    if (QSEP) {   // q_i = (3|c|^2 - 5) c_i, q^eq_i = -M_i
+      const long long d0 = s.X[1] - s.X[2], d1 = s.X[3] - s.X[4];
+      const long long aqx = __mul64hi(2 * s.Mx - 3 * d0, r.CQ) >> 1;
+      const long long aqy = __mul64hi(2 * s.My - 3 * d1, r.CQ) >> 1;
+      dq[0] = 2 * aqx;
+      dq[1] = 2 * aqy;
+      dq[2] = -(aqx + aqy);
+      dq[3] = -(aqx - aqy);
+    }
+  }
+  const long long ev[4] = {w.KA + 2 * Xx, w.KA + 2 * Xy, w.KD + Y, w.KD - Y};
+  const long long op = (Zx + Zy) >> 1, om = (Zx - Zy) >> 1;
+  const long long od[4] = {G ? (s.Mx >> 1) - (op + om) : 2 * Zx, G ? (s.My >> 1) - (op - om) : 2 * Zy, op, om};
+  out[0] = from_fixed<!INT>(relax(s.X[0], rest, Om, c0), s.E);
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const long long c = p < 2 ? cA : cD;
+    long long ca = c, cb = c;
+    if (MRT && QSEP && G) {
+      ca += dq[p];
+      cb -= dq[p];
+      // Both stay separate values: folded into the relaxation's sum, ptxas 13.0 (-O1 and up,
+      // not -O0) loses a carry between the 32-bit halves (link 6 off by 2^32 units on a
+      // third of all nodes).
+      asm("" : "+l"(ca), "+l"(cb));
+    }
+    out[2 * p + 1] = from_fixed<!INT>(relax(s.X[2 * p + 1], ev[p] + od[p], Om, ca), s.E);
+    out[2 * p + 2] = from_fixed<!INT>(relax(s.X[2 * p + 2], ev[p] - od[p], Om, cb), s.E);
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Equilibrium of given FP64 fields on integers (the same sums as node_equilibrium):
 // gamma^2 and gamma from 1 - u^2 by fixed-point Newton steps, sigma = (4/3) e gamma^2 and
 // N0 = n gamma with their top bit at 2^60-2^62, so a unit is at most 2^-60 of them (FP64
@@ -1773,7 +1885,8 @@ __device__ __forceinline__ bool fx_equilibrium_store(const FxEquilibrium& e, S* 
   } else {
     Eq9 w;
     eq9_pieces<G>(D, e.Pf, SX, w);
-    out[0] = fx_round<S, INT>(w.r, U, e.tol, near);
+    const long long total = G ? (long long)D - e.Pf : (long long)D;
+    out[0] = fx_round<S, INT>(total - 4 * (w.KA + w.KD + SX), U, e.tol, near);
     const long long ev[4] = {w.KA + 2 * q.Xx, w.KA + 2 * q.Xy, w.KD + q.Yxy, w.KD - q.Yxy};
     const long long od[4] = {2 * q.Zx, 2 * q.Zy, (q.Zx + q.Zy) >> 1, (q.Zx - q.Zy) >> 1};
 #pragma unroll

@@ -218,3 +218,55 @@ def test_d3q19_mrt_with_eta_over_s():
     prm = O.Params(collision="mrt", tau_f=0.6, tau_e=0.05, tau_eps=0.05, tau_q=0.5, eta_over_s=0.2, bc=oracle_bc(bc))
     ref = oracle_fields(*O.run(*O.init_populations(e, torch.stack([ux, uy, uz]), n), prm, T))
     assert max(field_errors(gpu, ref).values()) < TOL64
+
+
+# ----------------------------------------------------------------------------- integer step, node numbering
+@pytest.mark.parametrize("collision, tau_q, corr", [("mrt", 0.0, False), ("mrt", 0.7, "c7"), ("bgk", 0.0, False)])
+@pytest.mark.parametrize("shape", [(1, 7, 1), (1, 1, 9), (1, 5, 3), (1, 33, 130)])
+def test_d2q9_step_rows_of_any_length_and_any_scale(shape, collision, tau_q, corr):
+    """Nodes are numbered across rows: rows of 1 to 130 nodes against the oracle, 20 steps
+    (1e-12 normwise per field, the FP64 parity bound).  Populations scaled by 2^-600 leave
+    the integer form's exponent range and take the FP64 form: the two agree within 20
+    steps of a few roundings (1e-13 of each distribution's largest population)."""
+    from paper_1211_3286_gb300.lattice import Lattice
+    e, ux, uy, uz, n = I.periodic_box(None, seed=61, shape=shape)
+    z = torch.zeros_like(uz)
+    bc = ("zero_gradient", "periodic", "periodic")
+    kw = dict(collision=collision, tau_f=0.8, tau_v=0.9, tau_e=0.6, tau_eps=0.7, tau_q=tau_q)
+    lat = Lattice(shape, bc=bc, lattice="d2q9", correction=corr, **kw)
+    lat.set_fields(*(t.cuda() for t in (e, ux, uy, z, n)))
+    s0 = lat.state()
+    lat.step(20)
+    a = lat.state()
+    gpu = lat.fields("cpu")
+    prm = O.Params(**kw, bc=oracle_bc(bc), lattice="d2q9", correction=bool(corr))
+    ref = oracle_fields(*O.run(*O.init_populations(e, torch.stack([ux, uy, z]), n, "d2q9"), prm, 20))
+    err = field_errors(gpu, ref)
+    assert max(err.values()) < TOL64, err
+    lat.load_state(s0 * 2.0 ** -600)
+    lat.step(20)
+    lat.check()
+    b = lat.state() * 2.0 ** 600
+    lat.close()
+    for p, q in ((a[:9], b[:9]), (a[9:], b[9:])):
+        assert float((p - q).abs().max()) <= 1e-13 * float(p.abs().max())
+
+
+def test_d2q9_negative_number_density_steps_like_the_oracle():
+    """A negative f is carried along (the velocity comes from g): one step against the oracle."""
+    from paper_1211_3286_gb300.lattice import Lattice
+    shape = (1, 6, 10)
+    e, ux, uy, uz, n = I.periodic_box(None, seed=62, shape=shape)
+    z = torch.zeros_like(uz)
+    f, g = O.init_populations(e, torch.stack([ux, uy, z]), n, "d2q9")
+    f[:, 0, 2, 3:6] *= -1.0
+    lat = Lattice(shape, collision="mrt", tau_f=0.8, tau_v=0.9, tau_e=0.6, tau_eps=0.7, lattice="d2q9")
+    lat.load_state(torch.cat([f, g]).cuda())
+    lat.step(1)
+    lat.check()
+    s = lat.state("cpu")
+    lat.close()
+    prm = O.Params(collision="mrt", tau_f=0.8, tau_v=0.9, tau_e=0.6, tau_eps=0.7, lattice="d2q9")
+    fo, go = O.step(f, g, prm)
+    assert float((s[:9] - fo).abs().max()) <= 1e-14 * float(fo.abs().max())
+    assert float((s[9:] - go).abs().max()) <= 1e-14 * float(go.abs().max())
