@@ -59,7 +59,8 @@ struct Geo {
   int nx, ny, nz;
   int bcx, bcy, bcz;   // 1 = zero-gradient
   unsigned long long plane;   // nodes
-  unsigned long long inv_nx;  // floor(2^64 / nx) + 1: high half of its product with i < 2^32 is i / nx
+  // floor(2^64 / n) + 1 (0 for n = 1): the high half of its product with i < 2^32 is i / n
+  unsigned long long inv_nx, inv_ny;
 };
 
 __device__ __forceinline__ int src_minus(int i, int n, int zg) {  // source of a pull with c = +1
@@ -115,6 +116,37 @@ __device__ __forceinline__ void pull19(const S* __restrict__ base, unsigned long
   }
 }
 
+// The same with the node's index and the index offsets of its pulls (rows numbered one
+// after the other, so a warp's lanes may lie in different rows).
+struct Nbr3 {
+  int xm, xp, ym, yp, zm, zp;   // a pull with c = +1 / -1 along each axis
+};
+__device__ __forceinline__ Nbr3 neighbours3(const Geo& geo, unsigned i) {
+  const unsigned q = geo.inv_nx ? (unsigned)__umul64hi(i, geo.inv_nx) : i;       // y + ny z
+  const unsigned z = geo.inv_ny ? (unsigned)__umul64hi(q, geo.inv_ny) : q;
+  const int x = (int)(i - q * (unsigned)geo.nx), y = (int)(q - z * (unsigned)geo.ny);
+  const int nxy = geo.nx * geo.ny, top = (int)geo.plane - nxy;
+  Nbr3 b;
+  b.xm = x > 0 ? -1 : (geo.bcx ? 0 : geo.nx - 1);
+  b.xp = x < geo.nx - 1 ? 1 : (geo.bcx ? 0 : 1 - geo.nx);
+  b.ym = y > 0 ? -geo.nx : (geo.bcy ? 0 : nxy - geo.nx);
+  b.yp = y < geo.ny - 1 ? geo.nx : (geo.bcy ? 0 : geo.nx - nxy);
+  b.zm = z > 0 ? -nxy : (geo.bcz ? 0 : top);
+  b.zp = (int)z < geo.nz - 1 ? nxy : (geo.bcz ? 0 : -top);
+  return b;
+}
+template <typename S>
+__device__ __forceinline__ void pull19(const S* __restrict__ base, unsigned long long plane, unsigned i, const Nbr3& b,
+                                       S (&v)[19]) {
+#pragma unroll
+  for (int a = 0; a < 19; ++a) {
+    const int cx = link_cx(a), cy = link_cy(a), cz = link_cz(a);
+    const unsigned idx = i + (unsigned)((cx > 0 ? b.xm : cx < 0 ? b.xp : 0) + (cy > 0 ? b.ym : cy < 0 ? b.yp : 0) +
+                                        (cz > 0 ? b.zm : cz < 0 ? b.zp : 0));
+    v[a] = ldg_nc(base + (unsigned long long)a * plane + idx);
+  }
+}
+
 // Resident 128-thread blocks per SM the FP64 step is compiled for (register cap
 // 65536 / (128 x blocks)).
 #ifndef RLB_F64_BLOCKS_PER_SM
@@ -125,30 +157,42 @@ __device__ __forceinline__ void pull19(const S* __restrict__ base, unsigned long
 #define RLB_F32_BLOCKS_PER_SM 6
 #endif
 
-template <typename S, bool MRT, bool QSEP, bool ETA = false>
+// FLAT: thread i of the grid takes node i, whatever the row length; else the grid's y and
+// z are the lattice's and each row has its own blocks, with the row offsets the same for
+// all lanes (flat_rows below says which).
+template <typename S, bool MRT, bool QSEP, bool FLAT, bool ETA = false>
 __global__ void __launch_bounds__(kBlockX, sizeof(S) == 8 ? RLB_F64_BLOCKS_PER_SM : RLB_F32_BLOCKS_PER_SM) k_step(const S* __restrict__ src, S* __restrict__ dst, Geo geo,
                                                   StepConst k, unsigned long long* __restrict__ bad) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= geo.nx) return;
-  const int y = blockIdx.y, z = blockIdx.z;
-  // source coordinates for offsets c = +1, 0, -1 (index 0, 1, 2 = 1 - c)
-  const int xs[3] = {src_minus(x, geo.nx, geo.bcx), x, src_plus(x, geo.nx, geo.bcx)};
-  const int ys[3] = {src_minus(y, geo.ny, geo.bcy), y, src_plus(y, geo.ny, geo.bcy)};
-  const int zs[3] = {src_minus(z, geo.nz, geo.bcz), z, src_plus(z, geo.nz, geo.bcz)};
-  unsigned row[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) row[i][j] = ((unsigned)zs[i] * (unsigned)geo.ny + (unsigned)ys[j]) * (unsigned)geo.nx;
-
   S f[19], g[19];
-  pull19<S>(src, geo.plane, xs, row, f);
-  pull19<S>(src + 19ull * geo.plane, geo.plane, xs, row, g);
+  unsigned node;
+  if constexpr (FLAT) {
+    node = blockIdx.x * blockDim.x + threadIdx.x;
+    if (node >= geo.plane) return;
+    const Nbr3 nb = neighbours3(geo, node);
+    pull19<S>(src, geo.plane, node, nb, f);
+    pull19<S>(src + 19ull * geo.plane, geo.plane, node, nb, g);
+  } else {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= geo.nx) return;
+    const int y = blockIdx.y, z = blockIdx.z;
+    // source coordinates for offsets c = +1, 0, -1 (index 0, 1, 2 = 1 - c)
+    const int xs[3] = {src_minus(x, geo.nx, geo.bcx), x, src_plus(x, geo.nx, geo.bcx)};
+    const int ys[3] = {src_minus(y, geo.ny, geo.bcy), y, src_plus(y, geo.ny, geo.bcy)};
+    const int zs[3] = {src_minus(z, geo.nz, geo.bcz), z, src_plus(z, geo.nz, geo.bcz)};
+    unsigned row[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        row[i][j] = ((unsigned)zs[i] * (unsigned)geo.ny + (unsigned)ys[j]) * (unsigned)geo.nx;
+    pull19<S>(src, geo.plane, xs, row, f);
+    pull19<S>(src + 19ull * geo.plane, geo.plane, xs, row, g);
+    node = row[1][1] + (unsigned)x;
+  }
   bool b;
   if constexpr (sizeof(S) == 8 && ETA) b = node_collide_f64<MRT, QSEP, true>(f, g, k);
   else if constexpr (sizeof(S) == 8) b = node_collide_fx<MRT, QSEP>(f, g, k);
   else b = node_collide_f32s<MRT, QSEP>(f, g, k);
-  const unsigned node = row[1][1] + (unsigned)x;
   if (b) atomicMin(bad, (unsigned long long)node);
 #pragma unroll
   for (int a = 0; a < 19; ++a) {
@@ -186,7 +230,7 @@ __global__ void __launch_bounds__(kBlockX, sizeof(S) == 8 ? RLB_F64_BLOCKS_PER_S
 #define RLB_WS_WARPS 4
 #endif
 
-template <int W, bool MRT, bool QSEP, int RV, int RF>
+template <int W, bool MRT, bool QSEP, bool FLAT, int RV, int RF>
 __global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2 * W))
     k_step_ws(const double* __restrict__ src, double* __restrict__ dst, Geo geo, StepConst k,
               unsigned long long* __restrict__ bad) {
@@ -195,21 +239,32 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2
   const int warp = threadIdx.x >> 5;
   const bool is_g = warp < W;
   const int slot = (is_g ? warp : warp - W) * 32 + (threadIdx.x & 31);
-  const int x0 = blockIdx.x * (32 * W) + slot;
-  const bool valid = x0 < geo.nx;
-  const int x = valid ? x0 : geo.nx - 1;
-  const int y = blockIdx.y, z = blockIdx.z;
-  const int xs[3] = {src_minus(x, geo.nx, geo.bcx), x, src_plus(x, geo.nx, geo.bcx)};
-  const int ys[3] = {src_minus(y, geo.ny, geo.bcy), y, src_plus(y, geo.ny, geo.bcy)};
-  const int zs[3] = {src_minus(z, geo.nz, geo.bcz), z, src_plus(z, geo.nz, geo.bcz)};
-  unsigned row[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) row[i][j] = ((unsigned)zs[i] * (unsigned)geo.ny + (unsigned)ys[j]) * (unsigned)geo.nx;
   const unsigned long long plane0 = is_g ? 19ull * geo.plane : 0ull;
   double v[19];
-  pull19<double>(src + plane0, geo.plane, xs, row, v);
+  unsigned node;
+  bool valid;
+  if constexpr (FLAT) {
+    const unsigned i = blockIdx.x * (32 * W) + slot;
+    valid = i < geo.plane;
+    node = valid ? i : (unsigned)geo.plane - 1;
+    pull19<double>(src + plane0, geo.plane, node, neighbours3(geo, node), v);
+  } else {
+    const int x0 = blockIdx.x * (32 * W) + slot;
+    valid = x0 < geo.nx;
+    const int x = valid ? x0 : geo.nx - 1;
+    const int y = blockIdx.y, z = blockIdx.z;
+    const int xs[3] = {src_minus(x, geo.nx, geo.bcx), x, src_plus(x, geo.nx, geo.bcx)};
+    const int ys[3] = {src_minus(y, geo.ny, geo.bcy), y, src_plus(y, geo.ny, geo.bcy)};
+    const int zs[3] = {src_minus(z, geo.nz, geo.bcz), z, src_plus(z, geo.nz, geo.bcz)};
+    unsigned row[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        row[i][j] = ((unsigned)zs[i] * (unsigned)geo.ny + (unsigned)ys[j]) * (unsigned)geo.nx;
+    pull19<double>(src + plane0, geo.plane, xs, row, v);
+    node = row[1][1] + (unsigned)x;
+  }
 
   using namespace fx;
   // both roles: block exponent and fixed-point values.  When every value of every
@@ -300,7 +355,7 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2
   // shift-free relaxation (fx::relax_r): RV / RF = 2 for omega >= 1, 1 below
   const unsigned long long Om = is_g ? k.Om2_v : k.Om2_f;
   long long c0 = (long long)(Om >> 1), cA = c0, cD = c0;
-  long long dq[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  long long aq[3] = {0, 0, 0};
   if (MRT && is_g) {
     // e and eps projections of g - g^eq from the class sums, at 1/8 scale
     const long long n0 = (X[0] - eq0) >> 3;
@@ -316,14 +371,11 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2
       const long long vx = ((Mx - 5 * dp0) >> 2) + (mulhi_su(Mx, kTwoThirds, h23) >> 2);
       const long long vy = ((My - 5 * dp1) >> 2) + (mulhi_su(My, kTwoThirds, h23) >> 2);
       const long long vz = ((Mz - 5 * dp2) >> 2) + (mulhi_su(Mz, kTwoThirds, h23) >> 2);
-      const long long aqx = __mul64hi(vx, k.CQ) >> 1, aqy = __mul64hi(vy, k.CQ) >> 1, aqz = __mul64hi(vz, k.CQ) >> 1;
-      dq[0] = 4 * aqx; dq[1] = 4 * aqy; dq[2] = 4 * aqz;
-      dq[3] = -(aqx + aqy); dq[4] = -(aqx - aqy);
-      dq[5] = -(aqx + aqz); dq[6] = -(aqx - aqz);
-      dq[7] = -(aqy + aqz); dq[8] = -(aqy - aqz);
+      aq[0] = __mul64hi(vx, k.CQ) >> 1;
+      aq[1] = __mul64hi(vy, k.CQ) >> 1;
+      aq[2] = __mul64hi(vz, k.CQ) >> 1;
     }
   }
-  const unsigned node = row[1][1] + (unsigned)x;
   if (valid && b) atomicMin(bad, (unsigned long long)node);
   // Lanes past the row repeat node nx - 1 and compute its values bit for bit, so every
   // lane stores: those lanes write the same bytes to node nx - 1 again, and no branch
@@ -331,10 +383,10 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2
   double* out = dst + plane0 + node;
   if (is_g) {
     out[0] = from_fixed<(RLB_WS_OUT_G >> 9) & 1>(relax_r<RV>(X[0], eq0, Om, c0), E);
-    relax_links_store<RLB_WS_OUT_G, MRT && QSEP, RV>(X, q, Om, cA, cD, dq, E, out, geo.plane, true);
+    relax_links_store<RLB_WS_OUT_G, MRT && QSEP, RV>(X, q, Om, cA, cD, aq, E, out, geo.plane, true);
   } else {
     out[0] = from_fixed<(RLB_WS_OUT_F >> 9) & 1>(relax_r<RF>(X[0], eq0, Om, c0), E);
-    relax_links_store<RLB_WS_OUT_F, false, RF>(X, q, Om, cA, cD, dq, E, out, geo.plane, true);
+    relax_links_store<RLB_WS_OUT_F, false, RF>(X, q, Om, cA, cD, aq, E, out, geo.plane, true);
   }
 }
 
@@ -797,6 +849,7 @@ Geo make_geo(const rlb_handle* h) {
   g.bcz = h->cfg.bc[2] == RLB_ZERO_GRADIENT;
   g.plane = h->nodes;
   g.inv_nx = g.nx > 1 ? ~0ull / (unsigned long long)g.nx + 1 : 0;
+  g.inv_ny = g.ny > 1 ? ~0ull / (unsigned long long)g.ny + 1 : 0;
   return g;
 }
 
@@ -806,14 +859,39 @@ bool qsep(const rlb_config& c) {
 }
 
 // The FP64 steps for the relaxation forms of omega_v and omega_f (1: omega < 1, 2: omega >= 1).
-template <int W, bool MRT, bool QSEP>
+template <int W, bool MRT, bool QSEP, bool FLAT>
 void launch_ws(int rv, int rf, dim3 grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
                const StepConst& k, unsigned long long* bad) {
-  if (rv == 2 && rf == 2) k_step_ws<W, MRT, QSEP, 2, 2><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
-  else if (rv == 2) k_step_ws<W, MRT, QSEP, 2, 1><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
-  else if (rf == 2) k_step_ws<W, MRT, QSEP, 1, 2><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
-  else k_step_ws<W, MRT, QSEP, 1, 1><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
+  if (rv == 2 && rf == 2) k_step_ws<W, MRT, QSEP, FLAT, 2, 2><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
+  else if (rv == 2) k_step_ws<W, MRT, QSEP, FLAT, 2, 1><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
+  else if (rf == 2) k_step_ws<W, MRT, QSEP, FLAT, 1, 2><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
+  else k_step_ws<W, MRT, QSEP, FLAT, 1, 1><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
 }
+template <int W, bool FLAT>
+void launch_ws_coll(bool mrt, bool q, int rv, int rf, dim3 grid, cudaStream_t st, const double* s, double* d,
+                    const Geo& geo, const StepConst& k, unsigned long long* bad) {
+  if (!mrt) launch_ws<W, false, false, FLAT>(rv, rf, grid, st, s, d, geo, k, bad);
+  else if (!q) launch_ws<W, true, false, FLAT>(rv, rf, grid, st, s, d, geo, k, bad);
+  else launch_ws<W, true, true, FLAT>(rv, rf, grid, st, s, d, geo, k, bad);
+}
+template <typename S, bool FLAT, bool ETA>
+void launch_one(bool mrt, bool q, dim3 grid, int bx, cudaStream_t st, const S* s, S* d, const Geo& geo,
+                const StepConst& k, unsigned long long* bad) {
+  if (!mrt) k_step<S, false, false, FLAT, ETA><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
+  else if (!q) k_step<S, true, false, FLAT, ETA><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
+  else k_step<S, true, true, FLAT, ETA><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
+}
+
+// Whether nodes are numbered across rows: where blocks of b nodes per row would leave more
+// than 1 lane in 32 idle.  Numbering them costs 2 % on a row that fills its blocks (256^3
+// FP64 1.798 against 1.834 ms per step, FP32 0.828 against 0.844) and saves the idle lanes:
+// 150 x 110 x 90 FP64 262 -> 175 us (with its own tau_q 313 -> 203), 120 x 128 x 128 233 ->
+// 223, 40 x 120 x 200 309 -> 114; FP32 90 -> 78, 107 -> 103, 82 -> 54.
+bool flat_rows(int nx, int b) {
+  const long long lanes = (long long)((nx + b - 1) / b) * b;
+  return (lanes - nx) * 32 > lanes;
+}
+
 template <bool MRT>
 void launch_quad(int rv, int rf, dim3 grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
                  const StepConst& k, unsigned long long* bad) {
@@ -854,45 +932,36 @@ cudaError_t launch_step(rlb_handle* h, const void* src, void* dst, cudaStream_t 
   // the FP64 pipe of an SM serves 2 lanes per clock, so fewer warps per SM means
   // shorter steps when the lattice cannot fill the GPU anyway
   const int bx = h->nodes <= 152ull * 128ull * 2ull ? 32 : kBlockX;
-  dim3 grid((geo.nx + bx - 1) / bx, geo.ny, geo.nz);
+  const bool flat = flat_rows(geo.nx, bx);
+  const dim3 grid = flat ? dim3((unsigned)((h->nodes + bx - 1) / bx))
+                         : dim3((unsigned)((geo.nx + bx - 1) / bx), geo.ny, geo.nz);
   const bool mrt = h->cfg.collision == RLB_MRT, q = qsep(h->cfg);
   const S* s = (const S*)src;
   S* d = (S*)dst;
   if constexpr (sizeof(S) == 8) {
-    if (h->cfg.eta_over_s > 0) {
-      if (!mrt) k_step<S, false, false, true><<<grid, bx, 0, st>>>(s, d, geo, h->k, h->d_bad);
-      else if (!q) k_step<S, true, false, true><<<grid, bx, 0, st>>>(s, d, geo, h->k, h->d_bad);
-      else k_step<S, true, true, true><<<grid, bx, 0, st>>>(s, d, geo, h->k, h->d_bad);
-      return cudaGetLastError();
-    }
-  }
-  if constexpr (sizeof(S) == 8) {
-    // warp roles: 64-thread blocks (one g and one f warp) for small lattices
-    const double* s8 = (const double*)src;
-    double* d8 = (double*)dst;
     const int rv = h->k.r_v, rf = h->k.r_f;
-    if (bx == 32 && !q) {
-      // four lanes per node: 8 nodes per 64-thread block
+    if (h->cfg.eta_over_s > 0) {
+      if (flat) launch_one<S, true, true>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
+      else launch_one<S, false, true>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
+    } else if (bx == 32 && !q) {
+      // small lattices, four lanes per node: 8 nodes per 64-thread block
       dim3 gq((geo.nx + 7) / 8, geo.ny, geo.nz);
-      if (mrt) launch_quad<true>(rv, rf, gq, st, s8, d8, geo, h->k, h->d_bad);
-      else launch_quad<false>(rv, rf, gq, st, s8, d8, geo, h->k, h->d_bad);
+      if (mrt) launch_quad<true>(rv, rf, gq, st, s, d, geo, h->k, h->d_bad);
+      else launch_quad<false>(rv, rf, gq, st, s, d, geo, h->k, h->d_bad);
     } else if (bx == 32) {
-      dim3 gw((geo.nx + 31) / 32, geo.ny, geo.nz);
-      launch_ws<1, true, true>(rv, rf, gw, st, s8, d8, geo, h->k, h->d_bad);
+      // warp roles, one g and one f warp per block (a block serves bx nodes)
+      if (flat) launch_ws<1, true, true, true>(rv, rf, grid, st, s, d, geo, h->k, h->d_bad);
+      else launch_ws<1, true, true, false>(rv, rf, grid, st, s, d, geo, h->k, h->d_bad);
     } else {
-      constexpr int W = RLB_WS_WARPS;
-      dim3 gw((geo.nx + 32 * W - 1) / (32 * W), geo.ny, geo.nz);
-      if (!mrt) launch_ws<W, false, false>(rv, rf, gw, st, s8, d8, geo, h->k, h->d_bad);
-      else if (!q) launch_ws<W, true, false>(rv, rf, gw, st, s8, d8, geo, h->k, h->d_bad);
-      else launch_ws<W, true, true>(rv, rf, gw, st, s8, d8, geo, h->k, h->d_bad);
+      static_assert(32 * RLB_WS_WARPS == kBlockX, "a block serves kBlockX nodes");
+      if (flat) launch_ws_coll<RLB_WS_WARPS, true>(mrt, q, rv, rf, grid, st, s, d, geo, h->k, h->d_bad);
+      else launch_ws_coll<RLB_WS_WARPS, false>(mrt, q, rv, rf, grid, st, s, d, geo, h->k, h->d_bad);
     }
-    return cudaGetLastError();
   } else {
-    if (!mrt) k_step<S, false, false><<<grid, bx, 0, st>>>(s, d, geo, h->k, h->d_bad);
-    else if (!q) k_step<S, true, false><<<grid, bx, 0, st>>>(s, d, geo, h->k, h->d_bad);
-    else k_step<S, true, true><<<grid, bx, 0, st>>>(s, d, geo, h->k, h->d_bad);
-    return cudaGetLastError();
+    if (flat) launch_one<S, true, false>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
+    else launch_one<S, false, false>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
   }
+  return cudaGetLastError();
 }
 
 int check_flag(rlb_handle* h) {

@@ -514,3 +514,26 @@ def test_small_lattice_step_bitwise_equals_wide_step(shape, reps, collision, bc,
         assert torch.equal(b, a.unsqueeze(1).expand_as(b)), steps
     small.close()
     big.close()
+
+
+# ----------------------------------------------------------------------------- node numbering of the large-lattice steps
+@pytest.mark.parametrize("precision, kw", [
+    ("fp64", dict(collision="mrt")), ("fp64", dict(collision="mrt", tau_q=0.7)), ("fp64", dict(collision="bgk")),
+    ("fp32", dict(collision="mrt")),
+])
+@pytest.mark.parametrize("shape", [(301, 130, 1), (139, 140, 2), (11, 125, 33), (70, 5, 128), (9, 37, 130)])
+def test_rows_of_any_length_vs_oracle(precision, kw, shape):
+    """Above the small-lattice threshold nodes are numbered across rows unless the rows fill
+    128-node blocks: rows of 1, 2, 33, 128 (filled) and 130 nodes, mixed boundaries, 3
+    steps against the oracle (FP64 1e-12; FP32 storage its rounding bound)."""
+    bc = ("zero_gradient", "periodic", "zero_gradient")
+    e, ux, uy, uz, n = I.periodic_box(None, seed=71, shape=shape)
+    lat = _lattice(shape, tau_f=0.7, tau_v=0.9, tau_e=0.55, tau_eps=0.8, bc=bc, precision=precision, **kw)
+    lat.set_fields(*(t.cuda() for t in (e, ux, uy, uz, n)))
+    lat.step(3)
+    gpu = lat.fields("cpu")
+    lat.close()
+    prm = O.Params(tau_f=0.7, tau_v=0.9, tau_e=0.55, tau_eps=0.8, bc=oracle_bc(bc), **kw)
+    ref = oracle_fields(*O.run(*O.init_populations(e, torch.stack([ux, uy, uz]), n), prm, 3))
+    err = field_errors(gpu, ref)
+    assert max(err.values()) < (TOL64 if precision == "fp64" else 50 * 2.0 ** -24 * 3 ** 0.5), err
