@@ -10,8 +10,7 @@
 // and written to the node's own slots.
 //   FP64 (k_step_ws): two threads per node -- g warps (sums, recovery, g update)
 //     and f warps (f update) of the same nodes, u handed over in shared memory;
-//   FP32 storage, and FP64 with per-node relaxation times (k_step): one thread
-//     per node;
+//   FP32 storage (k_step): one thread per node;
 //   D2Q9 (k_step_d2q9): one thread per node on the same integers, with k_macro_d2q9 first
 //     when the C7 correction needs gradients of the macroscopic fields.
 #include <cuda_runtime.h>
@@ -147,12 +146,8 @@ __device__ __forceinline__ void pull19(const S* __restrict__ base, unsigned long
   }
 }
 
-// Resident 128-thread blocks per SM the FP64 step is compiled for (register cap
-// 65536 / (128 x blocks)).
-#ifndef RLB_F64_BLOCKS_PER_SM
-#define RLB_F64_BLOCKS_PER_SM 3
-#endif
-// and the FP32-storage step (6: 80 registers, none spilled)
+// Resident 128-thread blocks per SM the FP32-storage step is compiled for (6: 80
+// registers, none spilled)
 #ifndef RLB_F32_BLOCKS_PER_SM
 #define RLB_F32_BLOCKS_PER_SM 6
 #endif
@@ -160,9 +155,10 @@ __device__ __forceinline__ void pull19(const S* __restrict__ base, unsigned long
 // FLAT: thread i of the grid takes node i, whatever the row length; else the grid's y and
 // z are the lattice's and each row has its own blocks, with the row offsets the same for
 // all lanes (flat_rows below says which).
-template <typename S, bool MRT, bool QSEP, bool FLAT, bool ETA = false>
-__global__ void __launch_bounds__(kBlockX, sizeof(S) == 8 ? RLB_F64_BLOCKS_PER_SM : RLB_F32_BLOCKS_PER_SM) k_step(const S* __restrict__ src, S* __restrict__ dst, Geo geo,
-                                                  StepConst k, unsigned long long* __restrict__ bad) {
+template <typename S, bool MRT, bool QSEP, bool FLAT>
+__global__ void __launch_bounds__(kBlockX, RLB_F32_BLOCKS_PER_SM) k_step(const S* __restrict__ src,
+                                                                         S* __restrict__ dst, Geo geo, StepConst k,
+                                                                         unsigned long long* __restrict__ bad) {
   S f[19], g[19];
   unsigned node;
   if constexpr (FLAT) {
@@ -189,10 +185,7 @@ __global__ void __launch_bounds__(kBlockX, sizeof(S) == 8 ? RLB_F64_BLOCKS_PER_S
     pull19<S>(src + 19ull * geo.plane, geo.plane, xs, row, g);
     node = row[1][1] + (unsigned)x;
   }
-  bool b;
-  if constexpr (sizeof(S) == 8 && ETA) b = node_collide_f64<MRT, QSEP, true>(f, g, k);
-  else if constexpr (sizeof(S) == 8) b = node_collide_fx<MRT, QSEP>(f, g, k);
-  else b = node_collide_f32s<MRT, QSEP>(f, g, k);
+  const bool b = node_collide_f32s<MRT, QSEP>(f, g, k);
   if (b) atomicMin(bad, (unsigned long long)node);
 #pragma unroll
   for (int a = 0; a < 19; ++a) {
@@ -230,12 +223,36 @@ __global__ void __launch_bounds__(kBlockX, sizeof(S) == 8 ? RLB_F64_BLOCKS_PER_S
 #define RLB_WS_WARPS 4
 #endif
 
-template <int W, bool MRT, bool QSEP, bool FLAT, int RV, int RF>
-__global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2 * W))
-    k_step_ws(const double* __restrict__ src, double* __restrict__ dst, Geo geo, StepConst k,
+// ETA (RV = RF = 0): relaxation rates per node from a fixed eta/s.  The f warps hand N0 to
+// the g warps, which form the rates (eta_rates) and hand omega_f back across a second
+// barrier; a node outside that form's range is left to its g lane, which runs the FP64 form
+// for both distributions.  128 x 96 x 80 MRT with its own tau_q: 598 -> 182 us per step (FP64
+// arithmetic held the FP64 pipe 88 % busy with 329 instructions per node, now 46; the limit
+// is the integer instruction stream, issue 58 %).
+template <bool MRT, bool QSEP>
+__device__ __noinline__ void step_eta_general(const double* __restrict__ src, double* __restrict__ dst, const Geo& geo,
+                                              const StepConst& k, unsigned long long* __restrict__ bad, unsigned node) {
+  double f[19], g[19];
+  const Nbr3 nb = neighbours3(geo, node);
+  pull19<double>(src, geo.plane, node, nb, f);
+  pull19<double>(src + 19ull * geo.plane, geo.plane, node, nb, g);
+  if (node_collide_f64<MRT, QSEP, true>(f, g, k)) atomicMin(bad, (unsigned long long)node);
+#pragma unroll
+  for (int a = 0; a < 19; ++a) {
+    dst[(unsigned long long)a * geo.plane + node] = f[a];
+    dst[(19ull + a) * geo.plane + node] = g[a];
+  }
+}
+
+template <int W, bool MRT, bool QSEP, bool FLAT, int RV, int RF, bool ETA = false>
+__global__ void __launch_bounds__(64 * W, W == 1 ? (ETA ? 8 : 14) : RLB_WS_WARPS_PER_SM / (2 * W))
+    k_step_ws(const double* __restrict__ src, double* __restrict__ dst, const __grid_constant__ Geo geo,
+              const __grid_constant__ StepConst k,
               unsigned long long* __restrict__ bad) {
   __shared__ unsigned long long s_ax[32 * W], s_ay[32 * W], s_az[32 * W];
   __shared__ unsigned s_sg[32 * W];
+  __shared__ unsigned long long s_n[ETA ? 32 * W : 1];
+  __shared__ int s_e[ETA ? 32 * W : 1];
   const int warp = threadIdx.x >> 5;
   const bool is_g = warp < W;
   const int slot = (is_g ? warp : warp - W) * 32 + (threadIdx.x & 31);
@@ -325,6 +342,10 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2
     N0 = X[0];
 #pragma unroll
     for (int a = 1; a < 19; ++a) N0 += X[a];
+    if (ETA) {
+      s_n[slot] = (unsigned long long)N0;
+      s_e[slot] = E;
+    }
   }
   // g warp i hands u to f warp i only: one named barrier per warp pair (ids 1..W, 64
   // threads each), so a slow g warp holds back its own f warp, not the whole block
@@ -352,17 +373,55 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2
     q.KA = (long long)mulhi((unsigned long long)N0, kEighteenth) - (long long)mulhi((unsigned long long)SX, kThird);
     eq0 = (long long)mulhi((unsigned long long)N0, kThird) - 2 * SX;   // N0/3 - N0 u^2 / 2
   }
+  long long hM[3] = {0, 0, 0};
+  if (ETA) {
+    // sums of the equilibrium equal to the populations' (relax_links_store, EXACT): the FP64
+    // arithmetic of this mode's general form does not drift as truncated integers do
+    const long long h = ((q.Xx + q.Xy) >> 1) + ((q.Xx + q.Xz) >> 1) + ((q.Xy + q.Xz) >> 1);
+    eq0 = (is_g ? T00 : N0) - (6 * q.KA + 2 * SX + 12 * (q.KA >> 1) + 4 * h);
+    if (is_g) {
+      hM[0] = Mx >> 1;
+      hM[1] = My >> 1;
+      hM[2] = Mz >> 1;
+    } else {   // N0 u / 2
+      hM[0] = with_sign(mulhi((unsigned long long)N0, u.ax), u.sx);
+      hM[1] = with_sign(mulhi((unsigned long long)N0, u.ay), u.sy);
+      hM[2] = with_sign(mulhi((unsigned long long)N0, u.az), u.sz);
+    }
+  }
   // shift-free relaxation (fx::relax_r): RV / RF = 2 for omega >= 1, 1 below
-  const unsigned long long Om = is_g ? k.Om2_v : k.Om2_f;
-  long long c0 = (long long)(Om >> 1), cA = c0, cD = c0;
+  unsigned long long Om = is_g ? k.Om2_v : k.Om2_f;
+  long long CE = k.CE, CP = k.CP, CQ = k.CQ;
+  if constexpr (ETA) {
+    bool gen = false;
+    if (is_g) {
+      Rates r;
+      gen = !eta_rates<MRT, QSEP>((long long)s_n[slot], s_e[slot], sig, Pf, E, k, r) || b;
+      s_n[slot] = gen ? 0ull : r.Omf;   // this lane alone reads N0
+      Om = r.Omv;
+      CE = r.CE;
+      CP = r.CP;
+      CQ = r.CQ;
+    }
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + (is_g ? warp : warp - W)) : "memory");
+    if (!is_g) {
+      Om = s_n[slot];
+      gen = Om == 0;
+    }
+    if (gen) {
+      if (is_g && valid) step_eta_general<MRT, QSEP>(src, dst, geo, k, bad, node);
+      return;
+    }
+  }
+  long long c0 = (long long)(Om >> 1) - (ETA ? 1 : 0), cA = c0, cD = c0;   // 1: truncation of the product
   long long aq[3] = {0, 0, 0};
   if (MRT && is_g) {
     // e and eps projections of g - g^eq from the class sums, at 1/8 scale
     const long long n0 = (X[0] - eq0) >> 3;
     const long long nA = (Sa - Pf) >> 3;
     const long long nD = (Sd - Pf - 2 * SX) >> 3;
-    const long long ae = __mul64hi(8 * nD - 11 * nA - 30 * n0, k.CE) >> 6;
-    const long long ap = __mul64hi(nD - 4 * nA + 12 * n0, k.CP) >> 2;
+    const long long ae = __mul64hi(8 * nD - 11 * nA - 30 * n0, CE) >> 6;
+    const long long ap = __mul64hi(nD - 4 * nA + 12 * n0, CP) >> 2;
     c0 += 30 * ae - 12 * ap;
     cA += 11 * ae + 4 * ap;
     cD -= 8 * ae + ap;
@@ -371,9 +430,9 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2
       const long long vx = ((Mx - 5 * dp0) >> 2) + (mulhi_su(Mx, kTwoThirds, h23) >> 2);
       const long long vy = ((My - 5 * dp1) >> 2) + (mulhi_su(My, kTwoThirds, h23) >> 2);
       const long long vz = ((Mz - 5 * dp2) >> 2) + (mulhi_su(Mz, kTwoThirds, h23) >> 2);
-      aq[0] = __mul64hi(vx, k.CQ) >> 1;
-      aq[1] = __mul64hi(vy, k.CQ) >> 1;
-      aq[2] = __mul64hi(vz, k.CQ) >> 1;
+      aq[0] = __mul64hi(vx, CQ) >> 1;
+      aq[1] = __mul64hi(vy, CQ) >> 1;
+      aq[2] = __mul64hi(vz, CQ) >> 1;
     }
   }
   if (valid && b) atomicMin(bad, (unsigned long long)node);
@@ -381,7 +440,9 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? 14 : RLB_WS_WARPS_PER_SM / (2
   // lane stores: those lanes write the same bytes to node nx - 1 again, and no branch
   // guards the 19 stores (1.8164 -> 1.7977 ms per 256^3 step).
   double* out = dst + plane0 + node;
-  if (is_g) {
+  if (ETA) {   // RV = 0 for both roles
+    relax_links_store<0, MRT && QSEP, 0, true>(X, q, Om, cA, cD, aq, E, out, geo.plane, true, hM, is_g ? T00 : N0);
+  } else if (is_g) {
     out[0] = from_fixed<(RLB_WS_OUT_G >> 9) & 1>(relax_r<RV>(X[0], eq0, Om, c0), E);
     relax_links_store<RLB_WS_OUT_G, MRT && QSEP, RV>(X, q, Om, cA, cD, aq, E, out, geo.plane, true);
   } else {
@@ -724,7 +785,7 @@ __global__ void __launch_bounds__(kBlockX) k_macro_d2q9(const double* __restrict
 // f is rounded on the integer pipe and g on the FP64 pipe, 9 FP64-pipe instructions per
 // node (31 with C_7), and f is pulled only when g is stored, which lets 8 blocks per SM
 // hold the launch's latency (64 registers; 5 blocks at 96 registers: 145 us with C_7).
-// 1200 x 900: 295 -> 70 us per step, with C_7 561 -> 126 (of that k_macro_d2q9 138 -> 30).
+// 1200 x 900: 295 -> 70 us per step, with C_7 561 -> 128 (of that k_macro_d2q9 138 -> 30).
 template <bool MRT, bool QSEP, bool CORR>
 __global__ void __launch_bounds__(kBlockX, 8) k_step_d2q9(const double* __restrict__ src, double* __restrict__ dst,
                                                        const __grid_constant__ Geo geo, const __grid_constant__ StepConst k,
@@ -874,18 +935,25 @@ void launch_ws_coll(bool mrt, bool q, int rv, int rf, dim3 grid, cudaStream_t st
   else if (!q) launch_ws<W, true, false, FLAT>(rv, rf, grid, st, s, d, geo, k, bad);
   else launch_ws<W, true, true, FLAT>(rv, rf, grid, st, s, d, geo, k, bad);
 }
-template <typename S, bool FLAT, bool ETA>
-void launch_one(bool mrt, bool q, dim3 grid, int bx, cudaStream_t st, const S* s, S* d, const Geo& geo,
+template <int W, bool FLAT>
+void launch_eta(bool mrt, bool q, dim3 grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
                 const StepConst& k, unsigned long long* bad) {
-  if (!mrt) k_step<S, false, false, FLAT, ETA><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
-  else if (!q) k_step<S, true, false, FLAT, ETA><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
-  else k_step<S, true, true, FLAT, ETA><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
+  if (!mrt) k_step_ws<W, false, false, FLAT, 0, 0, true><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
+  else if (!q) k_step_ws<W, true, false, FLAT, 0, 0, true><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
+  else k_step_ws<W, true, true, FLAT, 0, 0, true><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
+}
+template <bool FLAT>
+void launch_f32(bool mrt, bool q, dim3 grid, int bx, cudaStream_t st, const float* s, float* d, const Geo& geo,
+                const StepConst& k, unsigned long long* bad) {
+  if (!mrt) k_step<float, false, false, FLAT><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
+  else if (!q) k_step<float, true, false, FLAT><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
+  else k_step<float, true, true, FLAT><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
 }
 
 // Whether nodes are numbered across rows: where blocks of b nodes per row would leave more
 // than 1 lane in 32 idle.  Numbering them costs 2 % on a row that fills its blocks (256^3
 // FP64 1.798 against 1.834 ms per step, FP32 0.828 against 0.844) and saves the idle lanes:
-// 150 x 110 x 90 FP64 262 -> 175 us (with its own tau_q 313 -> 203), 120 x 128 x 128 233 ->
+// 150 x 110 x 90 FP64 262 -> 175 us (with its own tau_q 313 -> 194), 120 x 128 x 128 233 ->
 // 223, 40 x 120 x 200 309 -> 114; FP32 90 -> 78, 107 -> 103, 82 -> 54.
 bool flat_rows(int nx, int b) {
   const long long lanes = (long long)((nx + b - 1) / b) * b;
@@ -941,8 +1009,13 @@ cudaError_t launch_step(rlb_handle* h, const void* src, void* dst, cudaStream_t 
   if constexpr (sizeof(S) == 8) {
     const int rv = h->k.r_v, rf = h->k.r_f;
     if (h->cfg.eta_over_s > 0) {
-      if (flat) launch_one<S, true, true>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
-      else launch_one<S, false, true>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
+      if (bx == 32) {
+        if (flat) launch_eta<1, true>(mrt, q, grid, st, s, d, geo, h->k, h->d_bad);
+        else launch_eta<1, false>(mrt, q, grid, st, s, d, geo, h->k, h->d_bad);
+      } else {
+        if (flat) launch_eta<RLB_WS_WARPS, true>(mrt, q, grid, st, s, d, geo, h->k, h->d_bad);
+        else launch_eta<RLB_WS_WARPS, false>(mrt, q, grid, st, s, d, geo, h->k, h->d_bad);
+      }
     } else if (bx == 32 && !q) {
       // small lattices, four lanes per node: 8 nodes per 64-thread block
       dim3 gq((geo.nx + 7) / 8, geo.ny, geo.nz);
@@ -958,8 +1031,8 @@ cudaError_t launch_step(rlb_handle* h, const void* src, void* dst, cudaStream_t 
       else launch_ws_coll<RLB_WS_WARPS, false>(mrt, q, rv, rf, grid, st, s, d, geo, h->k, h->d_bad);
     }
   } else {
-    if (flat) launch_one<S, true, false>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
-    else launch_one<S, false, false>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
+    if (flat) launch_f32<true>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
+    else launch_f32<false>(mrt, q, grid, bx, st, s, d, geo, h->k, h->d_bad);
   }
   return cudaGetLastError();
 }
@@ -1065,6 +1138,7 @@ extern "C" int rlb_create(const rlb_config* cfg, rlb_handle** out) {
   h->k = make_step_const(eta_mode && cfg->tau_f <= 0 ? 1.0 : cfg->tau_f, eta_mode ? 1.0 : cfg->tau_v, cfg->tau_e,
                          cfg->tau_eps, cfg->tau_q, cfg->collision == RLB_MRT, h->Q);
   h->k.eta_s = cfg->eta_over_s;
+  h->k.eta3 = 3.0 * cfg->eta_over_s;
   h->k.tauf_local = eta_mode && cfg->tau_f <= 0;
   h->k.a_e = cfg->tau_e;
   h->k.a_p = cfg->tau_eps;

@@ -83,7 +83,7 @@ struct StepConst {
   float ce_f, cp_f, cq_f;
   // fixed-eta/s relaxation: eta_s > 0 derives tau_g (BGK) / tau_v (MRT) per node; tauf_local:
   // tau_f = tau_g; for MRT the ratios a_x = (tau_x - 1/2) / (tau_v - 1/2) of e, eps, q
-  double eta_s;
+  double eta_s, eta3;   // eta3 = 3 eta_s
   int tauf_local;
   double a_e, a_p, a_q;
   // 64-bit fixed-point copies for the integer-pipe FP64 collide: omega * 2^63 (even),
@@ -637,8 +637,7 @@ __device__ __forceinline__ long long to_fixed_pos(double x, int Er) {
   const unsigned tl = lo << 11;
   return (long long)(((unsigned long long)(th >> r) << 32) | __funnelshift_r(tl, th, r));
 }
-
-// The same through the FP64 pipe's int64 conversion (round to nearest even) of K | 1:
+// K * 2^(E - 1079) through the FP64 pipe's int64 conversion (round to nearest even) of K | 1:
 // setting the lowest bit keeps the converted value away from zero, so the exponent
 // can be rebased without a zero test.  It moves K by at most one grid unit (2^-56 of
 // the node's largest population, the grid's own resolution): an exact zero comes out
@@ -660,6 +659,12 @@ __device__ __forceinline__ double from_fixed_pos(long long K, int E) {
   const unsigned up = (rb > 0x400u) | ((rb == 0x400u) & ml);  // round half to even
   const unsigned long long m = (((unsigned long long)mh << 32) | ml) + up;
   return __hiloint2double((int)((unsigned)(m >> 32) + ((unsigned)(E + 6 - lz) << 20)), (int)(unsigned)m);
+}
+
+// K * 2^(E - 1079) by the FP64 pipe's conversion of K itself (zero stays zero): unbiased
+__device__ __forceinline__ double from_fixed_rn(long long K, int E) {
+  const double d = __ll2double_rn(K);
+  return __hiloint2double(__double2hiint(d) + (K != 0 ? (int)((unsigned)(E - 1079) << 20) : 0), __double2loint(d));
 }
 
 template <int DP>
@@ -733,8 +738,10 @@ __device__ __forceinline__ void relax_links(const long long (&X)[19], const EqPi
   for (int p = 0; p < 9; ++p) {
     const long long c = p < 3 ? cA : cD;
     const long long d = ODD ? dq[p] : 0;
-    const long long ya = relax(X[2 * p + 1], ev[p] + od[p], Om, c + d);
-    const long long yb = relax(X[2 * p + 2], ev[p] - od[p], Om, c - d);
+    long long ca = c + d, cb = c - d;
+    if (ODD) asm("" : "+l"(ca), "+l"(cb));   // as in relax_links_store
+    const long long ya = relax(X[2 * p + 1], ev[p] + od[p], Om, ca);
+    const long long yb = relax(X[2 * p + 2], ev[p] - od[p], Om, cb);
     // (DP >> p) & 1 is a constant once the loop is unrolled
     out[2 * p + 1] = ((DP >> p) & 1) ? from_fixed_dp(ya, E) : from_fixed_pos(ya, E);
     out[2 * p + 2] = ((DP >> p) & 1) ? from_fixed_dp(yb, E) : from_fixed_pos(yb, E);
@@ -745,19 +752,29 @@ __device__ __forceinline__ void relax_links(const long long (&X)[19], const EqPi
 // relax_links writing each link straight to out[a * stride] (when st) as soon as it is
 // rounded, so that the results do not all stay live until a final store loop.  ODD: aq
 // holds the energy-flux corrections of the three axes (256^3 step with its own tau_q 2.09 ->
-// 1.97 ms against the nine per-pair values formed up front, 276 -> 180 bytes spilled).
-template <int DP, bool ODD, int R = 0>
+// 2.00 ms against the nine per-pair values formed up front, 276 -> 180 bytes spilled).
+// EXACT: no drift over thousands of steps.  The axis links' odd part comes from half the
+// momentum hM, so that the equilibrium's momentum is the populations' to the unit; the
+// rest link is what the relaxed moving links leave of the distribution's sum `total`; and
+// the conversion sets no low bit.
+template <int DP, bool ODD, int R = 0, bool EXACT = false>
 __device__ __forceinline__ void relax_links_store(const long long (&X)[19], const EqPieces& q, unsigned long long Om,
                                                   long long cA, long long cD, long long (&aq)[3], int E,
-                                                  double* __restrict__ out, unsigned long long stride, bool st) {
+                                                  double* __restrict__ out, unsigned long long stride, bool st,
+                                                  const long long (&hM)[3] = {0, 0, 0}, long long total = 0) {
   const long long KD = q.KA >> 1;
   const long long ev[9] = {q.KA + q.Xx, q.KA + q.Xy, q.KA + q.Xz,
                            KD + ((q.Xx + q.Xy) >> 1) + q.Yxy, KD + ((q.Xx + q.Xy) >> 1) - q.Yxy,
                            KD + ((q.Xx + q.Xz) >> 1) + q.Yxz, KD + ((q.Xx + q.Xz) >> 1) - q.Yxz,
                            KD + ((q.Xy + q.Xz) >> 1) + q.Yyz, KD + ((q.Xy + q.Xz) >> 1) - q.Yyz};
-  const long long od[9] = {q.Zx, q.Zy, q.Zz,
-                           (q.Zx + q.Zy) >> 1, (q.Zx - q.Zy) >> 1, (q.Zx + q.Zz) >> 1, (q.Zx - q.Zz) >> 1,
-                           (q.Zy + q.Zz) >> 1, (q.Zy - q.Zz) >> 1};
+  long long od[9] = {q.Zx, q.Zy, q.Zz,
+                     (q.Zx + q.Zy) >> 1, (q.Zx - q.Zy) >> 1, (q.Zx + q.Zz) >> 1, (q.Zx - q.Zz) >> 1,
+                     (q.Zy + q.Zz) >> 1, (q.Zy - q.Zz) >> 1};
+  if (EXACT) {
+    od[0] = hM[0] - ((od[3] + od[4]) + (od[5] + od[6]));
+    od[1] = hM[1] - ((od[3] - od[4]) + (od[7] + od[8]));
+    od[2] = hM[2] - ((od[5] - od[6]) + (od[7] - od[8]));
+  }
 #pragma unroll
   for (int p = 0; p < 9; ++p) {
     const long long c = p < 3 ? cA : cD;
@@ -767,15 +784,22 @@ __device__ __forceinline__ void relax_links_store(const long long (&X)[19], cons
       constexpr int pi[9] = {0, 1, 2, 0, 0, 0, 0, 1, 1}, pj[9] = {0, 1, 2, 1, 1, 2, 2, 2, 2};
       d = p < 3 ? 4 * aq[pi[p]] : -((p & 1) ? aq[pi[p]] + aq[pj[p]] : aq[pi[p]] - aq[pj[p]]);
     }
-    const long long ya = relax_r<R>(X[2 * p + 1], ev[p] + od[p], Om, c + d);
-    const long long yb = relax_r<R>(X[2 * p + 2], ev[p] - od[p], Om, c - d);
-    const double da = ((DP >> p) & 1) ? from_fixed_dp(ya, E) : from_fixed_pos(ya, E);
-    const double db = ((DP >> p) & 1) ? from_fixed_dp(yb, E) : from_fixed_pos(yb, E);
+    long long ca = c + d, cb = c - d;
+    // kept a separate value: folded into the relaxation's sum, ptxas 13.0 (-O1 and up, not
+    // -O0) can lose a carry between the 32-bit halves (a tube at rest across x then grew a
+    // transverse velocity of 1e-8)
+    if (ODD) asm("" : "+l"(cb));
+    const long long ya = relax_r<R>(X[2 * p + 1], ev[p] + od[p], Om, ca);
+    const long long yb = relax_r<R>(X[2 * p + 2], ev[p] - od[p], Om, cb);
+    const double da = EXACT ? from_fixed_rn(ya, E) : ((DP >> p) & 1) ? from_fixed_dp(ya, E) : from_fixed_pos(ya, E);
+    const double db = EXACT ? from_fixed_rn(yb, E) : ((DP >> p) & 1) ? from_fixed_dp(yb, E) : from_fixed_pos(yb, E);
+    if (EXACT) total -= ya + yb;
     if (st) {
       out[(2 * p + 1) * stride] = da;
       out[(2 * p + 2) * stride] = db;
     }
   }
+  if (EXACT) out[0] = from_fixed_rn(total, E);
 }
 
 // ---- stored populations of either precision on a node's grid (field output, totals)
@@ -1749,15 +1773,15 @@ __device__ __forceinline__ void d9_relax(const D9State& s, unsigned long long D,
   const long long SX = Xx + Xy;
   Eq9 w;
   eq9_pieces<G>(D, Pf, SX, w);
-  // The conserved sums of the equilibrium are those of the populations to the unit (rest
-  // link, and for g the axis links' odd part from M), and 2 units (3 on the diagonals of f)
-  // come off each relaxed link against the truncation of its product and, for g, the
-  // conversion's set low bit.  Without these a run of 40 steps drifted by five times the
-  // FP64 form's error; with them the errors against 64 bits are below that form's
-  // (1200 x 900, 40 steps: e 8.5e-16 -> 6.1e-16, u 3.6e-15 -> 3.0e-15, n 1.5e-15 -> 5.5e-16).
+  // No drift over many steps: g's axis links take what the diagonals leave of the momentum,
+  // the rest link what the relaxed moving links leave of the distribution's sum, and the
+  // conversion sets no low bit.  Truncated sums throughout drifted by five times the FP64
+  // form's error in 40 steps; this form's errors against 64 bits are below that form's
+  // (1200 x 900, 40 steps: e 8.5e-16 -> 4.3e-16, u 3.6e-15 -> 3.0e-15; the sum of N0 moves by
+  // 2e-21 of itself per step against 8e-17).
   const long long rest = s.T00 - 4 * (w.KA + w.KD + SX);
   const unsigned long long Om = G ? r.Omv : r.Omf;
-  long long c0 = (long long)(Om >> 1) - 2, cA = c0, cD = c0 - (INT ? 1 : 0), dq[4] = {0, 0, 0, 0};
+  long long c0 = (long long)(Om >> 1) - 1, cA = c0, cD = c0, dq[4] = {0, 0, 0, 0};
   if (MRT && G) {
     // class sums of g - g^eq (axis (4/3) P + sigma u^2 / 3, diagonal P / 3 + sigma u^2 / 3)
     const long long s3 = 2 * (long long)mulhi((unsigned long long)SX, kTwoThirds);
@@ -1767,7 +1791,6 @@ __device__ __forceinline__ void d9_relax(const D9State& s, unsigned long long D,
     const long long nD = (s.Sd - (P23 >> 1) - s3) >> 3;
     const long long ae = __mul64hi(2 * nD - 4 * n0 - nA, r.CE);
     const long long ap = __mul64hi(nD + 4 * n0 - 2 * nA, r.CP);
-    c0 += 4 * (ae - ap);
     cA += 2 * ap + ae;
     cD -= 2 * ae + ap;
     if (QSEP) {   // q_i = (3|c|^2 - 5) c_i, q^eq_i = -M_i
@@ -1783,7 +1806,7 @@ __device__ __forceinline__ void d9_relax(const D9State& s, unsigned long long D,
   const long long ev[4] = {w.KA + 2 * Xx, w.KA + 2 * Xy, w.KD + Y, w.KD - Y};
   const long long op = (Zx + Zy) >> 1, om = (Zx - Zy) >> 1;
   const long long od[4] = {G ? (s.Mx >> 1) - (op + om) : 2 * Zx, G ? (s.My >> 1) - (op - om) : 2 * Zy, op, om};
-  out[0] = from_fixed<!INT>(relax(s.X[0], rest, Om, c0), s.E);
+  long long left = s.T00;
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
     const long long c = p < 2 ? cA : cD;
@@ -1796,9 +1819,96 @@ __device__ __forceinline__ void d9_relax(const D9State& s, unsigned long long D,
       // third of all nodes).
       asm("" : "+l"(ca), "+l"(cb));
     }
-    out[2 * p + 1] = from_fixed<!INT>(relax(s.X[2 * p + 1], ev[p] + od[p], Om, ca), s.E);
-    out[2 * p + 2] = from_fixed<!INT>(relax(s.X[2 * p + 2], ev[p] - od[p], Om, cb), s.E);
+    const long long ya = relax(s.X[2 * p + 1], ev[p] + od[p], Om, ca);
+    const long long yb = relax(s.X[2 * p + 2], ev[p] - od[p], Om, cb);
+    left -= ya + yb;
+    out[2 * p + 1] = INT ? from_fixed_pos(ya, s.E) : from_fixed_rn(ya, s.E);
+    out[2 * p + 2] = INT ? from_fixed_pos(yb, s.E) : from_fixed_rn(yb, s.E);
   }
+  out[0] = INT ? from_fixed_pos(left, s.E) : from_fixed_rn(left, s.E);
+}
+
+// ---------------------------------------------------------------------------
+// Relaxation rates of a node in the fixed-eta/s mode, on integers (the FP64 form is
+// tau_eta_over_s with set_*_coefficients).  With n = N0 / gamma, T = P / n, w = 1 - u^2 =
+// 4 P / sigma (P = e / 3), the paper's tau_g (Sec. II, III.B) needs neither gamma nor a
+// square root:
+//   n / n_eq = pi^2 N0^4 / (sigma^2 P),  tau_g - 1/2 = 3 (eta/s) (N0 / sigma) (4 - ln(n / n_eq)).
+// The quotients are fixed-point reciprocals and products, the logarithm is the series of
+// 2 artanh((v - 1) / (v + 1)) on v in (0.7, 1.42) (12 terms, below 2^-60) plus a multiple
+// of ln 2, to 2^-55; tau_g itself is formed in FP64.  8 FP64-pipe instructions against
+// about 170 of the FP64 form.
+__device__ __forceinline__ long long ln_fixed(unsigned long long m, int k) {   // ln(m 2^(k - 63)) 2^55, m >= 2^63
+  using namespace fx;
+  const bool up = m > 0xb504f333f9de6484ull;   // sqrt(2) 2^63
+  const unsigned long long v = up ? m >> 1 : m;
+  k += up;
+  const bool neg = up;                          // v < 1
+  const unsigned long long num = neg ? (1ull << 63) - v : v - (1ull << 63);
+  const unsigned long long z = mulhi(num, rcp_fixed((v >> 1) + (1ull << 62)));   // |v - 1| / (v + 1) 2^63
+  const unsigned long long zz = mulhi(z, z) << 2;                                // its square 2^64
+  constexpr unsigned long long c[12] = {   // 2^63 / (2 i + 1)
+      0x8000000000000000ull, 0x2aaaaaaaaaaaaaabull, 0x199999999999999aull, 0x1249249249249249ull,
+      0x0e38e38e38e38e39ull, 0x0ba2e8ba2e8ba2e9ull, 0x09d89d89d89d89d9ull, 0x0888888888888889ull,
+      0x0787878787878788ull, 0x06bca1af286bca1bull, 0x0618618618618618ull, 0x0590b21642c8590bull};
+  unsigned long long acc = c[11];
+#pragma unroll
+  for (int i = 10; i >= 0; --i) acc = c[i] + mulhi(acc, zz);
+  const long long ln = with_sign(mulhi(z, acc) >> 6, neg);                       // 2 z S 2^61, at 2^55
+  // k ln 2 2^55 from ln 2 2^62 in two halves
+  constexpr unsigned long long l2 = 3196577161300663915ull;
+  return ln + (((long long)k * (long long)(l2 >> 32)) << 25) + (((long long)k * (long long)(l2 & 0xffffffffull)) >> 7);
+}
+// 1 / tau as omega 2^63 (even) for tau in (1/2, 2^60)
+__device__ __forceinline__ unsigned long long omega_fixed(double tau) {
+  const int hi = __double2hiint(tau), ex = hi >> 20;
+  const unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 43) |
+                               ((unsigned long long)(unsigned)__double2loint(tau) << 11);
+  const unsigned long long R = fx::rcp_fixed(m);                                 // 2^126 / m
+  return (ex < 1023 ? R << 1 : R >> (ex - 1023)) & ~1ull;
+}
+// False where a quantity leaves the range of this form (N0 <= 0, tau_g outside (1/2 + 2^-30,
+// 2^30), exponents): the FP64 form then decides.
+template <bool MRT, bool QSEP>
+__device__ __forceinline__ bool eta_rates(long long N0, int Ef, unsigned long long sig, long long Pf, int Eg,
+                                          const StepConst& k, Rates& r) {
+  using namespace fx;
+  bool ok = N0 > 0 && Pf > 0 && FxUnit<double>::in_range(Ef) && FxUnit<double>::in_range(Eg);
+  const unsigned long long n0 = ok ? (unsigned long long)N0 : 1ull, p0 = ok ? (unsigned long long)Pf : 1ull;
+  const int ln = __clzll((long long)n0), ls = __clzll((long long)sig), lp = __clzll((long long)p0);
+  const unsigned long long an = n0 << ln;
+  const unsigned long long q = mulhi(an, rcp_fixed(sig << ls));                  // N0 / sigma, in (2^61, 2^63)
+  const int eq = Ef - Eg + ls - ln - 62;                                         // at 2^eq
+  unsigned long long v = mulhi(an, q);                                           // N0^2 / sigma
+  const int c1 = __clzll((long long)v);
+  v <<= c1;
+  v = mulhi(mulhi(v, v), rcp_fixed(p0 << lp));                                   // N0^4 / (sigma^2 P)
+  const int c3 = __clzll((long long)v);
+  v <<= c3;
+  const int e1 = 64 + Ef - 1079 - ln + eq - c1;
+  const int kx = 64 + (64 + 2 * e1) - 126 - Eg + 1079 + lp - c3 + 63;            // v in [1, 2) 2^kx
+  ok = ok && kx > -300 && kx < 300 && eq > -900 && eq < 900;
+  const long long s = 61628706678236207ll - ln_fixed(v, ok ? kx : 0);            // (4 - ln(n / n_eq)) 2^55
+  const double h = k.eta3 * (scale_pow2(__ll2double_rn((long long)q), ok ? eq - 55 : 0) * __ll2double_rn(s));
+  const int hh = __double2hiint(h);
+  ok = ok && hh > ((1023 - 30) << 20) && hh < ((1023 + 30) << 20);
+  const double t = ok ? h : 0.5;
+  r.Omv = omega_fixed(t + 0.5);
+  r.Omf = k.tauf_local ? r.Omv : k.Om_f;
+  r.CE = r.CP = r.CQ = 0;
+  if (MRT) {   // tau_x = 1/2 + a_x (tau_v - 1/2); constants 2^11 / 2394, 2^7 / 252, 2^5 / 40 at 2^63
+    const double te = fma(k.a_e, t, 0.5), tp = fma(k.a_p, t, 0.5), tq = fma(k.a_q, t, 0.5);
+    const int lim = (1023 + 50) << 20;   // taus in (1/2, 2^50): at 1/2 omega 2^63 would be 2^64
+    ok = ok && __double2hiint(te) < lim && __double2hiint(tp) < lim && te > 0.5 && tp > 0.5;
+    const long long wv = (long long)(r.Omv >> 1);
+    r.CE = __mul64hi((long long)(omega_fixed(ok ? te : 1.0) >> 1) - wv, 0x6d801b6006d801b6ll) << 1;
+    r.CP = __mul64hi((long long)(omega_fixed(ok ? tp : 1.0) >> 1) - wv, 0x4104104104104104ll) << 1;
+    if (QSEP) {
+      ok = ok && __double2hiint(tq) < lim && tq > 0.5;
+      r.CQ = __mul64hi((long long)(omega_fixed(ok ? tq : 1.0) >> 1) - wv, 0x6666666666666666ll) << 1;
+    }
+  }
+  return ok;
 }
 
 // ---------------------------------------------------------------------------

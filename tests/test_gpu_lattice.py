@@ -537,3 +537,54 @@ def test_rows_of_any_length_vs_oracle(precision, kw, shape):
     ref = oracle_fields(*O.run(*O.init_populations(e, torch.stack([ux, uy, uz]), n), prm, 3))
     err = field_errors(gpu, ref)
     assert max(err.values()) < (TOL64 if precision == "fp64" else 50 * 2.0 ** -24 * 3 ** 0.5), err
+
+
+@pytest.mark.parametrize("collision, tau_f, tau_q", [("bgk", 0.0, 0.0), ("mrt", 0.6, 0.5), ("mrt", 0.0, 0.0)])
+@pytest.mark.parametrize("shape", [(1, 1, 9), (3, 5, 37), (9, 37, 130)])
+def test_eta_over_s_rates_inside_and_outside_the_integer_form(shape, collision, tau_f, tau_q):
+    """One step with tau from eta/s where tau_g - 1/2 is ordinary, next to zero and negative
+    (n times 1, 4.3, 50: s changes sign near n = e^4 n_eq; such nodes leave the integer
+    rates' range and take the FP64 form): populations against the oracle, 1e-13 of each
+    distribution's largest (one step of a few roundings) times omega^2 where a rate exceeds
+    1: the rounding of tau_x = 1/2 + a_x (tau_g - 1/2) enters omega_x = 1 / tau_x as
+    omega_x^2, and tau_x passes through zero on the negative side."""
+    e, ux, uy, uz, n = I.periodic_box(None, seed=81, shape=shape, e0=3 * 2.4e-7, n0=2.4e-7 / 0.0314, umax=0.2)
+    n = n * torch.tensor([1.0, 1.0, 4.3, 50.0], dtype=torch.float64)[torch.arange(n.numel()) % 4].reshape(shape)
+    kw = dict(collision=collision, tau_f=tau_f, tau_e=0.05, tau_eps=0.1, tau_q=tau_q, eta_over_s=0.1)
+    lat = _lattice(shape, tau_v=0.9, **kw)
+    u = torch.stack([ux, uy, uz])
+    f, g = O.init_populations(e, u, n)
+    lat.load_state(torch.cat([f, g]).cuda())
+    lat.step(1)
+    lat.check()
+    s = lat.state("cpu")
+    lat.close()
+    fo, go = O.step(f, g, O.Params(**kw), check=False)
+    prm = O.Params(**kw)
+    fl = O.fields(O.stream_pull(f, prm.bc), O.stream_pull(g, prm.bc), check=False)
+    h = O.tau_from_eta_over_s(0.1, fl) - 0.5
+    taus = torch.stack([0.5 + a * h for a in (1.0, 0.05, 0.1, tau_q or 1.0)])
+    w2 = (1.0 / taus.abs().amin(0)).clamp(min=1.0) ** 2
+    assert bool(((s[:19] - fo).abs() <= 1e-13 * w2 * fo.abs().max()).all())
+    assert bool(((s[19:] - go).abs() <= 1e-13 * w2 * go.abs().max()).all())
+
+
+@pytest.mark.parametrize("kw", [dict(tau_q=0.7), dict(tau_q=0.7, tau_v=1.3), dict(eta_over_s=0.1, tau_f=0.6, tau_e=0.05,
+                                                                               tau_eps=0.1, tau_q=0.5)])
+@pytest.mark.parametrize("shape", [(1, 1, 320), (5, 4, 2000)])
+def test_flow_along_x_stays_along_x_with_its_own_tau_q(shape, kw):
+    """A shock along x with its own energy-flux time: 20 steps against the oracle, and no
+    transverse velocity at all (equal populations get equal integers)."""
+    bc = ("zero_gradient", "periodic", "periodic")
+    state = I.PAPER_LATTICE_UNITS if "eta_over_s" in kw else {}
+    e, ux, uy, uz, n = (torch.from_numpy(a).expand(shape).contiguous() for a in I.shock_tube(shape[2], **state))
+    kw = dict(dict(collision="mrt", tau_f=0.7, tau_v=0.9, tau_e=0.55, tau_eps=0.8), **kw)
+    lat = _lattice(shape, bc=bc, **kw)
+    lat.set_fields(*(t.cuda() for t in (e, ux, uy, uz, n)))
+    lat.step(20)
+    gpu = lat.fields("cpu")
+    lat.close()
+    assert float(gpu["uy"].abs().max()) == 0.0 and float(gpu["uz"].abs().max()) == 0.0
+    ref = oracle_fields(*O.run(*O.init_populations(e, torch.stack([ux, uy, uz]), n), O.Params(bc=oracle_bc(bc), **kw), 20))
+    err = field_errors(gpu, ref)
+    assert max(err.values()) < TOL64, err
