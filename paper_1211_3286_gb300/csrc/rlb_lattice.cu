@@ -15,6 +15,7 @@
 //     when the C7 correction needs gradients of the macroscopic fields.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <cstdio>
@@ -51,6 +52,8 @@ int cuda_fail(rlb_handle* h, cudaError_t e, const char* what) {
   } while (0)
 
 constexpr int kBlockX = 128;
+constexpr unsigned long long kSmallNodes = 152ull * 128ull * 2ull;   // lattices that cannot fill the GPU
+constexpr int kTubeWarps = 4;     // g (and f) warps of a block of k_tube_steps
 constexpr int kRedBlocks = 608;   // 4 x 152 SMs; fixed so the reduction order is fixed
 constexpr int kRedThreads = 256;
 
@@ -451,16 +454,17 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? (ETA ? 8 : 14) : RLB_WS_WARPS
   }
 }
 
-// FP64 step for small lattices with four lanes per node and distribution: a 64-thread
-// block serves 8 nodes along x, warp 0 their g and warp 1 their f.  Lane j = 0, 1, 2 of
-// a node holds axis pair j (links 2j + 1, 2j + 2) and the two diagonal pairs of one
-// plane, (a, b) = (x, y), (y, z), (x, z): the pairs e_a + e_b and e_a - e_b (pairs 3-4,
-// 7-8, 5-6), six links each; lane 3 holds the rest link.  The block exponent, the exact
-// integer sums and the rest value are combined over the node's lanes with shuffles, the
-// recovery and the equilibrium pieces run in every lane, and each lane relaxes and
-// stores its own links: the arithmetic of k_step_ws, link for link, with a node's
-// dependent chain about a third as long.  u goes to the f warp through shared memory
-// across named barrier 1.  No separate tau_q (QSEP) in this form.
+// ---- FP64 steps of small lattices: four lanes per node and distribution
+//
+// A g warp holds the g of 8 nodes along x, an f warp their f.  Lane j = 0, 1, 2 of a node
+// holds axis pair j (links 2j + 1, 2j + 2) and the two diagonal pairs of one plane, (a, b)
+// = (x, y), (y, z), (x, z): the pairs e_a + e_b and e_a - e_b (pairs 3-4, 7-8, 5-6), six
+// links each; lane 3 holds the rest link.  The block exponent, the exact integer sums and
+// the rest value are combined over the node's lanes with shuffles, the recovery and the
+// equilibrium pieces run in every lane, and each lane relaxes its own links: the
+// arithmetic of k_step_ws, link for link, with a node's dependent chain about a third as
+// long.  u goes to the f warp through shared memory across a named barrier of the warp
+// pair.  No separate tau_q (QSEP) in this form.
 __device__ __forceinline__ long long quad_sum64(long long v) {
   v += __shfl_xor_sync(0xffffffffu, v, 1);
   v += __shfl_xor_sync(0xffffffffu, v, 2);
@@ -469,62 +473,43 @@ __device__ __forceinline__ long long quad_sum64(long long v) {
 __device__ __forceinline__ long long sel3(int j, long long v0, long long v1, long long v2) {
   return j == 0 ? v0 : (j == 1 ? v1 : v2);
 }
-
-template <bool MRT, int RV, int RF>
-__global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ src, double* __restrict__ dst, Geo geo,
-                                                     StepConst k, unsigned long long* __restrict__ bad) {
-  using namespace fx;
-  __shared__ unsigned long long s_ax[8], s_ay[8], s_az[8];
-  __shared__ unsigned s_sg[8];
-  const int lane = threadIdx.x & 31;
-  const bool is_g = threadIdx.x < 32;
-  const int m = lane >> 2, j = lane & 3;
-  const int xv = blockIdx.x * 8 + m;
-  const bool valid = xv < geo.nx;
-  const int x = valid ? xv : geo.nx - 1;
-  const int y = blockIdx.y, z = blockIdx.z;
-  const int xm = src_minus(x, geo.nx, geo.bcx), xp = src_plus(x, geo.nx, geo.bcx);
-  const int ym = src_minus(y, geo.ny, geo.bcy), yp = src_plus(y, geo.ny, geo.bcy);
-  const int zm = src_minus(z, geo.nz, geo.bcz), zp = src_plus(z, geo.nz, geo.bcz);
-  // this lane's axes: axis pair i = j; diagonal plane (a, b) = (x, y), (y, z), (x, z)
-  const int ai = j < 3 ? j : 0, da = j == 1 ? 1 : 0, db = j == 0 ? 1 : 2;
+// slot sl of lane j: link and direction (slots 0-1 the axis pair, 2-3 the first diagonal
+// pair of the lane's plane, 4-5 the second); lane 3 reads the rest link in every slot
+__device__ __forceinline__ int quad_link(int j, int sl) {
   const int pd = j == 0 ? 3 : (j == 1 ? 7 : 5);   // first diagonal pair of the plane
-  // slot sl: link and direction (slots 0-1 the axis pair, 2-3 pair pd, 4-5 pair pd + 1);
-  // lane 3 reads the rest link in every slot
-  int link[6], cxs[6], cys[6], czs[6];
-#pragma unroll
-  for (int sl = 0; sl < 6; ++sl) {
-    int cx, cy, cz;
-    if (sl < 2) {
-      const int c = sl == 0 ? 1 : -1;
-      cx = ai == 0 ? c : 0;
-      cy = ai == 1 ? c : 0;
-      cz = ai == 2 ? c : 0;
-      link[sl] = 2 * ai + 1 + sl;
-    } else {
-      const int sa = (sl & 1) ? -1 : 1;              // +(e_a + e_b), -(e_a + e_b), +(e_a - e_b), -(e_a - e_b)
-      const int sb = sl < 4 ? sa : -sa;
-      cx = da == 0 ? sa : 0;                          // db is never x
-      cy = (da == 1 ? sa : 0) + (db == 1 ? sb : 0);
-      cz = db == 2 ? sb : 0;                          // da is never z
-      link[sl] = 2 * pd + 1 + (sl - 2);
-    }
-    const bool rest = j == 3;
-    link[sl] = rest ? 0 : link[sl];
-    cxs[sl] = rest ? 0 : cx;
-    cys[sl] = rest ? 0 : cy;
-    czs[sl] = rest ? 0 : cz;
+  return j == 3 ? 0 : sl < 2 ? 2 * j + 1 + sl : 2 * pd + 1 + (sl - 2);
+}
+__device__ __forceinline__ void quad_dir(int j, int sl, int& cx, int& cy, int& cz) {
+  const int da = j == 1 ? 1 : 0, db = j == 0 ? 1 : 2;
+  if (sl < 2) {
+    const int c = sl == 0 ? 1 : -1;
+    cx = j == 0 ? c : 0;
+    cy = j == 1 ? c : 0;
+    cz = j == 2 ? c : 0;
+  } else {
+    const int sa = (sl & 1) ? -1 : 1;              // +(e_a + e_b), -(e_a + e_b), +(e_a - e_b), -(e_a - e_b)
+    const int sb = sl < 4 ? sa : -sa;
+    cx = da == 0 ? sa : 0;                          // db is never x
+    cy = (da == 1 ? sa : 0) + (db == 1 ? sb : 0);
+    cz = db == 2 ? sb : 0;                          // da is never z
   }
-  const unsigned long long plane0 = is_g ? 19ull * geo.plane : 0ull;
-  double v[6];
-#pragma unroll
-  for (int sl = 0; sl < 6; ++sl) {
-    const int sx = cxs[sl] > 0 ? xm : (cxs[sl] < 0 ? xp : x);
-    const int sy = cys[sl] > 0 ? ym : (cys[sl] < 0 ? yp : y);
-    const int sz = czs[sl] > 0 ? zm : (czs[sl] < 0 ? zp : z);
-    const unsigned idx = ((unsigned)sz * (unsigned)geo.ny + (unsigned)sy) * (unsigned)geo.nx + (unsigned)sx;
-    v[sl] = ldg_nc(src + plane0 + (unsigned long long)link[sl] * geo.plane + idx);
-  }
+  if (j == 3) cx = cy = cz = 0;
+}
+// u of the 8 nodes of a warp pair
+struct QuadU {
+  unsigned long long ax[8], ay[8], az[8];
+  unsigned sg[8];
+};
+// Collides the pulled values v of lane (m, j) and leaves the relaxed ones in v (lane 3:
+// the rest link in v[0]); true if the node is non-physical (valid in every lane of a g
+// warp; of an f warp: its own exponent).  PAIR: an f warp runs beside the g warp (named
+// barrier bar_id); else g alone.
+template <bool MRT, int RV, int RF, bool PAIR = true>
+__device__ __forceinline__ bool quad_collide(bool is_g, int lane, double (&v)[6], const StepConst& k, QuadU& su,
+                                             int bar_id) {
+  using namespace fx;
+  const int m = lane >> 2, j = lane & 3;
+  const int ai = j < 3 ? j : 0, da = j == 1 ? 1 : 0, db = j == 0 ? 1 : 2;
   // block exponent over the node's 19 values (max over its four lanes)
   int hmax = __double2hiint(v[0]), hmin = hmax;
 #pragma unroll
@@ -575,23 +560,23 @@ __global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ 
     bool br;
     sig = fx_recover(T00, Mx, My, Mz, u, br);
     Pf = (long long)sig - T00;
-    if (j == 0) {
-      s_ax[m] = u.ax;
-      s_ay[m] = u.ay;
-      s_az[m] = u.az;
-      s_sg[m] = u.sx | (u.sy << 1) | (u.sz << 2);
+    if (PAIR && j == 0) {
+      su.ax[m] = u.ax;
+      su.ay[m] = u.ay;
+      su.az[m] = u.az;
+      su.sg[m] = u.sx | (u.sy << 1) | (u.sz << 2);
     }
     ufix_products(u);
     b |= br | (Pf <= 0) | (u.xx + u.yy + u.zz >= (1ull << 62));
   } else {
     N0 = Xr + quad_sum64(pairs ? (spa + spp) + spm : 0);
   }
-  asm volatile("bar.sync 1, 64;" ::: "memory");
+  if (PAIR) asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
   if (!is_g) {
-    u.ax = s_ax[m];
-    u.ay = s_ay[m];
-    u.az = s_az[m];
-    const unsigned sg = s_sg[m];
+    u.ax = su.ax[m];
+    u.ay = su.ay[m];
+    u.az = su.az[m];
+    const unsigned sg = su.sg[m];
     u.sx = sg & 1u;
     u.sy = (sg >> 1) & 1u;
     u.sz = sg >> 2;
@@ -623,9 +608,6 @@ __global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ 
     cA += 11 * ae + 4 * ap;
     cD -= 8 * ae + ap;
   }
-  const unsigned node = ((unsigned)z * (unsigned)geo.ny + (unsigned)y) * (unsigned)geo.nx + (unsigned)x;
-  if (valid && b && j == 0) atomicMin(bad, (unsigned long long)node);
-  double* out = dst + plane0 + node;
   if (pairs) {
     // axis pair: ev = KA + X_i, od = Z_i; diagonal pairs: ev = KA/2 + (X_a + X_b)/2 +- Y_ab,
     // od = (Z_a +- Z_b)/2 (the pieces of relax_links_store)
@@ -640,16 +622,138 @@ __global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ 
     const long long y0 = rlx(X[0], evA + odA, Om, cA), y1 = rlx(X[1], evA - odA, Om, cA);
     const long long y2 = rlx(X[2], evP + odP, Om, cD), y3 = rlx(X[3], evP - odP, Om, cD);
     const long long y4 = rlx(X[4], evM + odM, Om, cD), y5 = rlx(X[5], evM - odM, Om, cD);
-    {   // every lane stores (lanes past the row repeat node nx - 1 bit for bit)
-      out[(unsigned long long)link[0] * geo.plane] = from_fixed_dp(y0, E);
-      out[(unsigned long long)link[1] * geo.plane] = from_fixed_dp(y1, E);
-      out[(unsigned long long)link[2] * geo.plane] = from_fixed_dp(y2, E);
-      out[(unsigned long long)link[3] * geo.plane] = from_fixed_dp(y3, E);
-      out[(unsigned long long)link[4] * geo.plane] = from_fixed_dp(y4, E);
-      out[(unsigned long long)link[5] * geo.plane] = from_fixed_dp(y5, E);
-    }
+    v[0] = from_fixed_dp(y0, E);
+    v[1] = from_fixed_dp(y1, E);
+    v[2] = from_fixed_dp(y2, E);
+    v[3] = from_fixed_dp(y3, E);
+    v[4] = from_fixed_dp(y4, E);
+    v[5] = from_fixed_dp(y5, E);
   } else {
-    out[0] = from_fixed_dp(rlx(X[0], eq0, Om, c0), E);
+    v[0] = from_fixed_dp(rlx(X[0], eq0, Om, c0), E);
+#pragma unroll
+    for (int sl = 1; sl < 6; ++sl) v[sl] = v[0];   // the rest link in every slot, as pulled
+  }
+  return b;
+}
+
+// One step of a small lattice: a 64-thread block serves 8 nodes along x.
+template <bool MRT, int RV, int RF>
+__global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ src, double* __restrict__ dst, Geo geo,
+                                                     StepConst k, unsigned long long* __restrict__ bad) {
+  __shared__ QuadU su;
+  const int lane = threadIdx.x & 31;
+  const bool is_g = threadIdx.x < 32;
+  const int m = lane >> 2, j = lane & 3;
+  const int xv = blockIdx.x * 8 + m;
+  const bool valid = xv < geo.nx;
+  const int x = valid ? xv : geo.nx - 1;
+  const int y = blockIdx.y, z = blockIdx.z;
+  const int xm = src_minus(x, geo.nx, geo.bcx), xp = src_plus(x, geo.nx, geo.bcx);
+  const int ym = src_minus(y, geo.ny, geo.bcy), yp = src_plus(y, geo.ny, geo.bcy);
+  const int zm = src_minus(z, geo.nz, geo.bcz), zp = src_plus(z, geo.nz, geo.bcz);
+  const unsigned long long plane0 = is_g ? 19ull * geo.plane : 0ull;
+  double v[6];
+#pragma unroll
+  for (int sl = 0; sl < 6; ++sl) {
+    int cx, cy, cz;
+    quad_dir(j, sl, cx, cy, cz);
+    const int sx = cx > 0 ? xm : (cx < 0 ? xp : x);
+    const int sy = cy > 0 ? ym : (cy < 0 ? yp : y);
+    const int sz = cz > 0 ? zm : (cz < 0 ? zp : z);
+    const unsigned idx = ((unsigned)sz * (unsigned)geo.ny + (unsigned)sy) * (unsigned)geo.nx + (unsigned)sx;
+    v[sl] = ldg_nc(src + plane0 + (unsigned long long)quad_link(j, sl) * geo.plane + idx);
+  }
+  const bool b = quad_collide<MRT, RV, RF>(is_g, lane, v, k, su, 1);
+  const unsigned node = ((unsigned)z * (unsigned)geo.ny + (unsigned)y) * (unsigned)geo.nx + (unsigned)x;
+  if (valid && b && j == 0) atomicMin(bad, (unsigned long long)node);
+  double* out = dst + plane0 + node;
+  // every lane stores (lanes past the row repeat node nx - 1 bit for bit)
+  out[(unsigned long long)quad_link(j, 0) * geo.plane] = v[0];
+  if (j < 3) {
+#pragma unroll
+    for (int sl = 1; sl < 6; ++sl) out[(unsigned long long)quad_link(j, sl) * geo.plane] = v[sl];
+  }
+}
+
+// Several steps of a quasi-1D lattice (ny = nz = 1) per launch.  A block holds kTubeTile nodes
+// in registers (four lanes per node and distribution) and advances them by `steps`: the
+// first step pulls from src, later ones exchange the x-moving links through shared memory.
+// What a block does not know of its neighbours grows inwards by one node per later step,
+// so it stores the `core` nodes in its middle, core <= kTubeTile - 2 (steps - 1): neighbouring
+// blocks advance the overlap as well, with the same arithmetic, instead of waiting for one
+// another.  k_step_quad takes 6.2 us per step of a 1600-node tube, launched one after the
+// other (4.7 with BGK): 4 of them are the launch and the loads' latency, 2.1 the dependent
+// integer chain.  Here a launch of 10 steps takes 1.4 + 10 x 2.24 us; the bound is that chain
+// (issue slots 66 % busy on the SMs that have a block).  1600 nodes: 6.17 -> 2.37 us per step,
+// 6400: 6.18 -> 3.31, 38912: 16.5 -> 13.4.  Tried: 16- and 64-node tiles (2.58 and 3.7 us at
+// 1600 nodes), the output rounding on the integer pipe (2.84 against 2.59 at 8 steps).
+//   G_ONLY: g alone (it does not depend on f), every step's g stored at dst + s * stride (the
+//   adjoint's recompute).
+constexpr int kTubeTile = 8 * kTubeWarps;
+template <bool MRT, int RV, int RF, bool G_ONLY>
+__global__ void __launch_bounds__((G_ONLY ? 32 : 64) * kTubeWarps)
+    k_tube_steps(const double* __restrict__ src, double* __restrict__ dst, int nx, int bcx, StepConst k, int steps,
+                 int core, unsigned long long stride, unsigned long long* __restrict__ bad) {
+  __shared__ QuadU su[kTubeWarps];
+  __shared__ double ex[2][G_ONLY ? 1 : 2][2][6][kTubeTile];   // [parity][role][lane 0 / 2][slot][node]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m = lane >> 2, j = lane & 3;
+  const bool is_g = G_ONLY || warp < kTubeWarps;
+  const int pair = is_g ? warp : warp - kTubeWarps;
+  const int i = pair * 8 + m;                                   // node of the tile
+  const int halo = (kTubeTile - core) >> 1;
+  const int xg = (int)blockIdx.x * core - halo + i;             // its place in the lattice
+  const bool own = i >= halo && i < halo + core && xg < nx;     // stored (and checked) by this block
+  int x = xg;
+  if (bcx) x = min(max(xg, 0), nx - 1);                         // past an open end: idle copies
+  else x = xg < 0 ? (xg % nx + nx) % nx : xg % nx;
+  const unsigned long long n = (unsigned long long)nx;
+  const double* in = src + (is_g ? 19ull * n : 0ull);
+  const double* at[6];
+#pragma unroll
+  for (int sl = 0; sl < 6; ++sl) {
+    int cx, cy, cz;
+    quad_dir(j, sl, cx, cy, cz);
+    const int sx = cx > 0 ? src_minus(x, nx, bcx) : (cx < 0 ? src_plus(x, nx, bcx) : x);
+    at[sl] = in + (unsigned long long)quad_link(j, sl) * n + (unsigned)sx;
+  }
+  double v[6];
+  // launched while the grid before it drains (launch_tube_as): nothing is read or written
+  // until that grid is complete
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll
+  for (int sl = 0; sl < 6; ++sl) v[sl] = __ldcg(at[sl]);
+  // sources of the exchange: the tile's neighbours, at an open end the node itself; a tile
+  // that holds the whole lattice (core = kTubeTile, no overlap) wraps onto itself
+  const bool whole = core == kTubeTile;
+  const int im = xg == 0 && (bcx || whole) ? (bcx ? i : nx - 1) : max(i - 1, 0);
+  const int ip = xg == nx - 1 && (bcx || whole) ? (bcx ? i : 0) : min(i + 1, kTubeTile - 1);
+  const bool axis_moves = j == 0, moves = j == 0 || j == 2;     // slots 0-1; slots 2-5
+  for (int s = 0;; ++s) {
+    const bool b = quad_collide<MRT, RV, RF, !G_ONLY>(is_g, lane, v, k, su[pair], 1 + pair);
+    if (own && b && j == 0) atomicMin(bad, (unsigned long long)x);
+    if (G_ONLY || s == steps - 1) {
+      if (own) {
+        double* out = dst + (G_ONLY ? (unsigned long long)s * stride : (is_g ? 19ull * n : 0ull)) + (unsigned)x;
+        out[(unsigned long long)quad_link(j, 0) * n] = v[0];
+        if (j < 3) {
+#pragma unroll
+          for (int sl = 1; sl < 6; ++sl) out[(unsigned long long)quad_link(j, sl) * n] = v[sl];
+        }
+      }
+      if (s == steps - 1) return;
+    }
+    auto& e = ex[s & 1][is_g ? 0 : 1][j >> 1];
+    if (moves) {
+#pragma unroll
+      for (int sl = 0; sl < 6; ++sl)
+        if (sl >= 2 || axis_moves) e[sl][i] = v[sl];
+    }
+    __syncthreads();
+    if (moves) {
+#pragma unroll
+      for (int sl = 0; sl < 6; ++sl)
+        if (sl >= 2 || axis_moves) v[sl] = e[sl][(sl & 1) ? ip : im];
+    }
   }
 }
 
@@ -969,12 +1073,63 @@ void launch_quad(int rv, int rf, dim3 grid, cudaStream_t st, const double* s, do
   else k_step_quad<MRT, 1, 1><<<grid, 64, 0, st>>>(s, d, geo, k, bad);
 }
 
+template <bool MRT, int RV, int RF, bool G_ONLY>
+void launch_tube_as(int grid, cudaStream_t st, const double* s, double* d, const Geo& geo, const StepConst& k,
+                    int steps, int core, unsigned long long stride, unsigned long long* bad) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)grid);
+  lc.blockDim = dim3((G_ONLY ? 32 : 64) * kTubeWarps);
+  lc.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits for the grid before it
+  at.val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = &at;
+  lc.numAttrs = 1;
+  cudaLaunchKernelEx(&lc, k_tube_steps<MRT, RV, RF, G_ONLY>, s, d, geo.nx, geo.bcx, k, steps, core, stride, bad);
+}
+template <bool MRT, bool G_ONLY>
+void launch_tube(int rv, int rf, int grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
+                 const StepConst& k, int steps, int core, unsigned long long stride, unsigned long long* bad) {
+  if (G_ONLY) rf = rv;   // f is not advanced
+  if (rv == 2 && rf == 2) launch_tube_as<MRT, 2, 2, G_ONLY>(grid, st, s, d, geo, k, steps, core, stride, bad);
+  else if (rv == 2) launch_tube_as<MRT, 2, G_ONLY ? 2 : 1, G_ONLY>(grid, st, s, d, geo, k, steps, core, stride, bad);
+  else if (rf == 2) launch_tube_as<MRT, 1, G_ONLY ? 1 : 2, G_ONLY>(grid, st, s, d, geo, k, steps, core, stride, bad);
+  else launch_tube_as<MRT, 1, 1, G_ONLY>(grid, st, s, d, geo, k, steps, core, stride, bad);
+}
+
+// Whether several steps go into one launch (k_tube_steps), and how many.
+int tube_launch_steps(const rlb_handle* h, int& core) {
+  const rlb_config& c = h->cfg;
+  if (h->Q != 19 || h->esize != 8 || c.ny != 1 || c.nz != 1 || h->nodes > kSmallNodes || c.eta_over_s > 0 || qsep(c))
+    return 1;
+  if (c.nx <= kTubeTile) {   // one block holds the lattice
+    core = kTubeTile;
+    return INT_MAX;
+  }
+  // H steps per launch cost 1.4 us / H for the launch and, per step, the chain (2.24 us) times
+  // what w blocks per SM slow it down (measured: 1 block 1.0, 2 1.4, 3 1.8, 6 3.6, 9 5.7);
+  // more steps mean a smaller core and so more blocks
+  float best = 1e30f;
+  int H = 2;
+  for (int t = 2; t <= 12; ++t) {
+    const int c = kTubeTile - 2 * (t - 1);
+    const int w = (((int)h->nodes + c - 1) / c + 151) / 152;
+    const float cost = 1.4f / t + 2.24f * std::max(1.0f, 0.1f + 0.62f * w);
+    if (cost < best) {
+      best = cost;
+      H = t;
+    }
+  }
+  core = kTubeTile - 2 * (H - 1);
+  return H;
+}
+
 template <typename S>
 cudaError_t launch_step(rlb_handle* h, const void* src, void* dst, cudaStream_t st) {
   const Geo geo = make_geo(h);
   if (h->Q == 9) {
     // small planes spread over more SMs with one warp per block
-    const int bx = h->nodes <= 152ull * 128ull * 2ull ? 32 : kBlockX;
+    const int bx = h->nodes <= kSmallNodes ? 32 : kBlockX;
     const unsigned gr = (unsigned)((h->nodes + bx - 1) / bx);
     const bool mrt2 = h->cfg.collision == RLB_MRT, q2 = qsep(h->cfg);
     const double* s2 = (const double*)src;
@@ -999,7 +1154,7 @@ cudaError_t launch_step(rlb_handle* h, const void* src, void* dst, cudaStream_t 
   // small lattices (a 1600-node tube) spread over more SMs with one warp per block:
   // the FP64 pipe of an SM serves 2 lanes per clock, so fewer warps per SM means
   // shorter steps when the lattice cannot fill the GPU anyway
-  const int bx = h->nodes <= 152ull * 128ull * 2ull ? 32 : kBlockX;
+  const int bx = h->nodes <= kSmallNodes ? 32 : kBlockX;
   const bool flat = flat_rows(geo.nx, bx);
   const dim3 grid = flat ? dim3((unsigned)((h->nodes + bx - 1) / bx))
                          : dim3((unsigned)((geo.nx + bx - 1) / bx), geo.ny, geo.nz);
@@ -1071,6 +1226,25 @@ namespace rlb {
 void set_handleless_error(const std::string& msg) { g_create_error = msg; }
 
 cudaError_t enqueue_steps(rlb_handle* h, int nsteps, cudaStream_t st) {
+  int core = 0;
+  const int most = tube_launch_steps(h, core);
+  for (int s = 0; s < nsteps && most > 1 && nsteps > 1;) {
+    const int n = std::min(most, nsteps - s);
+    const Geo geo = make_geo(h);
+    const int grid = (geo.nx + core - 1) / core;
+    const double* src = (const double*)h->lat[h->cur];
+    double* dst = (double*)h->lat[1 - h->cur];
+    if (h->cfg.collision == RLB_MRT)
+      launch_tube<true, false>(h->k.r_v, h->k.r_f, grid, st, src, dst, geo, h->k, n, core, 0, h->d_bad);
+    else
+      launch_tube<false, false>(h->k.r_v, h->k.r_f, grid, st, src, dst, geo, h->k, n, core, 0, h->d_bad);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    h->cur = 1 - h->cur;
+    h->steps += n;
+    s += n;
+    if (s == nsteps) return cudaSuccess;
+  }
   for (int s = 0; s < nsteps; ++s) {
     const void* src = h->lat[h->cur];
     void* dst = h->lat[1 - h->cur];

@@ -588,3 +588,49 @@ def test_flow_along_x_stays_along_x_with_its_own_tau_q(shape, kw):
     ref = oracle_fields(*O.run(*O.init_populations(e, torch.stack([ux, uy, uz]), n), O.Params(bc=oracle_bc(bc), **kw), 20))
     err = field_errors(gpu, ref)
     assert max(err.values()) < TOL64, err
+
+
+@pytest.mark.parametrize("bcx", ["zero_gradient", "periodic"])
+@pytest.mark.parametrize("L", [1, 2, 7, 31, 32, 33, 45, 400, 1607, 6400, 38912])
+def test_tube_steps_per_launch_bitwise_equal_single_steps(L, bcx):
+    """Quasi-1D lattices advance several steps per launch in overlapping tiles: 1, 2, 3, 12, 13
+    and 29 steps in one call against as many calls of one step (the one-step kernel), bit
+    for bit; tiles that hold the whole lattice, ragged last tiles, MRT and BGK."""
+    e, ux, uy, uz, n = I.periodic_box(None, seed=91, shape=(1, 1, L), umax=0.4)
+    for kw in (dict(collision="mrt", tau_f=0.7), dict(collision="bgk", tau_f=1.3)):
+        a = _lattice((1, 1, L), tau_v=0.9, tau_e=0.55, tau_eps=0.8, bc=(bcx, "periodic", "periodic"), **kw)
+        b = _lattice((1, 1, L), tau_v=0.9, tau_e=0.55, tau_eps=0.8, bc=(bcx, "periodic", "periodic"), **kw)
+        for l in (a, b):
+            l.set_fields(*(t.cuda() for t in (e, ux, uy, uz, n)))
+        for steps in (1, 2, 3, 12, 13, 29):
+            a.step(steps)
+            for _ in range(steps):
+                b.step(1)
+            assert a.steps_done() == b.steps_done()
+            assert torch.equal(a.state().view(torch.int64), b.state().view(torch.int64)), steps
+        a.close()
+        b.close()
+
+
+def test_tube_steps_flag_the_non_physical_node():
+    """A bad node inside a launch of several steps is reported (the smallest index), and an
+    idle lane past an open end is not."""
+    from paper_1211_3286_gb300 import _lib as L
+    lat = _lattice((1, 1, 100), tau_v=0.9, tau_e=0.55, tau_eps=0.8, bc=("zero_gradient", "periodic", "periodic"))
+    e, ux, uy, uz, n = _tube(100)
+    lat.set_fields(*(t.cuda() for t in (e, ux, uy, uz, n)))
+    lat.step(25)
+    lat.check()
+    st = lat.state()
+    st[19 + 1, 0, 0, 59] = 1.0      # node 60 pulls +x from 59 and -x from 61
+    st[19 + 2, 0, 0, 61] = -0.9
+    lat.load_state(st)
+    lat.step(1)
+    with pytest.raises(L.RlbError) as one:
+        lat.check()
+    lat.load_state(st)
+    lat.step(5)
+    with pytest.raises(L.RlbError) as ex:
+        lat.check()
+    assert ex.value.code == L.RLB_ENONPHYS and one.value.code == L.RLB_ENONPHYS
+    lat.close()
