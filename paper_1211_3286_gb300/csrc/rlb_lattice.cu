@@ -72,7 +72,20 @@ __device__ __forceinline__ int src_plus(int i, int n, int zg) {   // source of a
   return i < n - 1 ? i + 1 : (zg ? n - 1 : 0);
 }
 
-// Read-only population load.  FP64 populations are streamed past L1 (each value is
+// A step kernel is launched while the grid before it in the stream drains (launch_after):
+// this waits until that grid is complete and its writes are visible.  The pointers pass
+// through, so that no load from them can be moved up; they are read with coherent loads,
+// since the grid before writes while this kernel is already resident.
+template <typename T>
+__device__ __forceinline__ void wait_for_grid(const T* __restrict__& p) {
+  asm volatile("griddepcontrol.wait;" : "+l"(p)::"memory");
+}
+template <typename T>
+__device__ __forceinline__ void wait_for_grid(const T* __restrict__& p, const T* __restrict__& q) {
+  asm volatile("griddepcontrol.wait;" : "+l"(p), "+l"(q)::"memory");
+}
+
+// Population load.  FP64 populations are streamed past L1 (each value is
 // read once per step from its plane; L2 serves the neighbouring rows' reuse), which
 // leaves L1 to the FP64 step's register spills.
 #ifndef RLB_LD_NOALLOC
@@ -89,9 +102,9 @@ __device__ __forceinline__ S ldg_nc(const S* p) { return __ldg(p); }
 template <>
 __device__ __forceinline__ double ldg_nc<double>(const double* p) {
   double v;
-  if (RLB_LD_PF == 256) asm("ld.global.nc.L1::no_allocate.L2::256B.f64 %0, [%1];" : "=d"(v) : "l"(p));
-  else if (RLB_LD_PF == 128) asm("ld.global.nc.L1::no_allocate.L2::128B.f64 %0, [%1];" : "=d"(v) : "l"(p));
-  else asm("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  if (RLB_LD_PF == 256) asm("ld.global.L1::no_allocate.L2::256B.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  else if (RLB_LD_PF == 128) asm("ld.global.L1::no_allocate.L2::128B.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  else asm("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
   return v;
 }
 #endif
@@ -99,8 +112,8 @@ __device__ __forceinline__ double ldg_nc<double>(const double* p) {
 template <>
 __device__ __forceinline__ float ldg_nc<float>(const float* p) {
   float v;
-  if (RLB_LD_PF == 256) asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  else asm("ld.global.nc.L2::128B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  if (RLB_LD_PF == 256) asm("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  else asm("ld.global.L2::128B.f32 %0, [%1];" : "=f"(v) : "l"(p));
   return v;
 }
 #endif
@@ -168,6 +181,7 @@ __global__ void __launch_bounds__(kBlockX, RLB_F32_BLOCKS_PER_SM) k_step(const S
     node = blockIdx.x * blockDim.x + threadIdx.x;
     if (node >= geo.plane) return;
     const Nbr3 nb = neighbours3(geo, node);
+    wait_for_grid(src);
     pull19<S>(src, geo.plane, node, nb, f);
     pull19<S>(src + 19ull * geo.plane, geo.plane, node, nb, g);
   } else {
@@ -184,6 +198,7 @@ __global__ void __launch_bounds__(kBlockX, RLB_F32_BLOCKS_PER_SM) k_step(const S
 #pragma unroll
       for (int j = 0; j < 3; ++j)
         row[i][j] = ((unsigned)zs[i] * (unsigned)geo.ny + (unsigned)ys[j]) * (unsigned)geo.nx;
+    wait_for_grid(src);
     pull19<S>(src, geo.plane, xs, row, f);
     pull19<S>(src + 19ull * geo.plane, geo.plane, xs, row, g);
     node = row[1][1] + (unsigned)x;
@@ -267,7 +282,9 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? (ETA ? 8 : 14) : RLB_WS_WARPS
     const unsigned i = blockIdx.x * (32 * W) + slot;
     valid = i < geo.plane;
     node = valid ? i : (unsigned)geo.plane - 1;
-    pull19<double>(src + plane0, geo.plane, node, neighbours3(geo, node), v);
+    const Nbr3 nb = neighbours3(geo, node);
+    wait_for_grid(src);
+    pull19<double>(src + plane0, geo.plane, node, nb, v);
   } else {
     const int x0 = blockIdx.x * (32 * W) + slot;
     valid = x0 < geo.nx;
@@ -282,6 +299,7 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? (ETA ? 8 : 14) : RLB_WS_WARPS
 #pragma unroll
       for (int j = 0; j < 3; ++j)
         row[i][j] = ((unsigned)zs[i] * (unsigned)geo.ny + (unsigned)ys[j]) * (unsigned)geo.nx;
+    wait_for_grid(src);
     pull19<double>(src + plane0, geo.plane, xs, row, v);
     node = row[1][1] + (unsigned)x;
   }
@@ -652,6 +670,7 @@ __global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ 
   const int ym = src_minus(y, geo.ny, geo.bcy), yp = src_plus(y, geo.ny, geo.bcy);
   const int zm = src_minus(z, geo.nz, geo.bcz), zp = src_plus(z, geo.nz, geo.bcz);
   const unsigned long long plane0 = is_g ? 19ull * geo.plane : 0ull;
+  wait_for_grid(src);
   double v[6];
 #pragma unroll
   for (int sl = 0; sl < 6; ++sl) {
@@ -717,11 +736,10 @@ __global__ void __launch_bounds__((G_ONLY ? 32 : 64) * kTubeWarps)
     at[sl] = in + (unsigned long long)quad_link(j, sl) * n + (unsigned)sx;
   }
   double v[6];
-  // launched while the grid before it drains (launch_tube_as): nothing is read or written
-  // until that grid is complete
+  // as wait_for_grid: nothing is read or written until the grid before is complete
   asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll
-  for (int sl = 0; sl < 6; ++sl) v[sl] = __ldcg(at[sl]);
+  for (int sl = 0; sl < 6; ++sl) asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v[sl]) : "l"(at[sl]));
   // sources of the exchange: the tile's neighbours, at an open end the node itself; a tile
   // that holds the whole lattice (core = kTubeTile, no overlap) wraps onto itself
   const bool whole = core == kTubeTile;
@@ -857,7 +875,9 @@ __global__ void __launch_bounds__(kBlockX) k_macro_d2q9(const double* __restrict
   NodeXY nd;
   if (!node_xy(geo, nd)) return;
   double v[9];
-  pull9(src + 9ull * geo.plane, geo, nd.node, neighbours(geo, nd), v);
+  const Nbr b = neighbours(geo, nd);
+  wait_for_grid(src);
+  pull9(src + 9ull * geo.plane, geo, nd.node, b, v);
   D9State s;
   d9_load(v, s);
   if (s.out) {
@@ -900,6 +920,8 @@ __global__ void __launch_bounds__(kBlockX, 8) k_step_d2q9(const double* __restri
   const unsigned node = nd.node;
   const Nbr b = neighbours(geo, nd);
   double v[9];
+  if (CORR) wait_for_grid(src, q);
+  else wait_for_grid(src);
   pull9(src + 9ull * geo.plane, geo, node, b, v);
   D9State g;
   d9_load(v, g);
@@ -952,6 +974,7 @@ __global__ void __launch_bounds__(kBlockX) k_step_d2q9_eta(const double* __restr
   if (!node_xy(geo, nd)) return;
   const Nbr b = neighbours(geo, nd);
   double f[9], g[9];
+  wait_for_grid(src);
   pull9(src, geo, nd.node, b, f);
   pull9(src + 9ull * geo.plane, geo, nd.node, b, g);
   NodeMacro m;
@@ -1023,14 +1046,32 @@ bool qsep(const rlb_config& c) {
   return c.collision == RLB_MRT && c.tau_q > 0 && c.tau_q != c.tau_v;
 }
 
+// Launch of a step kernel while the grid before it in the stream drains: the kernel waits for
+// that grid itself (wait_for_grid), so that only its launch latency overlaps, 2-3 us of every
+// step: 16 x 20 x 24 FP64 8.3 -> 5.3 us per step, 32^3 16.4 -> 13.4, FP32 storage 6.3 -> 3.8,
+// 64^3 FP32 16.5 -> 14.9, 256^3 FP64 1798.8 -> 1796.5, D2Q9 4 x 800 with C_7 12.4 -> 9.3.
+template <typename... P, typename... A>
+void launch_after(dim3 grid, int block, cudaStream_t st, void (*kernel)(P...), A... args) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = grid;
+  lc.blockDim = dim3((unsigned)block);
+  lc.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = &at;
+  lc.numAttrs = 1;
+  cudaLaunchKernelEx(&lc, kernel, P(args)...);
+}
+
 // The FP64 steps for the relaxation forms of omega_v and omega_f (1: omega < 1, 2: omega >= 1).
 template <int W, bool MRT, bool QSEP, bool FLAT>
 void launch_ws(int rv, int rf, dim3 grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
                const StepConst& k, unsigned long long* bad) {
-  if (rv == 2 && rf == 2) k_step_ws<W, MRT, QSEP, FLAT, 2, 2><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
-  else if (rv == 2) k_step_ws<W, MRT, QSEP, FLAT, 2, 1><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
-  else if (rf == 2) k_step_ws<W, MRT, QSEP, FLAT, 1, 2><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
-  else k_step_ws<W, MRT, QSEP, FLAT, 1, 1><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
+  if (rv == 2 && rf == 2) launch_after(grid, 64 * W, st, k_step_ws<W, MRT, QSEP, FLAT, 2, 2>, s, d, geo, k, bad);
+  else if (rv == 2) launch_after(grid, 64 * W, st, k_step_ws<W, MRT, QSEP, FLAT, 2, 1>, s, d, geo, k, bad);
+  else if (rf == 2) launch_after(grid, 64 * W, st, k_step_ws<W, MRT, QSEP, FLAT, 1, 2>, s, d, geo, k, bad);
+  else launch_after(grid, 64 * W, st, k_step_ws<W, MRT, QSEP, FLAT, 1, 1>, s, d, geo, k, bad);
 }
 template <int W, bool FLAT>
 void launch_ws_coll(bool mrt, bool q, int rv, int rf, dim3 grid, cudaStream_t st, const double* s, double* d,
@@ -1042,16 +1083,16 @@ void launch_ws_coll(bool mrt, bool q, int rv, int rf, dim3 grid, cudaStream_t st
 template <int W, bool FLAT>
 void launch_eta(bool mrt, bool q, dim3 grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
                 const StepConst& k, unsigned long long* bad) {
-  if (!mrt) k_step_ws<W, false, false, FLAT, 0, 0, true><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
-  else if (!q) k_step_ws<W, true, false, FLAT, 0, 0, true><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
-  else k_step_ws<W, true, true, FLAT, 0, 0, true><<<grid, 64 * W, 0, st>>>(s, d, geo, k, bad);
+  if (!mrt) launch_after(grid, 64 * W, st, k_step_ws<W, false, false, FLAT, 0, 0, true>, s, d, geo, k, bad);
+  else if (!q) launch_after(grid, 64 * W, st, k_step_ws<W, true, false, FLAT, 0, 0, true>, s, d, geo, k, bad);
+  else launch_after(grid, 64 * W, st, k_step_ws<W, true, true, FLAT, 0, 0, true>, s, d, geo, k, bad);
 }
 template <bool FLAT>
 void launch_f32(bool mrt, bool q, dim3 grid, int bx, cudaStream_t st, const float* s, float* d, const Geo& geo,
                 const StepConst& k, unsigned long long* bad) {
-  if (!mrt) k_step<float, false, false, FLAT><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
-  else if (!q) k_step<float, true, false, FLAT><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
-  else k_step<float, true, true, FLAT><<<grid, bx, 0, st>>>(s, d, geo, k, bad);
+  if (!mrt) launch_after(grid, bx, st, k_step<float, false, false, FLAT>, s, d, geo, k, bad);
+  else if (!q) launch_after(grid, bx, st, k_step<float, true, false, FLAT>, s, d, geo, k, bad);
+  else launch_after(grid, bx, st, k_step<float, true, true, FLAT>, s, d, geo, k, bad);
 }
 
 // Whether nodes are numbered across rows: where blocks of b nodes per row would leave more
@@ -1067,25 +1108,17 @@ bool flat_rows(int nx, int b) {
 template <bool MRT>
 void launch_quad(int rv, int rf, dim3 grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
                  const StepConst& k, unsigned long long* bad) {
-  if (rv == 2 && rf == 2) k_step_quad<MRT, 2, 2><<<grid, 64, 0, st>>>(s, d, geo, k, bad);
-  else if (rv == 2) k_step_quad<MRT, 2, 1><<<grid, 64, 0, st>>>(s, d, geo, k, bad);
-  else if (rf == 2) k_step_quad<MRT, 1, 2><<<grid, 64, 0, st>>>(s, d, geo, k, bad);
-  else k_step_quad<MRT, 1, 1><<<grid, 64, 0, st>>>(s, d, geo, k, bad);
+  if (rv == 2 && rf == 2) launch_after(grid, 64, st, k_step_quad<MRT, 2, 2>, s, d, geo, k, bad);
+  else if (rv == 2) launch_after(grid, 64, st, k_step_quad<MRT, 2, 1>, s, d, geo, k, bad);
+  else if (rf == 2) launch_after(grid, 64, st, k_step_quad<MRT, 1, 2>, s, d, geo, k, bad);
+  else launch_after(grid, 64, st, k_step_quad<MRT, 1, 1>, s, d, geo, k, bad);
 }
 
 template <bool MRT, int RV, int RF, bool G_ONLY>
 void launch_tube_as(int grid, cudaStream_t st, const double* s, double* d, const Geo& geo, const StepConst& k,
                     int steps, int core, unsigned long long stride, unsigned long long* bad) {
-  cudaLaunchConfig_t lc{};
-  lc.gridDim = dim3((unsigned)grid);
-  lc.blockDim = dim3((G_ONLY ? 32 : 64) * kTubeWarps);
-  lc.stream = st;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;   // the kernel waits for the grid before it
-  at.val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = &at;
-  lc.numAttrs = 1;
-  cudaLaunchKernelEx(&lc, k_tube_steps<MRT, RV, RF, G_ONLY>, s, d, geo.nx, geo.bcx, k, steps, core, stride, bad);
+  launch_after(grid, (G_ONLY ? 32 : 64) * kTubeWarps, st, k_tube_steps<MRT, RV, RF, G_ONLY>, s, d, geo.nx, geo.bcx, k,
+               steps, core, stride, bad);
 }
 template <bool MRT, bool G_ONLY>
 void launch_tube(int rv, int rf, int grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
@@ -1135,19 +1168,19 @@ cudaError_t launch_step(rlb_handle* h, const void* src, void* dst, cudaStream_t 
     const double* s2 = (const double*)src;
     double* d2 = (double*)dst;
     if (h->cfg.eta_over_s > 0) {
-      if (!mrt2) k_step_d2q9_eta<false, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad);
-      else if (!q2) k_step_d2q9_eta<true, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad);
-      else k_step_d2q9_eta<true, true><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad);
+      if (!mrt2) launch_after(gr, bx, st, k_step_d2q9_eta<false, false>, s2, d2, geo, h->k, h->d_bad);
+      else if (!q2) launch_after(gr, bx, st, k_step_d2q9_eta<true, false>, s2, d2, geo, h->k, h->d_bad);
+      else launch_after(gr, bx, st, k_step_d2q9_eta<true, true>, s2, d2, geo, h->k, h->d_bad);
     } else if (h->cfg.correction != RLB_CORR_NONE) {
-      k_macro_d2q9<<<gr, bx, 0, st>>>(s2, h->d_macro, geo);
-      if (!q2) k_step_d2q9<true, false, true><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, h->d_macro);
-      else k_step_d2q9<true, true, true><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, h->d_macro);
+      launch_after(gr, bx, st, k_macro_d2q9, s2, h->d_macro, geo);
+      if (!q2) launch_after(gr, bx, st, k_step_d2q9<true, false, true>, s2, d2, geo, h->k, h->d_bad, h->d_macro);
+      else launch_after(gr, bx, st, k_step_d2q9<true, true, true>, s2, d2, geo, h->k, h->d_bad, h->d_macro);
     } else if (!mrt2) {
-      k_step_d2q9<false, false, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
+      launch_after(gr, bx, st, k_step_d2q9<false, false, false>, s2, d2, geo, h->k, h->d_bad, (const double*)nullptr);
     } else if (!q2) {
-      k_step_d2q9<true, false, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
+      launch_after(gr, bx, st, k_step_d2q9<true, false, false>, s2, d2, geo, h->k, h->d_bad, (const double*)nullptr);
     } else {
-      k_step_d2q9<true, true, false><<<gr, bx, 0, st>>>(s2, d2, geo, h->k, h->d_bad, nullptr);
+      launch_after(gr, bx, st, k_step_d2q9<true, true, false>, s2, d2, geo, h->k, h->d_bad, (const double*)nullptr);
     }
     return cudaGetLastError();
   }
