@@ -39,4 +39,12 @@ int validate_taus(double tau_f, double tau_v, double tau_e, double tau_eps, doub
 void set_handleless_error(const std::string& msg);
 // Enqueue `nsteps` fused steps of h on stream s (no validation); returns the launch status.
 cudaError_t enqueue_steps(rlb_handle* h, int nsteps, cudaStream_t s);
+// Steps that one launch of the quasi-1D kernel takes on h (1: that kernel does not serve h), and
+// the nodes a block of it stores.
+int tube_launch_steps(const rlb_handle* h, int& core);
+// One such launch: src after nsteps (at most tube_launch_steps) into dst.  g_only: src and dst
+// hold g alone and every step's g is stored, one after the other.  early: the launch may
+// overlap the drain of the grid before it in s.
+cudaError_t enqueue_tube(const rlb_handle* h, const double* src, double* dst, int nsteps, int core, bool g_only,
+                         bool early, cudaStream_t s);
 }  // namespace rlb

@@ -26,6 +26,7 @@
 #include "../../include/rlb.h"
 #include "rlb_internal.h"
 #include "rlb_io.cuh"
+#include "rlb_launch.cuh"
 #include "rlb_node.cuh"
 
 using namespace rlb;
@@ -70,19 +71,6 @@ __device__ __forceinline__ int src_minus(int i, int n, int zg) {  // source of a
 }
 __device__ __forceinline__ int src_plus(int i, int n, int zg) {   // source of a pull with c = -1
   return i < n - 1 ? i + 1 : (zg ? n - 1 : 0);
-}
-
-// A step kernel is launched while the grid before it in the stream drains (launch_after):
-// this waits until that grid is complete and its writes are visible.  The pointers pass
-// through, so that no load from them can be moved up; they are read with coherent loads,
-// since the grid before writes while this kernel is already resident.
-template <typename T>
-__device__ __forceinline__ void wait_for_grid(const T* __restrict__& p) {
-  asm volatile("griddepcontrol.wait;" : "+l"(p)::"memory");
-}
-template <typename T>
-__device__ __forceinline__ void wait_for_grid(const T* __restrict__& p, const T* __restrict__& q) {
-  asm volatile("griddepcontrol.wait;" : "+l"(p), "+l"(q)::"memory");
 }
 
 // Population load.  FP64 populations are streamed past L1 (each value is
@@ -706,13 +694,13 @@ __global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ 
 // (issue slots 66 % busy on the SMs that have a block).  1600 nodes: 6.17 -> 2.37 us per step,
 // 6400: 6.18 -> 3.31, 38912: 16.5 -> 13.4.  Tried: 16- and 64-node tiles (2.58 and 3.7 us at
 // 1600 nodes), the output rounding on the integer pipe (2.84 against 2.59 at 8 steps).
-//   G_ONLY: g alone (it does not depend on f), every step's g stored at dst + s * stride (the
-//   adjoint's recompute).
+//   G_ONLY: g alone (it does not depend on f), src and dst hold g only, and every step's g
+//   is stored, step s at dst + 19 nx s (the adjoint's recompute).
 constexpr int kTubeTile = 8 * kTubeWarps;
 template <bool MRT, int RV, int RF, bool G_ONLY>
 __global__ void __launch_bounds__((G_ONLY ? 32 : 64) * kTubeWarps)
     k_tube_steps(const double* __restrict__ src, double* __restrict__ dst, int nx, int bcx, StepConst k, int steps,
-                 int core, unsigned long long stride, unsigned long long* __restrict__ bad) {
+                 int core, unsigned long long* __restrict__ bad) {
   __shared__ QuadU su[kTubeWarps];
   __shared__ double ex[2][G_ONLY ? 1 : 2][2][6][kTubeTile];   // [parity][role][lane 0 / 2][slot][node]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m = lane >> 2, j = lane & 3;
@@ -726,7 +714,7 @@ __global__ void __launch_bounds__((G_ONLY ? 32 : 64) * kTubeWarps)
   if (bcx) x = min(max(xg, 0), nx - 1);                         // past an open end: idle copies
   else x = xg < 0 ? (xg % nx + nx) % nx : xg % nx;
   const unsigned long long n = (unsigned long long)nx;
-  const double* in = src + (is_g ? 19ull * n : 0ull);
+  const double* in = src + (is_g && !G_ONLY ? 19ull * n : 0ull);
   const double* at[6];
 #pragma unroll
   for (int sl = 0; sl < 6; ++sl) {
@@ -751,7 +739,7 @@ __global__ void __launch_bounds__((G_ONLY ? 32 : 64) * kTubeWarps)
     if (own && b && j == 0) atomicMin(bad, (unsigned long long)x);
     if (G_ONLY || s == steps - 1) {
       if (own) {
-        double* out = dst + (G_ONLY ? (unsigned long long)s * stride : (is_g ? 19ull * n : 0ull)) + (unsigned)x;
+        double* out = dst + (G_ONLY ? (unsigned)s * 19ull * n : (is_g ? 19ull * n : 0ull)) + (unsigned)x;
         out[(unsigned long long)quad_link(j, 0) * n] = v[0];
         if (j < 3) {
 #pragma unroll
@@ -1046,32 +1034,14 @@ bool qsep(const rlb_config& c) {
   return c.collision == RLB_MRT && c.tau_q > 0 && c.tau_q != c.tau_v;
 }
 
-// Launch of a step kernel while the grid before it in the stream drains: the kernel waits for
-// that grid itself (wait_for_grid), so that only its launch latency overlaps, 2-3 us of every
-// step: 16 x 20 x 24 FP64 8.3 -> 5.3 us per step, 32^3 16.4 -> 13.4, FP32 storage 6.3 -> 3.8,
-// 64^3 FP32 16.5 -> 14.9, 256^3 FP64 1798.8 -> 1796.5, D2Q9 4 x 800 with C_7 12.4 -> 9.3.
-template <typename... P, typename... A>
-void launch_after(dim3 grid, int block, cudaStream_t st, void (*kernel)(P...), A... args) {
-  cudaLaunchConfig_t lc{};
-  lc.gridDim = grid;
-  lc.blockDim = dim3((unsigned)block);
-  lc.stream = st;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = &at;
-  lc.numAttrs = 1;
-  cudaLaunchKernelEx(&lc, kernel, P(args)...);
-}
-
 // The FP64 steps for the relaxation forms of omega_v and omega_f (1: omega < 1, 2: omega >= 1).
 template <int W, bool MRT, bool QSEP, bool FLAT>
 void launch_ws(int rv, int rf, dim3 grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
                const StepConst& k, unsigned long long* bad) {
-  if (rv == 2 && rf == 2) launch_after(grid, 64 * W, st, k_step_ws<W, MRT, QSEP, FLAT, 2, 2>, s, d, geo, k, bad);
-  else if (rv == 2) launch_after(grid, 64 * W, st, k_step_ws<W, MRT, QSEP, FLAT, 2, 1>, s, d, geo, k, bad);
-  else if (rf == 2) launch_after(grid, 64 * W, st, k_step_ws<W, MRT, QSEP, FLAT, 1, 2>, s, d, geo, k, bad);
-  else launch_after(grid, 64 * W, st, k_step_ws<W, MRT, QSEP, FLAT, 1, 1>, s, d, geo, k, bad);
+  if (rv == 2 && rf == 2) launch_after(grid, 64 * W, st, true, k_step_ws<W, MRT, QSEP, FLAT, 2, 2>, s, d, geo, k, bad);
+  else if (rv == 2) launch_after(grid, 64 * W, st, true, k_step_ws<W, MRT, QSEP, FLAT, 2, 1>, s, d, geo, k, bad);
+  else if (rf == 2) launch_after(grid, 64 * W, st, true, k_step_ws<W, MRT, QSEP, FLAT, 1, 2>, s, d, geo, k, bad);
+  else launch_after(grid, 64 * W, st, true, k_step_ws<W, MRT, QSEP, FLAT, 1, 1>, s, d, geo, k, bad);
 }
 template <int W, bool FLAT>
 void launch_ws_coll(bool mrt, bool q, int rv, int rf, dim3 grid, cudaStream_t st, const double* s, double* d,
@@ -1083,16 +1053,16 @@ void launch_ws_coll(bool mrt, bool q, int rv, int rf, dim3 grid, cudaStream_t st
 template <int W, bool FLAT>
 void launch_eta(bool mrt, bool q, dim3 grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
                 const StepConst& k, unsigned long long* bad) {
-  if (!mrt) launch_after(grid, 64 * W, st, k_step_ws<W, false, false, FLAT, 0, 0, true>, s, d, geo, k, bad);
-  else if (!q) launch_after(grid, 64 * W, st, k_step_ws<W, true, false, FLAT, 0, 0, true>, s, d, geo, k, bad);
-  else launch_after(grid, 64 * W, st, k_step_ws<W, true, true, FLAT, 0, 0, true>, s, d, geo, k, bad);
+  if (!mrt) launch_after(grid, 64 * W, st, true, k_step_ws<W, false, false, FLAT, 0, 0, true>, s, d, geo, k, bad);
+  else if (!q) launch_after(grid, 64 * W, st, true, k_step_ws<W, true, false, FLAT, 0, 0, true>, s, d, geo, k, bad);
+  else launch_after(grid, 64 * W, st, true, k_step_ws<W, true, true, FLAT, 0, 0, true>, s, d, geo, k, bad);
 }
 template <bool FLAT>
 void launch_f32(bool mrt, bool q, dim3 grid, int bx, cudaStream_t st, const float* s, float* d, const Geo& geo,
                 const StepConst& k, unsigned long long* bad) {
-  if (!mrt) launch_after(grid, bx, st, k_step<float, false, false, FLAT>, s, d, geo, k, bad);
-  else if (!q) launch_after(grid, bx, st, k_step<float, true, false, FLAT>, s, d, geo, k, bad);
-  else launch_after(grid, bx, st, k_step<float, true, true, FLAT>, s, d, geo, k, bad);
+  if (!mrt) launch_after(grid, bx, st, true, k_step<float, false, false, FLAT>, s, d, geo, k, bad);
+  else if (!q) launch_after(grid, bx, st, true, k_step<float, true, false, FLAT>, s, d, geo, k, bad);
+  else launch_after(grid, bx, st, true, k_step<float, true, true, FLAT>, s, d, geo, k, bad);
 }
 
 // Whether nodes are numbered across rows: where blocks of b nodes per row would leave more
@@ -1108,53 +1078,26 @@ bool flat_rows(int nx, int b) {
 template <bool MRT>
 void launch_quad(int rv, int rf, dim3 grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
                  const StepConst& k, unsigned long long* bad) {
-  if (rv == 2 && rf == 2) launch_after(grid, 64, st, k_step_quad<MRT, 2, 2>, s, d, geo, k, bad);
-  else if (rv == 2) launch_after(grid, 64, st, k_step_quad<MRT, 2, 1>, s, d, geo, k, bad);
-  else if (rf == 2) launch_after(grid, 64, st, k_step_quad<MRT, 1, 2>, s, d, geo, k, bad);
-  else launch_after(grid, 64, st, k_step_quad<MRT, 1, 1>, s, d, geo, k, bad);
+  if (rv == 2 && rf == 2) launch_after(grid, 64, st, true, k_step_quad<MRT, 2, 2>, s, d, geo, k, bad);
+  else if (rv == 2) launch_after(grid, 64, st, true, k_step_quad<MRT, 2, 1>, s, d, geo, k, bad);
+  else if (rf == 2) launch_after(grid, 64, st, true, k_step_quad<MRT, 1, 2>, s, d, geo, k, bad);
+  else launch_after(grid, 64, st, true, k_step_quad<MRT, 1, 1>, s, d, geo, k, bad);
 }
 
 template <bool MRT, int RV, int RF, bool G_ONLY>
-void launch_tube_as(int grid, cudaStream_t st, const double* s, double* d, const Geo& geo, const StepConst& k,
-                    int steps, int core, unsigned long long stride, unsigned long long* bad) {
-  launch_after(grid, (G_ONLY ? 32 : 64) * kTubeWarps, st, k_tube_steps<MRT, RV, RF, G_ONLY>, s, d, geo.nx, geo.bcx, k,
-               steps, core, stride, bad);
+void launch_tube_as(int grid, cudaStream_t st, bool early, const double* s, double* d, const Geo& geo,
+                    const StepConst& k, int steps, int core, unsigned long long* bad) {
+  launch_after(grid, (G_ONLY ? 32 : 64) * kTubeWarps, st, early, k_tube_steps<MRT, RV, RF, G_ONLY>, s, d, geo.nx,
+               geo.bcx, k, steps, core, bad);
 }
 template <bool MRT, bool G_ONLY>
-void launch_tube(int rv, int rf, int grid, cudaStream_t st, const double* s, double* d, const Geo& geo,
-                 const StepConst& k, int steps, int core, unsigned long long stride, unsigned long long* bad) {
+void launch_tube(int rv, int rf, int grid, cudaStream_t st, bool early, const double* s, double* d, const Geo& geo,
+                 const StepConst& k, int steps, int core, unsigned long long* bad) {
   if (G_ONLY) rf = rv;   // f is not advanced
-  if (rv == 2 && rf == 2) launch_tube_as<MRT, 2, 2, G_ONLY>(grid, st, s, d, geo, k, steps, core, stride, bad);
-  else if (rv == 2) launch_tube_as<MRT, 2, G_ONLY ? 2 : 1, G_ONLY>(grid, st, s, d, geo, k, steps, core, stride, bad);
-  else if (rf == 2) launch_tube_as<MRT, 1, G_ONLY ? 1 : 2, G_ONLY>(grid, st, s, d, geo, k, steps, core, stride, bad);
-  else launch_tube_as<MRT, 1, 1, G_ONLY>(grid, st, s, d, geo, k, steps, core, stride, bad);
-}
-
-// Whether several steps go into one launch (k_tube_steps), and how many.
-int tube_launch_steps(const rlb_handle* h, int& core) {
-  const rlb_config& c = h->cfg;
-  if (h->Q != 19 || h->esize != 8 || c.ny != 1 || c.nz != 1 || h->nodes > kSmallNodes || c.eta_over_s > 0 || qsep(c))
-    return 1;
-  if (c.nx <= kTubeTile) {   // one block holds the lattice
-    core = kTubeTile;
-    return INT_MAX;
-  }
-  // H steps per launch cost 1.4 us / H for the launch and, per step, the chain (2.24 us) times
-  // what w blocks per SM slow it down (measured: 1 block 1.0, 2 1.4, 3 1.8, 6 3.6, 9 5.7);
-  // more steps mean a smaller core and so more blocks
-  float best = 1e30f;
-  int H = 2;
-  for (int t = 2; t <= 12; ++t) {
-    const int c = kTubeTile - 2 * (t - 1);
-    const int w = (((int)h->nodes + c - 1) / c + 151) / 152;
-    const float cost = 1.4f / t + 2.24f * std::max(1.0f, 0.1f + 0.62f * w);
-    if (cost < best) {
-      best = cost;
-      H = t;
-    }
-  }
-  core = kTubeTile - 2 * (H - 1);
-  return H;
+  if (rv == 2 && rf == 2) launch_tube_as<MRT, 2, 2, G_ONLY>(grid, st, early, s, d, geo, k, steps, core, bad);
+  else if (rv == 2) launch_tube_as<MRT, 2, G_ONLY ? 2 : 1, G_ONLY>(grid, st, early, s, d, geo, k, steps, core, bad);
+  else if (rf == 2) launch_tube_as<MRT, 1, G_ONLY ? 1 : 2, G_ONLY>(grid, st, early, s, d, geo, k, steps, core, bad);
+  else launch_tube_as<MRT, 1, 1, G_ONLY>(grid, st, early, s, d, geo, k, steps, core, bad);
 }
 
 template <typename S>
@@ -1168,19 +1111,19 @@ cudaError_t launch_step(rlb_handle* h, const void* src, void* dst, cudaStream_t 
     const double* s2 = (const double*)src;
     double* d2 = (double*)dst;
     if (h->cfg.eta_over_s > 0) {
-      if (!mrt2) launch_after(gr, bx, st, k_step_d2q9_eta<false, false>, s2, d2, geo, h->k, h->d_bad);
-      else if (!q2) launch_after(gr, bx, st, k_step_d2q9_eta<true, false>, s2, d2, geo, h->k, h->d_bad);
-      else launch_after(gr, bx, st, k_step_d2q9_eta<true, true>, s2, d2, geo, h->k, h->d_bad);
+      if (!mrt2) launch_after(gr, bx, st, true, k_step_d2q9_eta<false, false>, s2, d2, geo, h->k, h->d_bad);
+      else if (!q2) launch_after(gr, bx, st, true, k_step_d2q9_eta<true, false>, s2, d2, geo, h->k, h->d_bad);
+      else launch_after(gr, bx, st, true, k_step_d2q9_eta<true, true>, s2, d2, geo, h->k, h->d_bad);
     } else if (h->cfg.correction != RLB_CORR_NONE) {
-      launch_after(gr, bx, st, k_macro_d2q9, s2, h->d_macro, geo);
-      if (!q2) launch_after(gr, bx, st, k_step_d2q9<true, false, true>, s2, d2, geo, h->k, h->d_bad, h->d_macro);
-      else launch_after(gr, bx, st, k_step_d2q9<true, true, true>, s2, d2, geo, h->k, h->d_bad, h->d_macro);
+      launch_after(gr, bx, st, true, k_macro_d2q9, s2, h->d_macro, geo);
+      if (!q2) launch_after(gr, bx, st, true, k_step_d2q9<true, false, true>, s2, d2, geo, h->k, h->d_bad, h->d_macro);
+      else launch_after(gr, bx, st, true, k_step_d2q9<true, true, true>, s2, d2, geo, h->k, h->d_bad, h->d_macro);
     } else if (!mrt2) {
-      launch_after(gr, bx, st, k_step_d2q9<false, false, false>, s2, d2, geo, h->k, h->d_bad, (const double*)nullptr);
+      launch_after(gr, bx, st, true, k_step_d2q9<false, false, false>, s2, d2, geo, h->k, h->d_bad, (const double*)nullptr);
     } else if (!q2) {
-      launch_after(gr, bx, st, k_step_d2q9<true, false, false>, s2, d2, geo, h->k, h->d_bad, (const double*)nullptr);
+      launch_after(gr, bx, st, true, k_step_d2q9<true, false, false>, s2, d2, geo, h->k, h->d_bad, (const double*)nullptr);
     } else {
-      launch_after(gr, bx, st, k_step_d2q9<true, true, false>, s2, d2, geo, h->k, h->d_bad, (const double*)nullptr);
+      launch_after(gr, bx, st, true, k_step_d2q9<true, true, false>, s2, d2, geo, h->k, h->d_bad, (const double*)nullptr);
     }
     return cudaGetLastError();
   }
@@ -1258,25 +1201,61 @@ int ensure_stage(rlb_handle* h) {
 namespace rlb {
 void set_handleless_error(const std::string& msg) { g_create_error = msg; }
 
+int tube_launch_steps(const rlb_handle* h, int& core) {
+  const rlb_config& c = h->cfg;
+  if (h->Q != 19 || h->esize != 8 || c.ny != 1 || c.nz != 1 || h->nodes > kSmallNodes || c.eta_over_s > 0 || qsep(c))
+    return 1;
+  if (c.nx <= kTubeTile) {   // one block holds the lattice
+    core = kTubeTile;
+    return INT_MAX;
+  }
+  // H steps per launch cost 1.4 us / H for the launch and, per step, the chain (2.24 us) times
+  // what w blocks per SM slow it down (measured: 1 block 1.0, 2 1.4, 3 1.8, 6 3.6, 9 5.7);
+  // more steps mean a smaller core and so more blocks
+  float best = 1e30f;
+  int H = 2;
+  for (int t = 2; t <= 12; ++t) {
+    const int c = kTubeTile - 2 * (t - 1);
+    const int w = (((int)h->nodes + c - 1) / c + 151) / 152;
+    const float cost = 1.4f / t + 2.24f * std::max(1.0f, 0.1f + 0.62f * w);
+    if (cost < best) {
+      best = cost;
+      H = t;
+    }
+  }
+  core = kTubeTile - 2 * (H - 1);
+  return H;
+}
+
+cudaError_t enqueue_tube(const rlb_handle* h, const double* src, double* dst, int nsteps, int core, bool g_only,
+                         bool early, cudaStream_t st) {
+  const Geo geo = make_geo(h);
+  const int grid = (geo.nx + core - 1) / core, rv = h->k.r_v, rf = h->k.r_f;
+  const bool mrt = h->cfg.collision == RLB_MRT;
+  if (g_only) {
+    if (mrt) launch_tube<true, true>(rv, rf, grid, st, early, src, dst, geo, h->k, nsteps, core, h->d_bad);
+    else launch_tube<false, true>(rv, rf, grid, st, early, src, dst, geo, h->k, nsteps, core, h->d_bad);
+  } else {
+    if (mrt) launch_tube<true, false>(rv, rf, grid, st, early, src, dst, geo, h->k, nsteps, core, h->d_bad);
+    else launch_tube<false, false>(rv, rf, grid, st, early, src, dst, geo, h->k, nsteps, core, h->d_bad);
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t enqueue_steps(rlb_handle* h, int nsteps, cudaStream_t st) {
   int core = 0;
   const int most = tube_launch_steps(h, core);
-  for (int s = 0; s < nsteps && most > 1 && nsteps > 1;) {
-    const int n = std::min(most, nsteps - s);
-    const Geo geo = make_geo(h);
-    const int grid = (geo.nx + core - 1) / core;
-    const double* src = (const double*)h->lat[h->cur];
-    double* dst = (double*)h->lat[1 - h->cur];
-    if (h->cfg.collision == RLB_MRT)
-      launch_tube<true, false>(h->k.r_v, h->k.r_f, grid, st, src, dst, geo, h->k, n, core, 0, h->d_bad);
-    else
-      launch_tube<false, false>(h->k.r_v, h->k.r_f, grid, st, src, dst, geo, h->k, n, core, 0, h->d_bad);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    h->cur = 1 - h->cur;
-    h->steps += n;
-    s += n;
-    if (s == nsteps) return cudaSuccess;
+  if (most > 1 && nsteps > 1) {
+    for (int s = 0; s < nsteps;) {
+      const int n = std::min(most, nsteps - s);
+      const cudaError_t e = enqueue_tube(h, (const double*)h->lat[h->cur], (double*)h->lat[1 - h->cur], n, core, false,
+                                         true, st);
+      if (e != cudaSuccess) return e;
+      h->cur = 1 - h->cur;
+      h->steps += n;
+      s += n;
+    }
+    return cudaSuccess;
   }
   for (int s = 0; s < nsteps; ++s) {
     const void* src = h->lat[h->cur];
