@@ -9,7 +9,8 @@
  * by Eq. 5, BGK g by Eq. 6 or MRT g by Eqs. 30-35).  rlb_batch_run advances all
  * tubes by nsteps in ONE persistent kernel launch replayed from a CUDA graph:
  * each CTA takes whole tubes from a longest-first work list and runs all the steps
- * of a tube with CTA-local barriers (tubes never exchange data).
+ * of a tube with CTA-local barriers (tubes never exchange data).  In a batch with fewer
+ * tubes than the GPU holds CTAs, a cluster of 2 to 8 CTAs takes each tube.
  *
  * Node numbering: tube t occupies the global node range [offset_t, offset_t + L_t)
  * with offset_t = L_0 + ... + L_{t-1}; field arrays of the batch are these
@@ -74,8 +75,8 @@ int rlb_batch_autotune(rlb_batch* b, int trial_steps, int* chosen);
  * rlb_batch_autotune chose earlier, say): threads per CTA, a multiple of 32 up to the
  * kernel's launch bound (320 for FP32 storage, 256 for FP64), and CTAs per SM, 1 up to
  * the occupancy limit at that block size (0 = that limit).  RLB_EINVAL (state
- * unchanged) for any other value.  Results do not depend on the shape: each tube is
- * advanced by one CTA and every node's arithmetic is the same. */
+ * unchanged) for any other value.  Results do not depend on the shape: every node's
+ * arithmetic is the same, whichever thread of a CTA or cluster takes it. */
 int rlb_batch_set_shape(rlb_batch* b, int threads, int ctas_per_sm);
 
 /* Advance every tube by nsteps (>= 0) in one persistent launch from a CUDA graph

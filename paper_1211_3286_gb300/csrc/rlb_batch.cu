@@ -6,8 +6,9 @@
 // Execution: one persistent kernel.  Each CTA repeatedly takes the next tube
 // from a longest-first work list (an atomic counter; longest-processing-time
 // order keeps the tail short) and advances that tube by all nsteps with
-// CTA-local barriers.  Tubes never exchange data, so no grid-wide barrier exists
-// and no CTA waits on another.  Steps run in place in pairs on one lattice (the AA
+// CTA-local barriers; in a batch too small to fill the GPU a cluster of CTAs takes a
+// tube, with cluster barriers.  Tubes never exchange data, so no grid-wide barrier exists
+// and no CTA (or cluster) waits on another.  Steps run in place in pairs on one lattice (the AA
 // scheme, tube_step), which halves a tube's working set in L2 against reading one
 // lattice and writing the other; an odd last step goes into the other lattice.
 // Lattice accesses use ld.global.cg / st.global.cg (coherent at L2 for the CTA's
@@ -71,6 +72,17 @@ __device__ __forceinline__ bool tube_collide(S (&f)[19], S (&g)[19], const StepC
   else return node_collide_f32s<MRT, false>(f, g, k);
 }
 
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_ctas() {
+  unsigned n;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+  return n;
+}
+
 // One step of a tube.  mode 0: two lattices, node x pulls from src (x - c_x, clamped
 // at the zero-gradient ends) and stores at x in dst.  Modes 1 and 2 are the in-place
 // pair of the AA scheme on one lattice (src == dst), which halves a tube's working set:
@@ -86,11 +98,13 @@ __device__ __forceinline__ bool tube_collide(S (&f)[19], S (&g)[19], const StepC
 //     and refreshes the edge copies.
 // One collide call site serves the three modes; the mode picks whole load and store
 // blocks, and only the two end nodes take the clamping / edge-copy path.
-template <typename S, bool MRT>
+// The tube's nodes go round the CTA's threads (CL: the cluster's).
+template <typename S, bool MRT, bool CL>
 __device__ __forceinline__ void tube_step(int mode, const S* src, S* dst, const TubeInfo& ti,
                                           unsigned long long nodes, const StepConst& k, S (&edge)[2][2][5],
                                           unsigned long long* bad) {
-  for (int x = threadIdx.x; x < ti.L; x += blockDim.x) {
+  for (int x = CL ? cluster_rank() * blockDim.x + threadIdx.x : threadIdx.x; x < ti.L;
+       x += CL ? cluster_ctas() * blockDim.x : blockDim.x) {
     const unsigned long long x0 = ti.off + (unsigned long long)x;
     const bool end = x == 0 || x == ti.L - 1;
     S f[19], g[19];
@@ -169,6 +183,16 @@ __device__ __forceinline__ void tube_step(int mode, const S* src, S* dst, const 
   }
 }
 
+template <bool CL>
+__device__ __forceinline__ void step_barrier() {
+  if (CL) {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+
 // Persistent tube kernel: each CTA takes the next tube of the longest-first list and
 // advances it by nsteps: in place pairs of steps on latA (AA scheme), and for an odd
 // nsteps one last two-lattice step into latB.
@@ -183,18 +207,30 @@ __device__ __forceinline__ void tube_step(int mode, const S* src, S* dst, const 
 #ifndef RLB_TUBES_F32_BLOCKS
 #define RLB_TUBES_F32_BLOCKS 2
 #endif
-template <typename S, bool MRT>
+// CL: a cluster of CTAs takes a tube together (batches with fewer tubes than the GPU holds
+// CTAs): the tube's nodes go round the cluster's threads, every step ends in a cluster
+// barrier instead of a CTA barrier, and the tubes are dealt out in order.  A node stays with
+// its thread, so the edge copies stay in the CTAs that own the end nodes.  Tubes of
+// 200-3200 nodes, 200 steps: 16 in FP64 17.3 -> 2.8 ms, 100 20.6 -> 12.8; FP32 storage, tuned: 16
+// 5.8 -> 1.4, 100 6.6 -> 3.0, 304 7.9 -> 6.8.
+template <typename S, bool MRT, bool CL>
 __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : RLB_TUBES_F32_THREADS, sizeof(S) == 8 ? 1 : RLB_TUBES_F32_BLOCKS) k_tubes(const TubeInfo* __restrict__ order, int ntubes, const StepConst* __restrict__ consts,
                         S* latA, S* latB, unsigned long long nodes, int nsteps, unsigned* __restrict__ counter,
                         unsigned long long* __restrict__ bad) {
   __shared__ int s_t;
   __shared__ S edge[2][2][5];   // [left/right end][f/g][link with c_x = +1 / its opposite]
   __shared__ StepConst s_k;     // the tube's constants, read from shared memory where used
-  for (;;) {
-    if (threadIdx.x == 0) s_t = (int)atomicAdd(counter, 1u);
-    __syncthreads();
-    const int t = s_t;
-    __syncthreads();
+  for (int turn = 0;; ++turn) {
+    int t;
+    if (CL) {
+      t = (int)((blockIdx.x + (unsigned)turn * gridDim.x) / cluster_ctas());
+      __syncthreads();   // the last tube's constants and edges are no longer read
+    } else {
+      if (threadIdx.x == 0) s_t = (int)atomicAdd(counter, 1u);
+      __syncthreads();
+      t = s_t;
+      __syncthreads();
+    }
     if (t >= ntubes) return;
     const TubeInfo ti = order[t];
     if (threadIdx.x == 0) s_k = consts[ti.id];
@@ -206,12 +242,12 @@ __global__ void __launch_bounds__(sizeof(S) == 8 ? 256 : RLB_TUBES_F32_THREADS, 
       const unsigned long long x0 = ti.off + (unsigned long long)(side == 0 ? 0 : ti.L - 1);
       edge[side][d][j] = ld_cg(latA + (19ull * d + a) * nodes + x0);
     }
-    __syncthreads();
+    step_barrier<CL>();   // a cluster: no CTA writes before every CTA has its edge copies
     for (int s = 0; s < nsteps; ++s) {
       // pairs in place (modes 1, 2); an odd last step into the other lattice (mode 0)
       const int mode = (nsteps & 1) && s == nsteps - 1 ? 0 : 1 + (s & 1);
-      tube_step<S, MRT>(mode, latA, mode == 0 ? latB : latA, ti, nodes, k, edge, bad);
-      __syncthreads();
+      tube_step<S, MRT, CL>(mode, latA, mode == 0 ? latB : latA, ti, nodes, k, edge, bad);
+      step_barrier<CL>();
     }
   }
 }
@@ -235,8 +271,9 @@ struct rlb_batch {
   unsigned* d_counter = nullptr;
   unsigned long long* d_bad = nullptr;
   double* d_stage = nullptr;
-  int threads = 128, ctas_per_sm = 0;         // 0 = maximum occupancy
+  int threads = 0, ctas_per_sm = 0;           // threads 0: chosen by tube_launch; CTAs 0: maximum occupancy
   int sms = 0;
+  int longest = 0;                            // nodes of the longest tube
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   int g_steps = -1, g_cur = -1, g_threads = -1, g_ctas = -1;
@@ -259,46 +296,93 @@ int bfail(rlb_batch* b, int code, const std::string& m) {
     if (e_ != cudaSuccess) return bfail(b, RLB_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-template <typename S, bool MRT>
-void* kernel_ptr() { return (void*)k_tubes<S, MRT>; }
+template <typename S, bool CL>
+void* kernel_ptr(bool mrt) { return mrt ? (void*)k_tubes<S, true, CL> : (void*)k_tubes<S, false, CL>; }
 
-void* tube_kernel(const rlb_batch* b) {
-  if (b->esize == 8) return b->collision == RLB_MRT ? kernel_ptr<double, true>() : kernel_ptr<double, false>();
-  return b->collision == RLB_MRT ? kernel_ptr<float, true>() : kernel_ptr<float, false>();
+void* tube_kernel(const rlb_batch* b, bool cl = false) {
+  const bool mrt = b->collision == RLB_MRT;
+  if (b->esize == 8) return cl ? kernel_ptr<double, true>(mrt) : kernel_ptr<double, false>(mrt);
+  return cl ? kernel_ptr<float, true>(mrt) : kernel_ptr<float, false>(mrt);
 }
 
-int grid_size(const rlb_batch* b, int threads, int ctas_per_sm) {
+int max_ctas(const rlb_batch* b, int threads, int ctas_per_sm) {
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, tube_kernel(b), threads, 0) != cudaSuccess) {
     cudaGetLastError();
     occ = 0;
   }
   if (occ < 1) occ = 1;
-  int per = ctas_per_sm > 0 ? std::min(ctas_per_sm, occ) : occ;
-  int grid = per * b->sms;
-  return std::max(1, std::min(grid, b->ntubes));
+  return (ctas_per_sm > 0 ? std::min(ctas_per_sm, occ) : occ) * b->sms;
 }
 
-cudaError_t launch_tubes(rlb_batch* b, cudaStream_t s, void* A, void* B, int nsteps, int threads, int grid) {
+// Launch of the tube kernel: CTAs, CTAs per cluster (1: no clusters) and threads per CTA.
+struct TubeLaunch {
+  int grid, cluster, threads;
+};
+// A batch that leaves CTA slots empty gives each tube a cluster: as many CTAs as there are
+// slots per tube, in powers of two up to 8, and no more threads than the longest tube has nodes.
+TubeLaunch tube_launch(const rlb_batch* b, int threads, int ctas_per_sm) {
+  if (threads == 0) {
+    // No shape set: 128 threads where that leaves room for clusters of at least 2 (FP32
+    // storage) or 4 (FP64) CTAs per tube; else the widest CTAs (431 tubes FP32 17.0 -> 11.3 ms per
+    // 200 steps, 1024 26.0 -> 19.8; 160 tubes FP64 22.5 -> 14.2), but 128 again for more than
+    // 600 FP64 tubes (1024: 55.7 against 57.4 ms).
+    const bool f32 = b->esize == 4;
+    const bool narrow = (long long)b->ntubes * (f32 ? 2 : 4) <= max_ctas(b, 128, 0) || (!f32 && b->ntubes > 600);
+    threads = narrow ? 128 : (f32 ? RLB_TUBES_F32_THREADS : 256);
+    ctas_per_sm = 0;
+  }
+  TubeLaunch l{0, 1, threads};
+  const int most = max_ctas(b, threads, ctas_per_sm);
+  l.grid = std::max(1, std::min(most, b->ntubes));
+  while (l.cluster < 8 && (long long)b->ntubes * l.cluster * 2 <= most && l.cluster * threads < b->longest) l.cluster *= 2;
+  if (l.cluster > 1) {
+    l.grid = b->ntubes * l.cluster;
+    cudaLaunchConfig_t lc{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)l.cluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    lc.gridDim = dim3((unsigned)l.grid);
+    lc.blockDim = dim3((unsigned)threads);
+    lc.attrs = &at;
+    lc.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, tube_kernel(b, true), &lc) != cudaSuccess || n < 1) {
+      cudaGetLastError();
+      l.cluster = 1;
+      l.grid = std::max(1, std::min(most, b->ntubes));
+    }
+  }
+  return l;
+}
+
+template <typename S, bool MRT>
+cudaError_t launch_tubes_as(rlb_batch* b, cudaStream_t s, void* A, void* B, int nsteps, const TubeLaunch& l) {
+  cudaLaunchConfig_t lc{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)l.cluster;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  lc.gridDim = dim3((unsigned)l.grid);
+  lc.blockDim = dim3((unsigned)l.threads);
+  lc.stream = s;
+  lc.attrs = &at;
+  lc.numAttrs = l.cluster > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&lc, l.cluster > 1 ? k_tubes<S, MRT, true> : k_tubes<S, MRT, false>,
+                            (const TubeInfo*)b->d_order, b->ntubes, (const StepConst*)b->d_consts, (S*)A, (S*)B,
+                            (unsigned long long)b->nodes, nsteps, b->d_counter, b->d_bad);
+}
+
+cudaError_t launch_tubes(rlb_batch* b, cudaStream_t s, void* A, void* B, int nsteps, const TubeLaunch& l) {
   cudaError_t e = cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
-  const unsigned long long N = b->nodes;
-  if (b->esize == 8) {
-    if (b->collision == RLB_MRT)
-      k_tubes<double, true><<<grid, threads, 0, s>>>(b->d_order, b->ntubes, b->d_consts, (double*)A, (double*)B, N,
-                                                     nsteps, b->d_counter, b->d_bad);
-    else
-      k_tubes<double, false><<<grid, threads, 0, s>>>(b->d_order, b->ntubes, b->d_consts, (double*)A, (double*)B, N,
-                                                      nsteps, b->d_counter, b->d_bad);
-  } else {
-    if (b->collision == RLB_MRT)
-      k_tubes<float, true><<<grid, threads, 0, s>>>(b->d_order, b->ntubes, b->d_consts, (float*)A, (float*)B, N,
-                                                    nsteps, b->d_counter, b->d_bad);
-    else
-      k_tubes<float, false><<<grid, threads, 0, s>>>(b->d_order, b->ntubes, b->d_consts, (float*)A, (float*)B, N,
-                                                     nsteps, b->d_counter, b->d_bad);
-  }
-  return cudaGetLastError();
+  const bool mrt = b->collision == RLB_MRT;
+  if (b->esize == 8)
+    e = mrt ? launch_tubes_as<double, true>(b, s, A, B, nsteps, l) : launch_tubes_as<double, false>(b, s, A, B, nsteps, l);
+  else
+    e = mrt ? launch_tubes_as<float, true>(b, s, A, B, nsteps, l) : launch_tubes_as<float, false>(b, s, A, B, nsteps, l);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 int ensure_stage(rlb_batch* b) {
@@ -365,6 +449,7 @@ extern "C" int rlb_batch_create(const rlb_batch_desc* d, rlb_batch** out) {
   b->nodes = total;
   b->stream = (cudaStream_t)d->stream;
   b->lengths.assign(d->lengths, d->lengths + d->ntubes);
+  b->longest = *std::max_element(b->lengths.begin(), b->lengths.end());
   b->offsets.resize(d->ntubes + 1);
   b->offsets[0] = 0;
   for (int t = 0; t < d->ntubes; ++t) b->offsets[t + 1] = b->offsets[t] + d->lengths[t];
@@ -501,7 +586,7 @@ extern "C" int rlb_batch_autotune(rlb_batch* b, int trial_steps, int* chosen) {
       if (c > occ) continue;
       cudaError_t e = cudaMemcpyAsync(tr[0], b->lat[b->cur], bytes, cudaMemcpyDeviceToDevice, b->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
-      if (e == cudaSuccess) e = launch_tubes(b, b->stream, tr[0], tr[1], trial_steps, th, grid_size(b, th, c));
+      if (e == cudaSuccess) e = launch_tubes(b, b->stream, tr[0], tr[1], trial_steps, tube_launch(b, th, c));
       if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       if (e != cudaSuccess) {
@@ -564,9 +649,9 @@ extern "C" int rlb_batch_run(rlb_batch* b, int nsteps) {
   if (!b->exec || b->g_steps != nsteps || b->g_cur != b->cur || b->g_threads != b->threads ||
       b->g_ctas != b->ctas_per_sm) {
     drop_graph(b);
-    const int grid = grid_size(b, b->threads, b->ctas_per_sm);
+    const TubeLaunch tl = tube_launch(b, b->threads, b->ctas_per_sm);
     BCUDA(b, cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-    cudaError_t le = launch_tubes(b, b->cap, b->lat[b->cur], b->lat[1 - b->cur], nsteps, b->threads, grid);
+    cudaError_t le = launch_tubes(b, b->cap, b->lat[b->cur], b->lat[1 - b->cur], nsteps, tl);
     cudaGraph_t g = nullptr;
     cudaError_t ce = cudaStreamEndCapture(b->cap, &g);
     if (le != cudaSuccess || ce != cudaSuccess) {

@@ -83,7 +83,7 @@ struct StepConst {
   float ce_f, cp_f, cq_f;
   // fixed-eta/s relaxation: eta_s > 0 derives tau_g (BGK) / tau_v (MRT) per node; tauf_local:
   // tau_f = tau_g; for MRT the ratios a_x = (tau_x - 1/2) / (tau_v - 1/2) of e, eps, q
-  double eta_s, eta3;   // eta3 = 3 eta_s
+  double eta_s;
   int tauf_local;
   double a_e, a_p, a_q;
   // 64-bit fixed-point copies for the integer-pipe FP64 collide: omega * 2^63 (even),
@@ -95,10 +95,11 @@ struct StepConst {
   unsigned long long Om2_f, Om2_v;
   int r_f, r_v;
   long long CE, CP, CQ;
-  // the D2Q9 row constants: ce * 2^67, cp * 2^67, cq * 2^65 (norms 36, 36, 12)
-  long long CE9, CP9, CQ9;
   // coefficient of the theta term of the C_7 correction (Eq. 38): 1 (Eq. A17) or 2 (as printed)
   double c7_theta;
+  // the D2Q9 row constants: ce * 2^67, cp * 2^67, cq * 2^65 (norms 36, 36, 12)
+  long long CE9, CP9, CQ9;
+  double eta3;   // 3 eta_s
 };
 
 // q = 19 (D3Q19: weights 1/3, 1/18, 1/36; MRT row norms e 2394, eps 252, q 40) or

@@ -213,3 +213,29 @@ def test_full_sweep_1024_tubes_fp32_4000_steps():
                     float((fo.reshape(19, -1) - nf).abs().max() / fo.abs().max()))
     assert worst < 4 * 2.0 ** -24, worst
     b.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("steps", [20, 21])
+def test_few_tubes_in_clusters_bitwise_equal_one_cta_per_tube(precision, steps):
+    """A small batch gives each tube a cluster of CTAs; the same tubes repeated until they
+    fill the GPU run one CTA per tube.  The states must be equal bit for bit (lengths below and
+    above a CTA's and a cluster's threads, even and odd step counts, pinned shapes)."""
+    from paper_1211_3286_gb300.batch import TubeBatch
+    lengths = LENGTHS + [2500]
+    reps = 70   # 910 tubes: more than the CTA slots of any launch shape
+    _, taus = I.tube_sweep(len(lengths), seed=44)
+    f = _batch_fields(lengths)
+    many = TubeBatch(lengths * reps, np.tile(taus, (reps, 1)), precision=precision)
+    many.set_fields(*(t.repeat(reps) for t in f))
+    many.run(steps)
+    ref = many.state()[:, :sum(lengths)]
+    for shape in (None, (32, 0), (96, 1), (256, 1)):
+        few = TubeBatch(lengths, taus, precision=precision)
+        if shape:
+            few.set_shape(*shape)
+        few.set_fields(*f)
+        few.run(steps)
+        assert torch.equal(few.state(), ref), shape
+        few.close()
+    many.close()
