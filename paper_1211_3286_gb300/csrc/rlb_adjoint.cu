@@ -8,9 +8,10 @@
 // walked backwards by hand), where lambda^{t+1} = S^T mu^{t+1} is gathered at the node
 // inside the same kernel: the adjoint of "node x pulls link a from src(x)" is "node y
 // collects link a from every x with src(x) = y" -- one node for a periodic axis, and
-// for a zero-gradient axis also the edge node's own clamped pull.  Small lattices run
-// the reverse step with four threads per node in two warp roles (k_adj_step_ws), larger
-// ones with one thread per node (k_adj_step).
+// for a zero-gradient axis also the edge node's own clamped pull.  Small quasi-1D lattices
+// take several reverse steps per launch on integers (k_adj_tube_steps), other small ones
+// run the reverse step with four threads per node in two warp roles (k_adj_step_ws),
+// larger ones with one thread per node (k_adj_step).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -24,6 +25,7 @@
 #include "rlb_internal.h"
 #include "rlb_launch.cuh"
 #include "rlb_node.cuh"
+#include "rlb_quad.cuh"
 
 using namespace rlb;
 
@@ -660,6 +662,279 @@ __global__ void __launch_bounds__(64) k_adj_step_ws(const double* __restrict__ g
   quad_backward<MRT>(F, pc, l0, ha, hb, la, lb, cd, j, valid, i, k, mu, tb, geo.n);
 }
 
+// ---- several reverse steps per launch (quasi-1D lattices)
+//
+// mu = C_h^T lambda depends on the forward state through u alone: with the cotangents of u
+// taken per sigma, every coefficient of the walk back through the collide is dimensionless
+// (r = sigma / sqrt(A) = 2 / (3 - u^2), T00 / sigma = (3 + u^2) / 4).  The walk runs in 64-bit
+// block fixed point on the grid of the node's largest |lambda| (unit 2^-54 to 2^-55 of it),
+// where an addition costs two issue slots instead of the 64 cycles that an FP64 instruction
+// holds its unit.  The omega cotangents, which do multiply g by lambda, leave this chain: the
+// lambda of every step is stored, and k_adj_omega forms them for a whole segment at once.
+//
+// A block holds kTubeTile nodes as k_tube_steps does (tiles that overlap by one node per
+// step): warps 0..3 hold lambda, four lanes per node, and warp 4 recovers u of the next
+// step's state, one node per lane, while they walk back through this one.  1600 nodes: 7.8 ->
+// 4.3 us per reverse step, 1600 nodes x 4000 steps 40.7 -> 26.3 ms per gradient; bound by the
+// dependent integer chains of the two roles.
+struct RevU {
+  unsigned long long ax[kTubeTile], ay[kTubeTile], az[kTubeTile];
+  unsigned sg[kTubeTile];
+};
+__device__ __forceinline__ long long mul_s(long long a, long long b) { return __mul64hi(a, b); }
+
+// Cotangents of one node's pulled populations from those of its relaxed ones (v, lane
+// (m, j)'s six links; lane 3 the rest link), in place.  W62 = omega_v 2^62.
+template <bool MRT>
+__device__ __forceinline__ void quad_vjp(int lane, double (&v)[6], const RevU& ru, int i, long long W62,
+                                         const StepConst& k) {
+  using namespace fx;
+  const int j = lane & 3, base = lane & ~3;
+  unsigned me = 0;
+#pragma unroll
+  for (int sl = 0; sl < 6; ++sl) me = max(me, (unsigned)__double2hiint(v[sl]) & 0x7fffffffu);
+  me = max(me, (unsigned)__shfl_xor_sync(0xffffffffu, (int)me, 1));
+  me = max(me, (unsigned)__shfl_xor_sync(0xffffffffu, (int)me, 2));
+  const bool finite = me < 0x7f000000u;   // else (NaN, infinities, above 1e304) the node comes out NaN
+  const int E = finite ? max((int)(me >> 20), 128) : 1023;
+  long long L[6];
+#pragma unroll
+  for (int sl = 0; sl < 6; ++sl) L[sl] = to_fixed(v[sl], E + 9);   // |L| < 2^55
+  const long long l0 = __shfl_sync(0xffffffffu, L[0], base + 3);
+  // u_i 2^62 and the pairs' c.u at 2^61
+  const unsigned sg = ru.sg[i];
+  const long long ux = with_sign(ru.ax[i] >> 1, sg & 1u), uy = with_sign(ru.ay[i] >> 1, (sg >> 1) & 1u),
+                  uz = with_sign(ru.az[i] >> 1, sg >> 2);
+  const unsigned long long u2 = mulhi(ru.ax[i], ru.ax[i]) + mulhi(ru.ay[i], ru.ay[i]) + mulhi(ru.az[i], ru.az[i]);
+  const bool pairs = j < 3;
+  const long long ca = sel3(j, ux, uy, uz) >> 1;
+  const long long cp = (sel3(j, ux, uy, ux) >> 1) + (sel3(j, uy, uz, uz) >> 1);
+  const long long cm = (sel3(j, ux, uy, ux) >> 1) - (sel3(j, uy, uz, uz) >> 1);
+  constexpr long long kT = 0x2aaaaaaaaaaaaaabll;   // 2^63 / 3
+  long long S[3], Q[3];
+  const long long ev[3] = {L[0] + L[1], L[2] + L[3], L[4] + L[5]};
+  const long long od[3] = {L[0] - L[1], L[2] - L[3], L[4] - L[5]}, cc[3] = {ca, cp, cm};
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    const long long p1 = mul_s(ev[p] << 3, cc[p]), o3 = mul_s(od[p] << 1, kT);   // c ev, od / 3
+    S[p] = mul_s((p1 + 2 * o3) << 3, cc[p]);                                     // c (c ev + 2 od / 3)
+    Q[p] = p1 + o3;
+  }
+  const long long hS = (Q[1] >> 1) + (Q[2] >> 1), hD = (Q[1] >> 1) - (Q[2] >> 1);
+  const long long KA = quad_sum64(pairs ? ev[0] : 0), KD = quad_sum64(pairs ? ev[1] + ev[2] : 0);
+  const long long SW = quad_sum64(pairs ? S[0] + ((S[1] + S[2]) >> 1) : 0);      // 4 times the density's cotangent
+  const long long Bx = quad_sum64(j == 0 ? Q[0] + hS : (j == 2 ? hS : 0));       // as the momentum sums of quad_collide
+  const long long By = quad_sum64(j == 0 ? hD : (j == 1 ? Q[0] + hS : 0));
+  const long long Bz = quad_sum64(j == 1 ? hD : (j == 2 ? Q[0] + hD : 0));
+  const auto om = [W62](long long x) { return mul_s(x << 2, W62); };             // omega x
+  long long gq = om(l0);                                                         // of g^eq_0
+  const long long kg = om(mul_s(2 * KA + KD, (long long)k36th));                 // of 3P - 1.5 sigma u^2
+  long long sb = om(SW >> 2), Sab = 0, Sdb = 0, Pb = 0, s2 = 0, h0 = 0;
+  if (MRT) {
+    const long long a16 = 30 * (l0 >> 4) + 11 * (KA >> 4) - 8 * (KD >> 4);
+    const long long p16 = 4 * (KA >> 4) - (KD >> 4) - 12 * (l0 >> 4);
+    const long long e8 = mul_s(a16, k.CE) >> 2, p8 = mul_s(p16 << 2, k.CP);      // 8 ce (..), 8 cp (..)
+    h0 = (12 * p8 - 30 * e8) >> 3;
+    Sab = -((11 * e8 + 4 * p8) >> 3);
+    Sdb = (8 * e8 + p8) >> 3;
+    gq -= h0;
+    Pb = -Sab - Sdb;
+    s2 = -(Sdb >> 1);
+  }
+  sb += gq;
+  s2 -= (gq + 3 * kg) >> 1;                                                      // of sigma u^2
+  Pb += 3 * (kg - gq);
+  sb += mul_s(s2 << 2, (long long)u2);
+  const long long bx = (om(Bx) >> 1) + 2 * mul_s(s2 << 2, ux), by = (om(By) >> 1) + 2 * mul_s(s2 << 2, uy),
+                  bz = (om(Bz) >> 1) + 2 * mul_s(s2 << 2, uz);                   // of u, per sigma
+  sb += Pb;
+  sb -= mul_s(bx << 2, ux) + mul_s(by << 2, uy) + mul_s(bz << 2, uz);
+  const long long r = (long long)(rcp_fixed((3ull << 62) - u2) >> 1);            // 2 / (3 - u^2) 2^62
+  const long long w = mul_s(sb << 2, r);
+  const long long T = 2 * w - Pb;                                                // of T00
+  const long long mx = bx - mul_s(w << 2, ux), my = by - mul_s(w << 2, uy), mz = bz - mul_s(w << 2, uz);
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
+  if (pairs) {
+    const long long da = sel3(j, mx, my, mz), a = sel3(j, mx, my, mx), b = sel3(j, my, mz, mz);
+    const long long d[3] = {da, a + b, a - b};
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      const long long t = (p == 0 ? Sab : Sdb) + T;
+      long long ya = L[2 * p] - om(L[2 * p]) + t, yb = L[2 * p + 1] - om(L[2 * p + 1]) + t;
+      asm("" : "+l"(ya), "+l"(yb));   // sums kept apart, as in relax_links_store
+      v[2 * p] = finite ? from_fixed_rn(ya + d[p], E + 2) : nan;
+      v[2 * p + 1] = finite ? from_fixed_rn(yb - d[p], E + 2) : nan;
+    }
+  } else {
+    v[0] = finite ? from_fixed_rn(l0 - om(l0) + T + h0, E + 2) : nan;
+#pragma unroll
+    for (int sl = 1; sl < 6; ++sl) v[sl] = v[0];
+  }
+}
+
+// `steps` reverse steps: the first works on the state g (one array of 19 nx), each later one
+// on the array before it, and stores its lambda at lam, each later one in the array before.
+// in: lambda of the first step itself (first), else the mu to gather it from; out: the last mu.
+template <bool MRT>
+__global__ void __launch_bounds__(32 * (kTubeWarps + 1))
+    k_adj_tube_steps(const double* __restrict__ g, double* __restrict__ lam, const double* __restrict__ in,
+                     double* __restrict__ out, int nx, int zg, StepConst k, int steps, int core, bool first) {
+  __shared__ RevU ru[2];
+  __shared__ double ex[2][2][6][kTubeTile];   // [parity][lane 0 / 2][slot][node]
+  wait_for_grid(g, in);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool u_warp = warp == kTubeWarps;
+  const int i = u_warp ? lane : warp * 8 + (lane >> 2), j = u_warp ? 0 : lane & 3;
+  const int halo = (kTubeTile - core) >> 1;
+  const int xg = (int)blockIdx.x * core - halo + i;
+  const bool own = i >= halo && i < halo + core && xg < nx;
+  const bool idle = zg && (xg < 0 || xg >= nx);                 // past an open end
+  const int x = zg ? min(max(xg, 0), nx - 1) : (xg < 0 ? (xg % nx + nx) % nx : xg % nx);
+  const bool whole = core == kTubeTile;
+  const unsigned long long n = (unsigned long long)nx;
+  if (u_warp) {
+    const int xm = x > 0 ? x - 1 : (zg ? 0 : nx - 1), xp = x < nx - 1 ? x + 1 : (zg ? nx - 1 : 0);
+    double h[19];
+    const auto load = [&](const double* gs) {
+#pragma unroll
+      for (int a = 0; a < 19; ++a) h[a] = gs[(unsigned long long)a * n + (link_cx(a) > 0 ? xm : link_cx(a) < 0 ? xp : x)];
+    };
+    load(g);
+    for (int s = 0; s < steps; ++s) {
+      bool fast;
+      const int E = fx::max_exponent(h, fast);
+      long long X[19];
+      if (__all_sync(0xffffffffu, fast)) {
+#pragma unroll
+        for (int a = 0; a < 19; ++a) X[a] = fx::to_fixed_pos(h[a], E + 7);
+      } else {
+#pragma unroll
+        for (int a = 0; a < 19; ++a) X[a] = fx::to_fixed(h[a], E + 7);
+      }
+      if (s + 1 < steps) load(g - (unsigned long long)(s + 1) * 19ull * n);   // in flight during the recovery
+      long long T = X[0], d[9];
+#pragma unroll
+      for (int p = 0; p < 9; ++p) {
+        T += X[2 * p + 1] + X[2 * p + 2];
+        d[p] = X[2 * p + 1] - X[2 * p + 2];
+      }
+      UFix u;
+      bool br;
+      fx_recover(T, d[0] + d[3] + d[4] + d[5] + d[6], d[1] + d[3] - d[4] + d[7] + d[8], d[2] + d[5] - d[6] + d[7] - d[8],
+                 u, br);
+      RevU& r = ru[s & 1];
+      r.ax[i] = u.ax;
+      r.ay[i] = u.ay;
+      r.az[i] = u.az;
+      r.sg[i] = u.sx | (u.sy << 1) | (u.sz << 2);
+      __syncthreads();   // step s may start; step s - 1 has read the other buffer
+    }
+    return;
+  }
+  // lambda of the first step
+  double v[6];
+#pragma unroll
+  for (int sl = 0; sl < 6; ++sl) {
+    int cx, cy, cz;
+    quad_dir(j, sl, cx, cy, cz);
+    const double* at = in + (unsigned long long)quad_link(j, sl) * n;
+    v[sl] = idle ? 0.0 : first ? at[x] : gather_link_tube(at, x, cx, AGeo{nx, 1, 1, zg, 0, 0, n});
+  }
+  const long long W62 = (long long)(k.Om_v >> 1);
+  // preimages of the x-moving links: cx = +1 (even slots) node i + 1, cx = -1 node i - 1; at an
+  // open end none beyond it, and the end node its own clamped pull
+  const bool lo = xg == 0, hi = xg == nx - 1;
+  const bool np = !(zg && hi), nm = !(zg && lo);
+  const int ip = whole && hi ? 0 : min(i + 1, kTubeTile - 1), im = whole && lo ? nx - 1 : max(i - 1, 0);
+  const bool axis_moves = j == 0, moves = j == 0 || j == 2;
+  for (int s = 0; s < steps; ++s) {
+    __syncthreads();
+    if (s > 0 && moves) {
+      auto& e = ex[s & 1][j >> 1];
+#pragma unroll
+      for (int sl = 0; sl < 6; ++sl)
+        if (sl >= 2 || axis_moves) {
+          const bool plus = (sl & 1) == 0;
+          double t = (plus ? np : nm) ? e[sl][plus ? ip : im] : 0.0;
+          if (zg && (plus ? lo : hi)) t += v[sl];
+          v[sl] = idle ? 0.0 : t;
+        }
+    }
+    if (own) {
+      double* ls = lam - (unsigned long long)s * 19ull * n + (unsigned)x;
+      ls[(unsigned long long)quad_link(j, 0) * n] = v[0];
+      if (j < 3) {
+#pragma unroll
+        for (int sl = 1; sl < 6; ++sl) ls[(unsigned long long)quad_link(j, sl) * n] = v[sl];
+      }
+    }
+    quad_vjp<MRT>(lane, v, ru[s & 1], i, W62, k);
+    if (s == steps - 1) break;
+    if (moves) {
+      auto& e = ex[(s + 1) & 1][j >> 1];
+#pragma unroll
+      for (int sl = 0; sl < 6; ++sl)
+        if (sl >= 2 || axis_moves) e[sl][i] = v[sl];
+    }
+  }
+  if (own) {
+    double* o = out + (unsigned)x;
+    o[(unsigned long long)quad_link(j, 0) * n] = v[0];
+    if (j < 3) {
+#pragma unroll
+      for (int sl = 1; sl < 6; ++sl) o[(unsigned long long)quad_link(j, sl) * n] = v[sl];
+    }
+  }
+}
+
+// The omega cotangents of every node and step of a segment (blockIdx.y: the step), from its
+// states and stored lambdas, and their sum over the steps in the order of the sweep.
+template <bool MRT>
+__global__ void __launch_bounds__(kThreads) k_adj_omega(const double* __restrict__ g, const double* __restrict__ lam,
+                                                       double* __restrict__ part, int nx, int zg, StepConst k) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= nx) return;
+  const unsigned long long n = (unsigned long long)nx, off = blockIdx.y * 19ull * n;
+  double h[19], lo[19];
+#pragma unroll
+  for (int a = 0; a < 19; ++a) {
+    h[a] = g[off + (unsigned long long)a * n + pull_src(x, link_cx(a), nx, zg)];
+    lo[a] = lam[off + (unsigned long long)a * n + x];
+  }
+  // d/d omega_v = lambda . (g^eq - h) less the e and eps rows; the differences link by link,
+  // before the product, keep what the sums over g^eq and h would cancel
+  GFwd F;
+  gforward(h, k, MRT, F);
+  double wvb = (F.geq0 - h[0]) * lo[0], KAb = 0, KDb = 0;
+#pragma unroll
+  for (int p = 0; p < 9; ++p) {
+    const double w = p < 3 ? 1.0 / 18.0 : 1.0 / 36.0, c = F.cu[p];
+    const double e = w * fma(4.5 * F.sigma * c, c, F.kg), o = (3.0 * w) * F.sigma * c;
+    const double la = lo[2 * p + 1], lb = lo[2 * p + 2];
+    wvb = fma((e + o) - h[2 * p + 1], la, fma((e - o) - h[2 * p + 2], lb, wvb));
+    if (p < 3) KAb += la + lb;
+    else KDb += la + lb;
+  }
+  double web = 0, wpb = 0;
+  if (MRT) {
+    web = F.ne * fma(11.0, KAb, fma(-8.0, KDb, 30.0 * lo[0])) * (1.0 / 2394.0);
+    wpb = F.np * (fma(4.0, KAb, -KDb) - 12.0 * lo[0]) * (1.0 / 252.0);
+    wvb -= web + wpb;
+  }
+  double* p = part + blockIdx.y * 3ull * n + x;
+  p[0] = wvb;
+  p[n] = web;
+  p[2 * n] = wpb;
+}
+__global__ void __launch_bounds__(kThreads) k_adj_omega_sum(const double* __restrict__ part, double* __restrict__ tb,
+                                                           unsigned long long n3, int steps) {
+  const unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
+  if (i >= n3) return;
+  double acc = tb[i];
+  for (int s = steps - 1; s >= 0; --s) acc += part[(unsigned long long)s * n3 + i];
+  tb[i] = acc;
+}
+
 // lambda^T = dJ/dg^T and the per-node misfit.
 __global__ void __launch_bounds__(kThreads) k_adj_loss(const double* __restrict__ g, const double* __restrict__ tP,
                                                       const double* __restrict__ tux, const double* __restrict__ tuy,
@@ -738,15 +1013,17 @@ struct AdjPlan {
   bool quad = false;                          // reverse steps with four threads per node
   double wP = 0.0, wu = 0.0;                  // misfit weights baked into the graph
   std::vector<void*> ckpt, owned;
-  // g^{t0 + j} of a recomputed segment at seg[s & 1][j] (quasi-1D: j >= 1, one array of g after
-  // the other, j = 0 read from the checkpoint; else whole states)
+  // g^{t0 + j} of a recomputed segment at seg[s & 1][j] (quasi-1D: one array of g after the
+  // other, and the lambda of each step in lamseg likewise; else whole states)
   std::vector<void*> seg[2];
   double *lam = nullptr, *mu = nullptr, *tb = nullptr, *lossn = nullptr, *sums = nullptr, *dde0 = nullptr;
   double* fw[2] = {nullptr, nullptr};         // QFwd of alternate reverse steps (two warp roles)
   double* tgt = nullptr;
+  double *lamseg[2] = {nullptr, nullptr}, *part = nullptr;   // quasi-1D: stored lambdas, omega cotangents per step
+  cudaStream_t cap3 = nullptr;                // the omega cotangents beside the sweep of the next segment
   cudaStream_t cap = nullptr;
   cudaStream_t cap2 = nullptr;                // recompute of segment s - 1 beside the reverse sweep of s
-  cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // fork, ready[2], free[2]
+  cudaEvent_t ev[7] = {};                     // fork, ready[2], free[2], swept[2]
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
 };
@@ -758,6 +1035,7 @@ void free_plan(void* p) {
   if (a->graph) cudaGraphDestroy(a->graph);
   if (a->cap) cudaStreamDestroy(a->cap);
   if (a->cap2) cudaStreamDestroy(a->cap2);
+  if (a->cap3) cudaStreamDestroy(a->cap3);
   for (cudaEvent_t e : a->ev)
     if (e) cudaEventDestroy(e);
   for (void* q : a->owned) cudaFree(q);
@@ -819,7 +1097,7 @@ cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, boo
   // Forward with checkpoints (of which the first is the initial state).  On a quasi-1D lattice
   // the forward run and the recompute take several steps per launch, the forward run writes
   // its checkpoints in place and the recompute advances g alone: 1600 nodes x 4000 steps
-  // 46.9 -> 40.7 ms per gradient, and a first gradient (capture included) 76.7 -> 52.5.
+  // 46.9 -> 40.7 ms per gradient with single reverse steps.
   const bool many = a->most > 1;
   ENQ(cudaMemcpyAsync(a->ckpt[0], h->lat[h->cur], state_bytes, cudaMemcpyDeviceToDevice, st));
   if (many) {
@@ -858,15 +1136,16 @@ cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, boo
   const int saved_cur = h->cur;
   // g at step t0 + j of segment s
   auto g_at = [&](int s, int j) -> const double* {
-    return many ? (j == 0 ? (const double*)a->ckpt[s] + 19 * N : (const double*)a->seg[s & 1][j])
-                : (const double*)a->seg[s & 1][j] + 19 * N;
+    return (const double*)a->seg[s & 1][j] + (many ? 0 : 19 * N);
   };
   auto recompute = [&](int s) -> cudaError_t {
     const std::vector<void*>& b = a->seg[s & 1];
     const int t0 = s * K, t1 = std::min(T, t0 + K);
     cudaError_t r = cudaSuccess;
     if (many) {
-      // g alone; the first launch of a segment follows another stream's event
+      // g alone
+      r = cudaMemcpyAsync(b[0], (const double*)a->ckpt[s] + 19 * N, 19 * N * sizeof(double), cudaMemcpyDeviceToDevice,
+                          cs);
       for (int j = 0; r == cudaSuccess && j + 1 < t1 - t0;) {
         const int n = std::min(a->most, t1 - t0 - 1 - j);
         r = enqueue_tube(h, g_at(s, j), (double*)b[j + 1], n, a->core, true, j > 0, cs);
@@ -895,6 +1174,31 @@ cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, boo
     }
     ENQ(cudaStreamWaitEvent(st, ev_ready[s & 1], 0));
     const int t0 = s * K, t1 = std::min(T, t0 + K);
+    if (many) {
+      // the sweep, then its omega cotangents on the third stream, beside the next segment's
+      for (int j = t1 - t0 - 1; j >= 0;) {
+        const int c = std::min(a->most, j + 1);
+        const bool first = t0 + j == T - 1;
+        double* out = mu_cur == a->mu ? a->lam : a->mu;
+        double* ls = a->lamseg[s & 1] + (size_t)j * 19 * N;
+        launch_after(dim3((unsigned)((N + a->core - 1) / a->core)), 32 * (kTubeWarps + 1), st, j < t1 - t0 - 1,
+                     mrt ? k_adj_tube_steps<true> : k_adj_tube_steps<false>, g_at(s, j), ls, first ? a->lam : mu_cur, out,
+                     geo.nx, geo.zgx, h->k, c, a->core, first);
+        ENQ(cudaGetLastError());
+        mu_cur = out;
+        j -= c;
+      }
+      cudaEvent_t swept = a->ev[5 + (s & 1)];
+      ENQ(cudaEventRecord(swept, st));
+      ENQ(cudaStreamWaitEvent(a->cap3, swept, 0));
+      const dim3 go((unsigned)((N + kThreads - 1) / kThreads), (unsigned)(t1 - t0));
+      if (mrt) k_adj_omega<true><<<go, kThreads, 0, a->cap3>>>(g_at(s, 0), a->lamseg[s & 1], a->part, geo.nx, geo.zgx, h->k);
+      else k_adj_omega<false><<<go, kThreads, 0, a->cap3>>>(g_at(s, 0), a->lamseg[s & 1], a->part, geo.nx, geo.zgx, h->k);
+      k_adj_omega_sum<<<(unsigned)((3 * N + kThreads - 1) / kThreads), kThreads, 0, a->cap3>>>(a->part, a->tb, 3 * N, t1 - t0);
+      ENQ(cudaGetLastError());
+      ENQ(cudaEventRecord(ev_free[s & 1], a->cap3));
+      continue;
+    }
     if (a->quad && t1 == T) {   // the QFwd of the last step
       if (tube) {
         if (mrt) k_adj_fwd<true, true><<<grid8, 64, 0, st>>>(g_at(s, T - 1 - t0), a->fw[(T - 1) & 1], geo, h->k);
@@ -937,6 +1241,7 @@ cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, boo
   // join the second stream back into the capture
   ENQ(cudaEventRecord(ev_fork, cs));
   ENQ(cudaStreamWaitEvent(st, ev_fork, 0));
+  if (many) ENQ(cudaStreamWaitEvent(st, ev_free[0], 0));   // segment 0's omega cotangents, the last of that stream
   ENQ(cudaGetLastError());
   k_adj_e0<<<grid3, th, 0, st>>>((const double*)a->ckpt[0] + 19 * N, mu_cur, a->dde0, geo, lanes);
   k_rowsum<<<3, 256, 0, st>>>(a->tb, N, a->sums);
@@ -1004,18 +1309,21 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
       if (a->most > 1) {
         void* all = nullptr;
         ok = ok && plan_alloc(a, &all, (size_t)a->K * gbytes);
-        for (int j = 1; j < a->K && ok; ++j) a->seg[q][j] = (char*)all + (size_t)(j - 1) * gbytes;
+        for (int j = 0; j < a->K && ok; ++j) a->seg[q][j] = (char*)all + (size_t)j * gbytes;
+        ok = ok && plan_alloc(a, (void**)&a->lamseg[q], (size_t)a->K * gbytes);
       } else {
         for (int j = 0; j <= a->K && ok; ++j) ok = plan_alloc(a, &a->seg[q][j], state_bytes);
       }
     }
-    for (int i = 0; i < 5 && ok; ++i) ok = cudaEventCreateWithFlags(&a->ev[i], cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaStreamCreateWithFlags(&a->cap2, cudaStreamNonBlocking) == cudaSuccess;
+    for (int i = 0; i < 7 && ok; ++i) ok = cudaEventCreateWithFlags(&a->ev[i], cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaStreamCreateWithFlags(&a->cap2, cudaStreamNonBlocking) == cudaSuccess &&
+         cudaStreamCreateWithFlags(&a->cap3, cudaStreamNonBlocking) == cudaSuccess;
     ok = ok && plan_alloc(a, (void**)&a->lam, gbytes) && plan_alloc(a, (void**)&a->mu, gbytes) &&
          plan_alloc(a, (void**)&a->tb, 3 * N * sizeof(double)) && plan_alloc(a, (void**)&a->lossn, N * sizeof(double)) &&
          plan_alloc(a, (void**)&a->sums, 8 * sizeof(double)) && plan_alloc(a, (void**)&a->dde0, N * sizeof(double)) &&
          plan_alloc(a, (void**)&a->tgt, 4 * N * sizeof(double));
-    for (int i = 0; i < 2 && ok && a->quad; ++i)
+    if (a->most > 1) ok = ok && plan_alloc(a, (void**)&a->part, (size_t)a->K * 3 * N * sizeof(double));
+    for (int i = 0; i < 2 && ok && a->quad && a->most == 1; ++i)
       ok = plan_alloc(a, (void**)&a->fw[i], (kFwdFields + 9 * kPairFields) * N * sizeof(double));
     if (!ok || cudaStreamCreateWithFlags(&a->cap, cudaStreamNonBlocking) != cudaSuccess) {
       free_plan(a);

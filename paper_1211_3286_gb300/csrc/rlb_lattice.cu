@@ -28,6 +28,7 @@
 #include "rlb_io.cuh"
 #include "rlb_launch.cuh"
 #include "rlb_node.cuh"
+#include "rlb_quad.cuh"
 
 using namespace rlb;
 
@@ -54,7 +55,6 @@ int cuda_fail(rlb_handle* h, cudaError_t e, const char* what) {
 
 constexpr int kBlockX = 128;
 constexpr unsigned long long kSmallNodes = 152ull * 128ull * 2ull;   // lattices that cannot fill the GPU
-constexpr int kTubeWarps = 4;     // g (and f) warps of a block of k_tube_steps
 constexpr int kRedBlocks = 608;   // 4 x 152 SMs; fixed so the reduction order is fixed
 constexpr int kRedThreads = 256;
 
@@ -471,36 +471,6 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? (ETA ? 8 : 14) : RLB_WS_WARPS
 // arithmetic of k_step_ws, link for link, with a node's dependent chain about a third as
 // long.  u goes to the f warp through shared memory across a named barrier of the warp
 // pair.  No separate tau_q (QSEP) in this form.
-__device__ __forceinline__ long long quad_sum64(long long v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  return v;
-}
-__device__ __forceinline__ long long sel3(int j, long long v0, long long v1, long long v2) {
-  return j == 0 ? v0 : (j == 1 ? v1 : v2);
-}
-// slot sl of lane j: link and direction (slots 0-1 the axis pair, 2-3 the first diagonal
-// pair of the lane's plane, 4-5 the second); lane 3 reads the rest link in every slot
-__device__ __forceinline__ int quad_link(int j, int sl) {
-  const int pd = j == 0 ? 3 : (j == 1 ? 7 : 5);   // first diagonal pair of the plane
-  return j == 3 ? 0 : sl < 2 ? 2 * j + 1 + sl : 2 * pd + 1 + (sl - 2);
-}
-__device__ __forceinline__ void quad_dir(int j, int sl, int& cx, int& cy, int& cz) {
-  const int da = j == 1 ? 1 : 0, db = j == 0 ? 1 : 2;
-  if (sl < 2) {
-    const int c = sl == 0 ? 1 : -1;
-    cx = j == 0 ? c : 0;
-    cy = j == 1 ? c : 0;
-    cz = j == 2 ? c : 0;
-  } else {
-    const int sa = (sl & 1) ? -1 : 1;              // +(e_a + e_b), -(e_a + e_b), +(e_a - e_b), -(e_a - e_b)
-    const int sb = sl < 4 ? sa : -sa;
-    cx = da == 0 ? sa : 0;                          // db is never x
-    cy = (da == 1 ? sa : 0) + (db == 1 ? sb : 0);
-    cz = db == 2 ? sb : 0;                          // da is never z
-  }
-  if (j == 3) cx = cy = cz = 0;
-}
 // u of the 8 nodes of a warp pair
 struct QuadU {
   unsigned long long ax[8], ay[8], az[8];
@@ -696,7 +666,6 @@ __global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ 
 // 1600 nodes), the output rounding on the integer pipe (2.84 against 2.59 at 8 steps).
 //   G_ONLY: g alone (it does not depend on f), src and dst hold g only, and every step's g
 //   is stored, step s at dst + 19 nx s (the adjoint's recompute).
-constexpr int kTubeTile = 8 * kTubeWarps;
 template <bool MRT, int RV, int RF, bool G_ONLY>
 __global__ void __launch_bounds__((G_ONLY ? 32 : 64) * kTubeWarps)
     k_tube_steps(const double* __restrict__ src, double* __restrict__ dst, int nx, int bcx, StepConst k, int steps,

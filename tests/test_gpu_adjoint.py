@@ -186,3 +186,38 @@ def test_adjoint_matches_oracle_at_mid_size(shape, kind, T, K):
     assert float((dtau - dref).abs().max() / dref.abs().max()) <= 1e-8, (dtau, dref)
     err = float((de0.cpu() - eref).abs().max() / eref.abs().max())
     assert err <= 1e-8, err
+
+
+@pytest.mark.parametrize("collision", ["mrt", "bgk"])
+@pytest.mark.parametrize("bcx", ["zero_gradient", "periodic"])
+@pytest.mark.parametrize("L", [1, 2, 31, 32, 33, 61])
+def test_adjoint_of_tubes_around_the_tile_size(L, bcx, collision):
+    """Quasi-1D gradients at the sizes where the tiles of the multi-step kernels change: one
+    node, a tile that holds the whole lattice (wrapping or open), one node more, a ragged
+    last tile; 25 steps (several launches, a ragged last segment) against the oracle's discrete
+    gradient, with the bounds of test_adjoint_matches_oracle_discrete_gradient plus, for
+    dJ/dtau, its rounding of about 2^-53 x 25 steps x 19 links x |lambda| |g| with |lambda| |g| <=
+    2e3 J (the targets are 1e-3 off), below 1e-9 J: on one node, and nearly so on two, dJ/dtau
+    is a sum that cancels (a single node stays at equilibrium)."""
+    taus = (0.9, 0.55, 0.8) if collision == "mrt" else (0.9, 0.9, 0.9)
+    bc = (bcx, "periodic", "periodic")
+    e, u, n, tgt = _case((1, 1, L), "box", 55, taus, collision, bc, 25)
+    loss, dtau, de0 = _gpu_grad(e, u, n, tgt, taus, collision, bc, 25)
+    prm = O.Params(collision=collision, tau_f=taus[0], tau_v=taus[0], tau_e=taus[1], tau_eps=taus[2], bc=_obc(bc))
+    lref, dref, eref = O.misfit_and_gradient(e, u, n, prm, 25, tgt.P, tgt.u)
+    assert abs(loss - lref) <= 1e-9 * abs(lref)
+    want = dref if collision == "mrt" else dref * torch.tensor([1.0, 0, 0])
+    assert float((dtau - want).abs().max()) <= 1e-8 * float(dref.abs().max()) + 1e-9 * abs(lref)
+    assert float((de0.cpu() - eref).abs().max()) <= 1e-8 * float(eref.abs().max())
+
+
+def test_adjoint_passes_nan_targets_on():
+    """A NaN in a target reaches the loss, the tau gradients and the initial field's gradient in
+    its domain of dependence, and nowhere else."""
+    taus, T = (0.9, 0.55, 0.8), 10
+    e, u, n, tgt = _case((1, 1, 100), "tube", 56, taus, "mrt", ZG, T)
+    tgt.P[0, 0, 50] = float("nan")
+    loss, dtau, de0 = _gpu_grad(e, u, n, tgt, taus, "mrt", ZG, T)
+    assert math.isnan(loss) and bool(torch.isnan(dtau).all())
+    bad = torch.isnan(de0.cpu()).reshape(-1)
+    assert bool(bad[45:56].all()) and not bool(bad[:50 - T - 1].any()) and not bool(bad[50 + T + 2:].any())
