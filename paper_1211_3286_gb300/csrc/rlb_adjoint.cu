@@ -675,7 +675,7 @@ __global__ void __launch_bounds__(64) k_adj_step_ws(const double* __restrict__ g
 // A block holds kTubeTile nodes as k_tube_steps does (tiles that overlap by one node per
 // step): warps 0..3 hold lambda, four lanes per node, and warp 4 recovers u of the next
 // step's state, one node per lane, while they walk back through this one.  1600 nodes: 7.8 ->
-// 4.3 us per reverse step, 1600 nodes x 4000 steps 40.7 -> 26.3 ms per gradient; bound by the
+// 4.3 us per reverse step, 1600 nodes x 4000 steps 40.7 -> 27 ms per gradient; bound by the
 // dependent integer chains of the two roles.
 struct RevU {
   unsigned long long ax[kTubeTile], ay[kTubeTile], az[kTubeTile];
@@ -1004,9 +1004,9 @@ int afail(rlb_handle* h, int code, const std::string& m) {
   return code;
 }
 
-// Buffers and the captured CUDA graph of one (nsteps, checkpoint interval) shape,
-// kept on the handle so repeated gradients replay instead of re-launching ~4 T
-// kernels one by one.
+// Buffers of one (nsteps, checkpoint interval) shape and, where every step is a launch of
+// its own, the captured CUDA graph, kept on the handle so repeated gradients replay instead
+// of re-launching ~4 T kernels one by one.
 struct AdjPlan {
   int nsteps = -1, K = 0, nseg = 0, start_cur = 0, end_cur = 0, threads = 128, lanes = 128;
   int most = 1, core = 0;                     // quasi-1D: steps per launch (tube_launch_steps)
@@ -1026,6 +1026,7 @@ struct AdjPlan {
   cudaEvent_t ev[7] = {};                     // fork, ready[2], free[2], swept[2]
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
+  int runs = 0;                               // gradients computed with this plan
 };
 
 void free_plan(void* p) {
@@ -1042,13 +1043,24 @@ void free_plan(void* p) {
   delete a;
 }
 
-bool plan_alloc(AdjPlan* a, void** p, size_t bytes) {
-  if (cudaMalloc(p, bytes) != cudaSuccess) {
+// The plan's buffers come from one allocation (a gradient of 400 steps has about 60 of them):
+// plan_alloc notes each, plan_commit allocates and hands out the addresses.
+struct PlanWant {
+  void** p;
+  size_t offset;
+};
+void plan_alloc(std::vector<PlanWant>& want, size_t& total, void** p, size_t bytes) {
+  want.push_back({p, total});
+  total += (bytes + 255) & ~(size_t)255;
+}
+bool plan_commit(AdjPlan* a, const std::vector<PlanWant>& want, size_t total) {
+  void* base = nullptr;
+  if (cudaMalloc(&base, total) != cudaSuccess) {
     cudaGetLastError();
-    *p = nullptr;
     return false;
   }
-  a->owned.push_back(*p);
+  a->owned.push_back(base);
+  for (const PlanWant& w : want) *w.p = (char*)base + w.offset;
   return true;
 }
 
@@ -1077,8 +1089,9 @@ cudaError_t reverse_step(bool quad, bool tube, bool mrt, dim3 grid8, dim3 grid3,
   return cudaGetLastError();
 }
 
-// Enqueue the whole gradient computation on stream st (captured into the plan's graph).
-cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, bool mrt) {
+// Enqueue the whole gradient computation on stream st (the handle's, or the plan's stream
+// whose work is being captured).
+cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, bool mrt, cudaStream_t st) {
   const unsigned long long N = h->nodes;
   const size_t state_bytes = 38 * N * sizeof(double);
   const int T = a->nsteps, K = a->K, th = a->threads;
@@ -1087,7 +1100,6 @@ cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, boo
   const dim3 grid3((unsigned)((h->cfg.nx + lanes - 1) / lanes), (unsigned)h->cfg.ny, (unsigned)h->cfg.nz);
   const dim3 grid8((unsigned)((h->cfg.nx + 7) / 8), (unsigned)h->cfg.ny, (unsigned)h->cfg.nz);
   double* mu_cur = nullptr;   // buffer holding the mu of the latest reverse step (lam / mu alternate)
-  cudaStream_t st = a->cap;
   AGeo geo{h->cfg.nx, h->cfg.ny, h->cfg.nz, h->cfg.bc[0] == RLB_ZERO_GRADIENT, h->cfg.bc[1] == RLB_ZERO_GRADIENT,
            h->cfg.bc[2] == RLB_ZERO_GRADIENT, N};
   const bool tube = h->cfg.ny == 1 && h->cfg.nz == 1;
@@ -1302,29 +1314,36 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
     a->quad = a->threads == 32;
     a->ckpt.assign(a->nseg, nullptr);
     a->most = tube_launch_steps(h, a->core);
-    bool ok = true;
-    for (int s = 0; s < a->nseg && ok; ++s) ok = plan_alloc(a, &a->ckpt[s], state_bytes);
+    std::vector<PlanWant> want;
+    size_t total = 0;
+    const auto need = [&](void** p, size_t bytes) { plan_alloc(want, total, p, bytes); };
+    for (int s = 0; s < a->nseg; ++s) need(&a->ckpt[s], state_bytes);
+    void* all[2] = {nullptr, nullptr};
     for (int q = 0; q < 2; ++q) {
       a->seg[q].assign(a->K + 1, nullptr);
       if (a->most > 1) {
-        void* all = nullptr;
-        ok = ok && plan_alloc(a, &all, (size_t)a->K * gbytes);
-        for (int j = 0; j < a->K && ok; ++j) a->seg[q][j] = (char*)all + (size_t)j * gbytes;
-        ok = ok && plan_alloc(a, (void**)&a->lamseg[q], (size_t)a->K * gbytes);
+        need(&all[q], (size_t)a->K * gbytes);
+        need((void**)&a->lamseg[q], (size_t)a->K * gbytes);
       } else {
-        for (int j = 0; j <= a->K && ok; ++j) ok = plan_alloc(a, &a->seg[q][j], state_bytes);
+        for (int j = 0; j <= a->K; ++j) need(&a->seg[q][j], state_bytes);
       }
     }
+    need((void**)&a->lam, gbytes);
+    need((void**)&a->mu, gbytes);
+    need((void**)&a->tb, 3 * N * sizeof(double));
+    need((void**)&a->lossn, N * sizeof(double));
+    need((void**)&a->sums, 8 * sizeof(double));
+    need((void**)&a->dde0, N * sizeof(double));
+    need((void**)&a->tgt, 4 * N * sizeof(double));
+    if (a->most > 1) need((void**)&a->part, (size_t)a->K * 3 * N * sizeof(double));
+    for (int i = 0; i < 2 && a->quad && a->most == 1; ++i)
+      need((void**)&a->fw[i], (kFwdFields + 9 * kPairFields) * N * sizeof(double));
+    bool ok = plan_commit(a, want, total);
+    for (int q = 0; q < 2 && a->most > 1; ++q)
+      for (int j = 0; j < a->K; ++j) a->seg[q][j] = (char*)all[q] + (size_t)j * gbytes;
     for (int i = 0; i < 7 && ok; ++i) ok = cudaEventCreateWithFlags(&a->ev[i], cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaStreamCreateWithFlags(&a->cap2, cudaStreamNonBlocking) == cudaSuccess &&
          cudaStreamCreateWithFlags(&a->cap3, cudaStreamNonBlocking) == cudaSuccess;
-    ok = ok && plan_alloc(a, (void**)&a->lam, gbytes) && plan_alloc(a, (void**)&a->mu, gbytes) &&
-         plan_alloc(a, (void**)&a->tb, 3 * N * sizeof(double)) && plan_alloc(a, (void**)&a->lossn, N * sizeof(double)) &&
-         plan_alloc(a, (void**)&a->sums, 8 * sizeof(double)) && plan_alloc(a, (void**)&a->dde0, N * sizeof(double)) &&
-         plan_alloc(a, (void**)&a->tgt, 4 * N * sizeof(double));
-    if (a->most > 1) ok = ok && plan_alloc(a, (void**)&a->part, (size_t)a->K * 3 * N * sizeof(double));
-    for (int i = 0; i < 2 && ok && a->quad && a->most == 1; ++i)
-      ok = plan_alloc(a, (void**)&a->fw[i], (kFwdFields + 9 * kPairFields) * N * sizeof(double));
     if (!ok || cudaStreamCreateWithFlags(&a->cap, cudaStreamNonBlocking) != cudaSuccess) {
       free_plan(a);
       return afail(h, RLB_ENOMEM, "cannot allocate adjoint checkpoints and buffers");
@@ -1345,13 +1364,28 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
       ACUDA(cudaMemcpyAsync(a->tgt + c * N, src[c], N * sizeof(double),
                             where == RLB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
   }
+  // Enqueued as it is, without a graph: every gradient with several steps per launch (its
+  // launches are few enough for the host to keep ahead; 1600 nodes x 4000 steps take 27.3 ms
+  // so and 27.2 from a graph), and the first gradient of any plan (a program that makes a new
+  // lattice per gradient, as the autograd function does, would not use a graph twice: 800
+  // nodes x 400 steps 5.1 -> 3.6 ms per call with the plan's buffers in one allocation).
+  const bool direct = a->most > 1 || a->runs++ == 0;
+  const long long steps_before = h->steps;
+  if (direct) {
+    const cudaError_t de = enqueue_adjoint(h, a, w_P, w_u, mrt, st);
+    if (de != cudaSuccess) {
+      h->cur = a->start_cur;
+      h->steps = steps_before;
+      return afail(h, RLB_ECUDA, std::string("adjoint launch: ") + cudaGetErrorString(de));
+    }
+  }
   // capture once per plan (the misfit weights are kernel arguments: recapture if they change)
-  if (!a->exec || a->wP != w_P || a->wu != w_u) {
+  if (!direct && (!a->exec || a->wP != w_P || a->wu != w_u)) {
     if (a->exec) { cudaGraphExecDestroy(a->exec); a->exec = nullptr; }
     if (a->graph) { cudaGraphDestroy(a->graph); a->graph = nullptr; }
     const long long steps0 = h->steps;
     ACUDA(cudaStreamBeginCapture(a->cap, cudaStreamCaptureModeThreadLocal));
-    cudaError_t ce = enqueue_adjoint(h, a, w_P, w_u, mrt);
+    cudaError_t ce = enqueue_adjoint(h, a, w_P, w_u, mrt, a->cap);
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(a->cap, &g);
     h->cur = a->start_cur;   // nothing ran yet
@@ -1365,7 +1399,7 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
     a->wP = w_P;
     a->wu = w_u;
   }
-  ACUDA(cudaGraphLaunch(a->exec, st));
+  if (!direct) ACUDA(cudaGraphLaunch(a->exec, st));
   double hs[4];
   ACUDA(cudaMemcpyAsync(hs, a->sums, 4 * sizeof(double), cudaMemcpyDeviceToHost, st));
   if (de0)
@@ -1373,7 +1407,7 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
                           where == RLB_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st));
   ACUDA(cudaStreamSynchronize(st));
   h->cur = a->end_cur;
-  h->steps += nsteps;
+  h->steps = steps_before + nsteps;
   {
     unsigned long long bad = ~0ull;
     ACUDA(cudaMemcpy(&bad, h->d_bad, sizeof bad, cudaMemcpyDeviceToHost));
