@@ -327,7 +327,6 @@ __device__ __forceinline__ double quad_sum(double v) {
 
 // The pulled g of lane j's three link pairs p = j, j + 4, j + 8 at node (x, y, z) (zeros
 // for p > 8) and their directions.
-template <bool TUBE>
 __device__ __forceinline__ void quad_pull(const double* __restrict__ g, int x, int y, int z, int j, const AGeo& geo,
                                           double (&ha)[3], double (&hb)[3], int (&cd)[3][3]) {
   const unsigned long long n = geo.n;
@@ -343,13 +342,11 @@ __device__ __forceinline__ void quad_pull(const double* __restrict__ g, int x, i
     if (p <= 8) {
       const unsigned long long a1 = 2 * p + 1, a2 = 2 * p + 2;
       const unsigned long long s1 =
-          TUBE ? (unsigned long long)pull_src(x, cx, geo.nx, geo.zgx)
-               : ((unsigned long long)pull_src(z, cz, geo.nz, geo.zgz) * geo.ny + pull_src(y, cy, geo.ny, geo.zgy)) *
-                         geo.nx + pull_src(x, cx, geo.nx, geo.zgx);
+          ((unsigned long long)pull_src(z, cz, geo.nz, geo.zgz) * geo.ny + pull_src(y, cy, geo.ny, geo.zgy)) * geo.nx +
+          pull_src(x, cx, geo.nx, geo.zgx);
       const unsigned long long s2 =
-          TUBE ? (unsigned long long)pull_src(x, -cx, geo.nx, geo.zgx)
-               : ((unsigned long long)pull_src(z, -cz, geo.nz, geo.zgz) * geo.ny + pull_src(y, -cy, geo.ny, geo.zgy)) *
-                         geo.nx + pull_src(x, -cx, geo.nx, geo.zgx);
+          ((unsigned long long)pull_src(z, -cz, geo.nz, geo.zgz) * geo.ny + pull_src(y, -cy, geo.ny, geo.zgy)) * geo.nx +
+          pull_src(x, -cx, geo.nx, geo.zgx);
       ha[s] = g[a1 * n + s1];
       hb[s] = g[a2 * n + s2];
     }
@@ -358,7 +355,7 @@ __device__ __forceinline__ void quad_pull(const double* __restrict__ g, int x, i
 
 // lambda of lane j's pairs at the node: read directly (FIRST, the last step) or
 // gathered from the mu of the step after it.
-template <bool FIRST, bool TUBE>
+template <bool FIRST>
 __device__ __forceinline__ void quad_lambda(const double* __restrict__ in, int x, int y, int z, int j,
                                             unsigned long long i, const AGeo& geo, const int (&cd)[3][3],
                                             double (&la)[3], double (&lb)[3]) {
@@ -370,8 +367,8 @@ __device__ __forceinline__ void quad_lambda(const double* __restrict__ in, int x
     if (p <= 8) {
       const unsigned long long a1 = 2 * p + 1, a2 = 2 * p + 2;
       const int cx = cd[s][0], cy = cd[s][1], cz = cd[s][2];
-      la[s] = FIRST ? in[a1 * n + i] : gather_any<TUBE>(in + a1 * n, x, y, z, cx, cy, cz, geo);
-      lb[s] = FIRST ? in[a2 * n + i] : gather_any<TUBE>(in + a2 * n, x, y, z, -cx, -cy, -cz, geo);
+      la[s] = FIRST ? in[a1 * n + i] : gather_link(in + a1 * n, x, y, z, cx, cy, cz, geo);
+      lb[s] = FIRST ? in[a2 * n + i] : gather_link(in + a2 * n, x, y, z, -cx, -cy, -cz, geo);
     }
   }
 }
@@ -610,7 +607,7 @@ __device__ __forceinline__ void quad_backward(const QFwd& F, const double (&pc)[
 // (from g_prev, the state at step t - 1, into fw_prev) for the next launch.  The two
 // warps run on different sub-partitions, so each has its own FP64 unit.  k_adj_fwd
 // stores the values of one step on its own (the last step, where the sweep starts).
-template <bool MRT, bool TUBE>
+template <bool MRT>
 __global__ void __launch_bounds__(64) k_adj_fwd(const double* __restrict__ g, double* __restrict__ fw, AGeo geo,
                                                 StepConst k) {
   const int j = threadIdx.x & 3;
@@ -622,13 +619,13 @@ __global__ void __launch_bounds__(64) k_adj_fwd(const double* __restrict__ g, do
   double ha[3], hb[3], pc[3][kPairFields];
   int cd[3][3];
   const double h0 = g[i];
-  quad_pull<TUBE>(g, x, y, z, j, geo, ha, hb, cd);
+  quad_pull(g, x, y, z, j, geo, ha, hb, cd);
   QFwd F;
   quad_forward<MRT>(h0, ha, hb, cd, j, k, F, pc);
   if (valid) store_fwd(fw, i, geo.n, F, j == 0, j, pc);
 }
 
-template <bool MRT, bool FIRST, bool TUBE>
+template <bool MRT, bool FIRST>
 __global__ void __launch_bounds__(64) k_adj_step_ws(const double* __restrict__ g, const double* __restrict__ in,
                                                     double* __restrict__ mu, double* __restrict__ tb,
                                                     const double* __restrict__ fw, const double* __restrict__ g_prev,
@@ -649,15 +646,15 @@ __global__ void __launch_bounds__(64) k_adj_step_ws(const double* __restrict__ g
     // step t - 1's forward values (none before step 0)
     if (g_prev == nullptr) return;
     const double h0 = g_prev[i];
-    quad_pull<TUBE>(g_prev, x, y, z, j, geo, ha, hb, cd);
+    quad_pull(g_prev, x, y, z, j, geo, ha, hb, cd);
     quad_forward<MRT>(h0, ha, hb, cd, j, k, F, pc);
     if (valid) store_fwd(fw_prev, i, geo.n, F, j == 0, j, pc);
     return;
   }
   const double l0 = in[i];
   double la[3], lb[3];
-  quad_pull<TUBE>(g, x, y, z, j, geo, ha, hb, cd);
-  quad_lambda<FIRST, TUBE>(in, x, y, z, j, i, geo, cd, la, lb);
+  quad_pull(g, x, y, z, j, geo, ha, hb, cd);
+  quad_lambda<FIRST>(in, x, y, z, j, i, geo, cd, la, lb);
   load_fwd(fw, i, geo.n, j, F, pc);
   quad_backward<MRT>(F, pc, l0, ha, hb, la, lb, cd, j, valid, i, k, mu, tb, geo.n);
 }
@@ -1072,13 +1069,8 @@ cudaError_t reverse_step(bool quad, bool tube, bool mrt, dim3 grid8, dim3 grid3,
                          const double* gt, const double* in, double* out, double* tb, const double* fw,
                          const double* g_prev, double* fw_prev, const AGeo& geo, const StepConst& k, int lanes) {
   if (quad) {
-    if (tube) {
-      if (mrt) launch_after(grid8, 64, st, early, k_adj_step_ws<true, FIRST, true>, gt, in, out, tb, fw, g_prev, fw_prev, geo, k);
-      else launch_after(grid8, 64, st, early, k_adj_step_ws<false, FIRST, true>, gt, in, out, tb, fw, g_prev, fw_prev, geo, k);
-    } else {
-      if (mrt) launch_after(grid8, 64, st, early, k_adj_step_ws<true, FIRST, false>, gt, in, out, tb, fw, g_prev, fw_prev, geo, k);
-      else launch_after(grid8, 64, st, early, k_adj_step_ws<false, FIRST, false>, gt, in, out, tb, fw, g_prev, fw_prev, geo, k);
-    }
+    if (mrt) launch_after(grid8, 64, st, early, k_adj_step_ws<true, FIRST>, gt, in, out, tb, fw, g_prev, fw_prev, geo, k);
+    else launch_after(grid8, 64, st, early, k_adj_step_ws<false, FIRST>, gt, in, out, tb, fw, g_prev, fw_prev, geo, k);
   } else if (tube) {
     if (mrt) k_adj_step<true, FIRST, true><<<grid3, th, 0, st>>>(gt, in, out, tb, geo, k, lanes);
     else k_adj_step<false, FIRST, true><<<grid3, th, 0, st>>>(gt, in, out, tb, geo, k, lanes);
@@ -1212,13 +1204,8 @@ cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, boo
       continue;
     }
     if (a->quad && t1 == T) {   // the QFwd of the last step
-      if (tube) {
-        if (mrt) k_adj_fwd<true, true><<<grid8, 64, 0, st>>>(g_at(s, T - 1 - t0), a->fw[(T - 1) & 1], geo, h->k);
-        else k_adj_fwd<false, true><<<grid8, 64, 0, st>>>(g_at(s, T - 1 - t0), a->fw[(T - 1) & 1], geo, h->k);
-      } else {
-        if (mrt) k_adj_fwd<true, false><<<grid8, 64, 0, st>>>(g_at(s, T - 1 - t0), a->fw[(T - 1) & 1], geo, h->k);
-        else k_adj_fwd<false, false><<<grid8, 64, 0, st>>>(g_at(s, T - 1 - t0), a->fw[(T - 1) & 1], geo, h->k);
-      }
+      if (mrt) k_adj_fwd<true><<<grid8, 64, 0, st>>>(g_at(s, T - 1 - t0), a->fw[(T - 1) & 1], geo, h->k);
+      else k_adj_fwd<false><<<grid8, 64, 0, st>>>(g_at(s, T - 1 - t0), a->fw[(T - 1) & 1], geo, h->k);
       ENQ(cudaGetLastError());
     }
     for (int t = t1 - 1; t >= t0; --t) {
