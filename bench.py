@@ -397,12 +397,16 @@ def run_adjoint(args, dist, rank, ws, local):
 
 
 def adjoint_launches(T):
-    """librlb kernels of one gradient on the 1600-node tube: k_init (set_fields); T forward
-    steps; k_adj_loss; k_adj_fwd; T - nseg recompute steps (segments of K = ceil(sqrt T)
-    steps, each refilled from its checkpoint); T reverse steps; k_adj_e0; two k_rowsum."""
-    K = max(1, math.ceil(math.sqrt(T)))
-    nseg = (T + K - 1) // K
-    return 1 + T + 1 + 1 + (T - nseg) + T + 1 + 2
+    """librlb kernels of one gradient on the 1600-node tube, where H = 11 steps go into one
+    launch: k_init (set_fields); the forward run (launches end at the checkpoints, every
+    K = ceil(sqrt T) steps); k_adj_loss; per segment its recompute (one step less than it
+    has), its reverse sweep and two kernels for the rate cotangents; k_adj_e0; two k_rowsum."""
+    H, K = 11, max(1, math.ceil(math.sqrt(T)))
+    n = 1 + 1 + 1 + 2
+    for t0 in range(0, T, K):
+        m = min(K, T - t0)
+        n += 2 * math.ceil(m / H) + math.ceil((m - 1) / H) + 2
+    return n
 
 
 def time_box(args, wl, steps, dist, ws, local, min_repeats=5, min_seconds=2.0, e2e=True):
