@@ -1195,9 +1195,13 @@ cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, boo
       cudaEvent_t swept = a->ev[5 + (s & 1)];
       ENQ(cudaEventRecord(swept, st));
       ENQ(cudaStreamWaitEvent(a->cap3, swept, 0));
-      const dim3 go((unsigned)((N + kThreads - 1) / kThreads), (unsigned)(t1 - t0));
-      if (mrt) k_adj_omega<true><<<go, kThreads, 0, a->cap3>>>(g_at(s, 0), a->lamseg[s & 1], a->part, geo.nx, geo.zgx, h->k);
-      else k_adj_omega<false><<<go, kThreads, 0, a->cap3>>>(g_at(s, 0), a->lamseg[s & 1], a->part, geo.nx, geo.zgx, h->k);
+      for (int j = 0; j < t1 - t0; j += 65535) {   // steps along the grid's y
+        const dim3 go((unsigned)((N + kThreads - 1) / kThreads), (unsigned)std::min(t1 - t0 - j, 65535));
+        const double *gj = g_at(s, j), *lj = a->lamseg[s & 1] + (size_t)j * 19 * N;
+        double* pj = a->part + (size_t)j * 3 * N;
+        if (mrt) k_adj_omega<true><<<go, kThreads, 0, a->cap3>>>(gj, lj, pj, geo.nx, geo.zgx, h->k);
+        else k_adj_omega<false><<<go, kThreads, 0, a->cap3>>>(gj, lj, pj, geo.nx, geo.zgx, h->k);
+      }
       k_adj_omega_sum<<<(unsigned)((3 * N + kThreads - 1) / kThreads), kThreads, 0, a->cap3>>>(a->part, a->tb, 3 * N, t1 - t0);
       ENQ(cudaGetLastError());
       ENQ(cudaEventRecord(ev_free[s & 1], a->cap3));

@@ -1176,9 +1176,9 @@ int tube_launch_steps(const rlb_handle* h, int& core) {
   const rlb_config& c = h->cfg;
   if (h->Q != 19 || h->esize != 8 || c.ny != 1 || c.nz != 1 || h->nodes > kSmallNodes || c.eta_over_s > 0 || qsep(c))
     return 1;
-  if (c.nx <= kTubeTile) {   // one block holds the lattice
+  if (c.nx <= kTubeTile) {   // one block holds the lattice: only the launch limits the steps (9 ms here)
     core = kTubeTile;
-    return INT_MAX;
+    return 4096;
   }
   // H steps per launch cost 1.4 us / H for the launch and, per step, the chain (2.24 us) times
   // what w blocks per SM slow it down (measured: 1 block 1.0, 2 1.4, 3 1.8, 6 3.6, 9 5.7);

@@ -221,3 +221,13 @@ def test_adjoint_passes_nan_targets_on():
     assert math.isnan(loss) and bool(torch.isnan(dtau).all())
     bad = torch.isnan(de0.cpu()).reshape(-1)
     assert bool(bad[45:56].all()) and not bool(bad[:50 - T - 1].any()) and not bool(bad[50 + T + 2:].any())
+
+
+def test_adjoint_with_one_segment_of_66000_steps():
+    """A checkpoint interval beyond the 65535 blocks of a grid's y (the rate cotangents take a
+    segment's steps along it): the gradient equals the one with the default interval bit for bit."""
+    taus, T = (0.9, 0.55, 0.8), 66000
+    e, u, n, tgt = _case((1, 1, 8), "tube", 57, taus, "mrt", ZG, 3)
+    a = _gpu_grad(e, u, n, tgt, taus, "mrt", ZG, T, K=T)
+    b = _gpu_grad(e, u, n, tgt, taus, "mrt", ZG, T)
+    assert a[0] == b[0] and torch.equal(a[1], b[1]) and torch.equal(a[2], b[2])
