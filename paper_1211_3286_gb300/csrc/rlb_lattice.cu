@@ -406,7 +406,8 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? (ETA ? 8 : 14) : RLB_WS_WARPS
     if (is_g) {
       Rates r;
       gen = !eta_rates<MRT, QSEP>((long long)s_n[slot], s_e[slot], sig, Pf, E, k, r) || b;
-      s_n[slot] = gen ? 0ull : r.Omf;   // this lane alone reads N0
+      // 1 for the FP64 form: no rate is odd (0 is one: tau_f above 2^62).  This lane alone reads N0
+      s_n[slot] = gen ? 1ull : r.Omf;
       Om = r.Omv;
       CE = r.CE;
       CP = r.CP;
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? (ETA ? 8 : 14) : RLB_WS_WARPS
     asm volatile("bar.sync %0, 64;" ::"r"(1 + (is_g ? warp : warp - W)) : "memory");
     if (!is_g) {
       Om = s_n[slot];
-      gen = Om == 0;
+      gen = Om == 1;
     }
     if (gen) {
       if (is_g && valid) step_eta_general<MRT, QSEP>(src, dst, geo, k, bad, node);

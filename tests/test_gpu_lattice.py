@@ -634,3 +634,24 @@ def test_tube_steps_flag_the_non_physical_node():
         lat.check()
     assert ex.value.code == L.RLB_ENONPHYS and one.value.code == L.RLB_ENONPHYS
     lat.close()
+
+
+# ----------------------------------------------------------------------------- fixed eta/s with a frozen f
+@pytest.mark.parametrize("tau_f", [math.inf, 2.0 ** 63, 2.0 ** 40])
+@pytest.mark.parametrize("collision", ["mrt", "bgk"])
+@pytest.mark.parametrize("shape", [(1, 1, 9), (3, 5, 37), (9, 37, 130)])
+def test_eta_over_s_with_a_frozen_f(shape, collision, tau_f):
+    """tau_f so large that omega_f 2^63 is 0 (or small): f streams and g takes its rates per node.  One
+    step against the oracle with the bounds of the rates' test (no rate above 1 here)."""
+    e, ux, uy, uz, n = I.periodic_box(None, seed=82, shape=shape, e0=3 * 2.4e-7, n0=2.4e-7 / 0.0314, umax=0.2)
+    kw = dict(collision=collision, tau_f=tau_f, tau_e=0.9, tau_eps=0.9, eta_over_s=0.1)
+    f, g = O.init_populations(e, torch.stack([ux, uy, uz]), n)
+    lat = _lattice(shape, tau_v=0.9, **kw)
+    lat.load_state(torch.cat([f, g]).cuda())
+    lat.step(1)
+    lat.check()
+    s = lat.state("cpu")
+    lat.close()
+    fo, go = O.step(f, g, O.Params(**kw))
+    assert float((s[:19] - fo).abs().max()) <= 1e-13 * float(fo.abs().max())
+    assert float((s[19:] - go).abs().max()) <= 1e-13 * float(go.abs().max())
