@@ -423,7 +423,8 @@ __global__ void __launch_bounds__(64 * W, W == 1 ? (ETA ? 8 : 14) : RLB_WS_WARPS
       return;
     }
   }
-  long long c0 = (long long)(Om >> 1) - (ETA ? 1 : 0), cA = c0, cD = c0;   // 1: truncation of the product
+  // 1: truncation of the product (none for omega = 0, a frozen distribution)
+  long long c0 = (long long)(Om >> 1) - (ETA ? (long long)(Om != 0) : 0), cA = c0, cD = c0;
   long long aq[3] = {0, 0, 0};
   if (MRT && is_g) {
     // e and eps projections of g - g^eq from the class sums, at 1/8 scale

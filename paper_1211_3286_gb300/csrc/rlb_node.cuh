@@ -1782,7 +1782,8 @@ __device__ __forceinline__ void d9_relax(const D9State& s, unsigned long long D,
   // 2e-21 of itself per step against 8e-17).
   const long long rest = s.T00 - 4 * (w.KA + w.KD + SX);
   const unsigned long long Om = G ? r.Omv : r.Omf;
-  long long c0 = (long long)(Om >> 1) - 1, cA = c0, cD = c0, dq[4] = {0, 0, 0, 0};
+  // 1: truncation of the product (none for omega = 0, a frozen distribution)
+  long long c0 = (long long)(Om >> 1) - (long long)(Om != 0), cA = c0, cD = c0, dq[4] = {0, 0, 0, 0};
   if (MRT && G) {
     // class sums of g - g^eq (axis (4/3) P + sigma u^2 / 3, diagonal P / 3 + sigma u^2 / 3)
     const long long s3 = 2 * (long long)mulhi((unsigned long long)SX, kTwoThirds);

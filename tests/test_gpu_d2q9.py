@@ -270,3 +270,24 @@ def test_d2q9_negative_number_density_steps_like_the_oracle():
     fo, go = O.step(f, g, prm)
     assert float((s[:9] - fo).abs().max()) <= 1e-14 * float(fo.abs().max())
     assert float((s[9:] - go).abs().max()) <= 1e-14 * float(go.abs().max())
+
+
+def test_d2q9_streams_a_frozen_f_unchanged():
+    """tau_f infinite: after 200 steps in a periodic plane f is the initial f moved along its
+    links, but for one cut below the grid of the largest node it passes (2^-54 of the largest
+    f; the rest link takes the 8 cuts of its node)."""
+    from paper_1211_3286_gb300.lattice import Lattice
+    shape = (1, 30, 50)
+    e, ux, uy, uz, n = I.periodic_box(None, seed=63, shape=shape)
+    f, g = O.init_populations(e, torch.stack([ux, uy, torch.zeros_like(uz)]), n, "d2q9")
+    lat = Lattice(shape, collision="mrt", tau_f=float("inf"), tau_v=0.9, tau_e=0.6, tau_eps=0.7, lattice="d2q9")
+    lat.load_state(torch.cat([f, g]).cuda())
+    lat.step(200)
+    lat.check()
+    s = lat.state("cpu")[:9]
+    lat.close()
+    E, _ = O.lattice("d2q9")
+    for a in range(9):
+        want = torch.roll(f[a], shifts=[200 * int(E[a][1]), 200 * int(E[a][0])], dims=[1, 2])
+        err = float((s[a] - want).abs().max())
+        assert err <= (8 if a == 0 else 1) * 2.0 ** -54 * float(f.max()), (a, err)

@@ -655,3 +655,25 @@ def test_eta_over_s_with_a_frozen_f(shape, collision, tau_f):
     fo, go = O.step(f, g, O.Params(**kw))
     assert float((s[:19] - fo).abs().max()) <= 1e-13 * float(fo.abs().max())
     assert float((s[19:] - go).abs().max()) <= 1e-13 * float(go.abs().max())
+
+
+def test_eta_over_s_streams_a_frozen_f_unchanged():
+    """tau_f infinite: after 200 steps in a periodic box f is the initial f moved along its links.  A
+    value loses at most what lies below the grid of the largest node that it passes, 2^-56 of
+    that node's power of two; that cut is made once, so 2^-54 of the largest f bounds it (and the
+    rest link, which takes the 18 cuts of one node: 18 times that)."""
+    shape = (4, 6, 40)
+    e, ux, uy, uz, n = I.periodic_box(None, seed=83, shape=shape, e0=3 * 2.4e-7, n0=2.4e-7 / 0.0314, umax=0.2)
+    f, g = O.init_populations(e, torch.stack([ux, uy, uz]), n)
+    lat = _lattice(shape, collision="mrt", tau_f=math.inf, tau_v=0.9, tau_e=0.9, tau_eps=0.9, eta_over_s=0.1)
+    lat.load_state(torch.cat([f, g]).cuda())
+    lat.step(200)
+    lat.check()
+    s = lat.state("cpu")[:19]
+    lat.close()
+    E, _ = O.lattice("d3q19")
+    for a in range(19):
+        c = [int(v) for v in E[a]]
+        want = torch.roll(f[a], shifts=[200 * c[2], 200 * c[1], 200 * c[0]], dims=[0, 1, 2])
+        err = float((s[a] - want).abs().max())
+        assert err <= (18 if a == 0 else 1) * 2.0 ** -54 * float(f.max()), (a, err)
