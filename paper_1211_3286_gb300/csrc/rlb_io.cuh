@@ -177,10 +177,10 @@ __device__ __forceinline__ bool stored_sums(const S* __restrict__ lat, unsigned 
   } else {
     bool fast;
     s.Eg = fx::max_exponent(v, fast);
-    if (fast) g_sums<Q>([&](int a) { return fx::to_fixed_pos(v[a], s.Eg + 7); }, s);
+    if (fast) g_sums<Q>([&](int a) { return fx::to_fixed_pos(v[a], s.Eg + 6); }, s);
     else g_sums<Q>([&](int a) { return fx::grid_value(v[a], s.Eg); }, s);
     s.Ef = fx::max_exponent(w, fast);
-    if (fast) f_sum<Q>([&](int a) { return fx::to_fixed_pos(w[a], s.Ef + 7); }, s);
+    if (fast) f_sum<Q>([&](int a) { return fx::to_fixed_pos(w[a], s.Ef + 6); }, s);
     else f_sum<Q>([&](int a) { return fx::grid_value(w[a], s.Ef); }, s);
   }
   return fx::FxUnit<S>::in_range(s.Eg) && fx::FxUnit<S>::in_range(s.Ef);
@@ -201,7 +201,9 @@ __global__ void __launch_bounds__(256) k_fields(const S* __restrict__ lat, unsig
     bool ok = stored_sums<S, Q>(lat, nodes, i, s);
     UFix u;
     bool br;
-    const unsigned long long sig = fx_recover(s.T00, s.Mx, s.My, s.Mz, u, br);
+    unsigned long long R;
+    int nsh;
+    const unsigned long long sig = fx_recover(s.T00, s.Mx, s.My, s.Mz, u, br, R, nsh);
     const long long Pf = (long long)sig - s.T00;
     const unsigned long long u2 = fx::mulhi(u.ax, u.ax) + fx::mulhi(u.ay, u.ay) + fx::mulhi(u.az, u.az);   // u^2 2^62
     ok = ok && !br && Pf > 0 && u2 < (1ull << 62) - (1ull << 30);
@@ -213,9 +215,9 @@ __global__ void __launch_bounds__(256) k_fields(const S* __restrict__ lat, unsig
     const double Pd = scale_pow2(__ll2double_rn(Pf), s.Eg - B);
     e[i] = 3.0 * Pd;
     P[i] = Pd;
-    ux[i] = scale_pow2(__ll2double_rn(fx::with_sign(u.ax, u.sx)), -63);
-    uy[i] = scale_pow2(__ll2double_rn(fx::with_sign(u.ay, u.sy)), -63);
-    uz[i] = scale_pow2(__ll2double_rn(fx::with_sign(u.az, u.sz)), -63);
+    ux[i] = fx_velocity(s.Mx, R, nsh);
+    uy[i] = fx_velocity(s.My, R, nsh);
+    uz[i] = fx_velocity(s.Mz, R, nsh);
     // n = N0 / gamma: 1/gamma = sqrt(1 - u^2) as Sq 2^(-63 - h)
     int h;
     const unsigned long long Sq = fx::sqrt_one_minus((1ull << 62) - u2, h);

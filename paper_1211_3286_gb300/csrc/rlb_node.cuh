@@ -806,11 +806,13 @@ __device__ __forceinline__ void relax_links_store(const long long (&X)[19], cons
 // ---- stored populations of either precision on a node's grid (field output, totals)
 
 // Unit of the integer grid: a value is X 2^(E - bias) with E the largest biased exponent
-// of its distribution, |X| < 2^57; in_range: exponents for which the FP64 form's T00^2 (and
+// of its distribution, |X| < 2^57 (FP32) or 2^58 (19 such values stay below 2^63, and
+// populations down to 1/32 of the largest, of which slow D2Q9 flow has some below 1/16, keep all
+// their bits); in_range: exponents for which the FP64 form's T00^2 (and
 // with it what that form accepts) and every result stay normal.
 template <typename S> struct FxUnit;
 template <> struct FxUnit<double> {
-  static constexpr int bias = 1079;
+  static constexpr int bias = 1080;
   static __device__ __forceinline__ bool in_range(int E) { return E >= 543 && E <= 1503; }
 };
 template <> struct FxUnit<float> {
@@ -841,7 +843,7 @@ __device__ __forceinline__ int max_exponent(const float (&v)[N]) {
   for (int a = 0; a < N; ++a) m = max(m, __float_as_uint(v[a]) & 0x7fffffffu);
   return (int)(m >> 23);
 }
-__device__ __forceinline__ long long grid_value(double x, int E) { return to_fixed(x, E + 7); }
+__device__ __forceinline__ long long grid_value(double x, int E) { return to_fixed(x, E + 6); }
 // 24-bit significand at 2^33 times the value's distance from the grid's top exponent
 __device__ __forceinline__ long long grid_value(float x, int E) {
   const unsigned b = __float_as_uint(x);
@@ -936,16 +938,16 @@ __device__ __forceinline__ void ufix_products(UFix& u) {
 // the square root and the reciprocal act on numbers in a fixed binary range: an FP32
 // seed each, then two Newton steps on 64-bit products (sigma within a few grid units,
 // u within 2^-58).  Returns sigma on the grid and |u_i| 2^63 with sign bits in u; sets
-// bad for T00 <= 0 or |M| >= T00 (|u| >= 1).
+// bad for T00 <= 0 or |M| >= T00 (|u| >= 1).  R and nsh: u_i = (3/2) |M_i| R 2^(nsh - 127).
 __device__ __forceinline__ unsigned long long fx_recover(long long T00, long long Mx, long long My, long long Mz,
-                                                         UFix& u, bool& bad) {
+                                                         UFix& u, bool& bad, unsigned long long& R, int& nsh) {
   using namespace fx;
   const unsigned long long amx = (unsigned long long)(Mx < 0 ? -Mx : Mx);
   const unsigned long long amy = (unsigned long long)(My < 0 ? -My : My);
   const unsigned long long amz = (unsigned long long)(Mz < 0 ? -Mz : Mz);
   const unsigned long long T = T00 > 0 ? (unsigned long long)T00 : 1ull;
   bool badr = (T00 <= 0) | (amx >= T) | (amy >= T) | (amz >= T);
-  const int nsh = __clzll((long long)T);                       // >= 2: T00 < 2^62
+  nsh = __clzll((long long)T);                                 // >= 1: T00 < 2^63
   const unsigned long long Tn = T << nsh;
   const unsigned long long mxn = badr ? 0ull : amx << nsh, myn = badr ? 0ull : amy << nsh,
                            mzn = badr ? 0ull : amz << nsh;
@@ -959,7 +961,7 @@ __device__ __forceinline__ unsigned long long fx_recover(long long T00, long lon
   const unsigned long long Sq = mulhi(a, Y) << 3;              // sqrt(A/4) 2^nsh, in (2^62, 2^64)
   const unsigned long long h = (Tn >> 1) + (Sq >> 1);          // H 2^(nsh - 1), in (1.5 2^62, 2^64)
   // R = 2^126 / h: R <- R (2 - h R 2^-126)
-  const unsigned long long R = rcp_fixed(h);
+  R = rcp_fixed(h);
   // |u_i| 2^63 = (3/4)(|M_i| 2^nsh / h) 2^63 = (3/2) mulhi(|M_i| 2^nsh, R)
   const unsigned long long ux = mulhi(mxn, R), uy = mulhi(myn, R), uz = mulhi(mzn, R);
   u.ax = ux + (ux >> 1);
@@ -971,6 +973,24 @@ __device__ __forceinline__ unsigned long long fx_recover(long long T00, long lon
   bad = badr;
   // sigma = 2H/3 = (4/3) h 2^(1 - nsh)
   return mulhi(h, kTwoThirds) >> (nsh - 1);
+}
+__device__ __forceinline__ unsigned long long fx_recover(long long T00, long long Mx, long long My, long long Mz,
+                                                         UFix& u, bool& bad) {
+  unsigned long long R;
+  int nsh;
+  return fx_recover(T00, Mx, My, Mz, u, bad, R, nsh);
+}
+// A velocity component in FP64 from its momentum and the recovery's R and nsh.  u on the 2^-63
+// grid is as good as the populations are, but has few digits left in slow flow (u of 1e-9 to
+// 6e-10 of itself, where FP64 arithmetic on the same populations gives 3e-16); with |M_i|'s own
+// top bit at 2^63 the product keeps them.
+__device__ __forceinline__ double fx_velocity(long long M, unsigned long long R, int nsh) {
+  using namespace fx;
+  const unsigned neg = (unsigned)((unsigned long long)M >> 63);
+  const unsigned long long a = with_sign((unsigned long long)M, neg);
+  const int lz = __clzll((long long)(a | 1ull));
+  const unsigned long long p = mulhi(a << lz, R);                // below 2^64 2/3
+  return scale_pow2(__ll2double_rn(with_sign((p >> 1) + (p >> 2), neg)), nsh - lz - 62);
 }
 
 // g half of the integer-pipe FP64 collide: block exponent, fixed-point values, the
