@@ -678,7 +678,21 @@ struct RevU {
   unsigned long long ax[kTubeTile], ay[kTubeTile], az[kTubeTile];
   unsigned sg[kTubeTile];
 };
-__device__ __forceinline__ long long mul_s(long long a, long long b) { return __mul64hi(a, b); }
+// a b / 2^64, to the nearest.  Rounded, the walk's error is 0.64 x 2^-53 of the node's largest
+// |lambda| (rms over random lambda and u, MRT; FP64 arithmetic: 1.67) with no bias; products cut
+// off below gave 2.5 with a bias of -1.9, which added up over the steps.
+__device__ __forceinline__ long long mul_s(long long a, long long b) {
+  const unsigned a0 = (unsigned)a, a1 = (unsigned)((unsigned long long)a >> 32), b0 = (unsigned)b,
+                 b1 = (unsigned)((unsigned long long)b >> 32);
+  const unsigned long long t = (unsigned long long)a0 * b1 + ((unsigned long long)__umulhi(a0, b0) + 0x80000000ull);
+  const unsigned long long m = (unsigned long long)a1 * b0 + (unsigned)t;
+  const unsigned long long hi = (unsigned long long)a1 * b1 + ((t >> 32) + (m >> 32));
+  return (long long)(hi - ((unsigned long long)(a >> 63) & (unsigned long long)b) -
+                     ((unsigned long long)(b >> 63) & (unsigned long long)a));
+}
+// x / 2^K, to the nearest
+template <int K>
+__device__ __forceinline__ long long half_up(long long x) { return (x + (1ll << (K - 1))) >> K; }
 
 // Cotangents of one node's pulled populations from those of its relaxed ones (v, lane
 // (m, j)'s six links; lane 3 the rest link), in place.  W62 = omega_v 2^62.
@@ -717,33 +731,31 @@ __device__ __forceinline__ void quad_vjp(int lane, double (&v)[6], const RevU& r
     S[p] = mul_s((p1 + 2 * o3) << 3, cc[p]);                                     // c (c ev + 2 od / 3)
     Q[p] = p1 + o3;
   }
-  const long long hS = (Q[1] >> 1) + (Q[2] >> 1), hD = (Q[1] >> 1) - (Q[2] >> 1);
+  const long long hS = Q[1] + Q[2], hD = Q[1] - Q[2];
   const long long KA = quad_sum64(pairs ? ev[0] : 0), KD = quad_sum64(pairs ? ev[1] + ev[2] : 0);
-  const long long SW = quad_sum64(pairs ? S[0] + ((S[1] + S[2]) >> 1) : 0);      // 4 times the density's cotangent
-  const long long Bx = quad_sum64(j == 0 ? Q[0] + hS : (j == 2 ? hS : 0));       // as the momentum sums of quad_collide
-  const long long By = quad_sum64(j == 0 ? hD : (j == 1 ? Q[0] + hS : 0));
-  const long long Bz = quad_sum64(j == 1 ? hD : (j == 2 ? Q[0] + hD : 0));
+  const long long SW = quad_sum64(pairs ? 2 * S[0] + S[1] + S[2] : 0);           // 8 times the density's cotangent
+  const long long Bx = quad_sum64(j == 0 ? 2 * Q[0] + hS : (j == 2 ? hS : 0));   // twice the momentum sums of quad_collide
+  const long long By = quad_sum64(j == 0 ? hD : (j == 1 ? 2 * Q[0] + hS : 0));
+  const long long Bz = quad_sum64(j == 1 ? hD : (j == 2 ? 2 * Q[0] + hD : 0));
   const auto om = [W62](long long x) { return mul_s(x << 2, W62); };             // omega x
   long long gq = om(l0);                                                         // of g^eq_0
   const long long kg = om(mul_s(2 * KA + KD, (long long)k36th));                 // of 3P - 1.5 sigma u^2
-  long long sb = om(SW >> 2), Sab = 0, Sdb = 0, Pb = 0, s2 = 0, h0 = 0;
+  long long sb = mul_s(SW, W62 >> 1), Sab = 0, Sdb = 0, Pb = 0, h0 = 0;
   if (MRT) {
-    const long long a16 = 30 * (l0 >> 4) + 11 * (KA >> 4) - 8 * (KD >> 4);
-    const long long p16 = 4 * (KA >> 4) - (KD >> 4) - 12 * (l0 >> 4);
-    const long long e8 = mul_s(a16, k.CE) >> 2, p8 = mul_s(p16 << 2, k.CP);      // 8 ce (..), 8 cp (..)
-    h0 = (12 * p8 - 30 * e8) >> 3;
-    Sab = -((11 * e8 + 4 * p8) >> 3);
-    Sdb = (8 * e8 + p8) >> 3;
+    const long long a2 = 15 * l0 + 11 * (KA >> 1) - 4 * KD, p4 = KA - (KD >> 2) - 3 * l0;
+    const long long e8 = half_up<5>(mul_s(a2, k.CE)), p8 = mul_s(p4, k.CP);      // 8 ce (..), 8 cp (..)
+    h0 = half_up<3>(12 * p8 - 30 * e8);
+    Sab = -half_up<3>(11 * e8 + 4 * p8);
+    Sdb = half_up<3>(8 * e8 + p8);
     gq -= h0;
     Pb = -Sab - Sdb;
-    s2 = -(Sdb >> 1);
   }
   sb += gq;
-  s2 -= (gq + 3 * kg) >> 1;                                                      // of sigma u^2
+  const long long s2 = -Sdb - (gq + 3 * kg);                                     // of sigma u^2, twice
   Pb += 3 * (kg - gq);
-  sb += mul_s(s2 << 2, (long long)u2);
-  const long long bx = (om(Bx) >> 1) + 2 * mul_s(s2 << 2, ux), by = (om(By) >> 1) + 2 * mul_s(s2 << 2, uy),
-                  bz = (om(Bz) >> 1) + 2 * mul_s(s2 << 2, uz);                   // of u, per sigma
+  sb += mul_s(s2 << 1, (long long)u2);
+  const long long bx = mul_s(Bx, W62) + mul_s(s2 << 2, ux), by = mul_s(By, W62) + mul_s(s2 << 2, uy),
+                  bz = mul_s(Bz, W62) + mul_s(s2 << 2, uz);                      // of u, per sigma
   sb += Pb;
   sb -= mul_s(bx << 2, ux) + mul_s(by << 2, uy) + mul_s(bz << 2, uz);
   const long long r = (long long)(rcp_fixed((3ull << 62) - u2) >> 1);            // 2 / (3 - u^2) 2^62

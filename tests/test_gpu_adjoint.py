@@ -231,3 +231,17 @@ def test_adjoint_with_one_segment_of_66000_steps():
     a = _gpu_grad(e, u, n, tgt, taus, "mrt", ZG, T, K=T)
     b = _gpu_grad(e, u, n, tgt, taus, "mrt", ZG, T)
     assert a[0] == b[0] and torch.equal(a[1], b[1]) and torch.equal(a[2], b[2])
+
+
+@pytest.mark.parametrize("collision", ["mrt", "bgk"])
+def test_gradient_is_odd_in_the_misfit_weights(collision):
+    """-w_P, -w_u give the negated gradient but for the walk's roundings, which carry no sign: at most
+    about 0.64 x 2^-53 of a node's |lambda| (rms) per reverse step, 200 steps of them in quadrature
+    14 times that, three standard deviations and |lambda| up to twice |dJ/de0|: 64 x 2^-53.
+    Products cut off downwards would add up to some 700 x 2^-53."""
+    taus = (0.9, 0.55, 0.8) if collision == "mrt" else (0.9, 0.9, 0.9)
+    e, u, n, tgt = _case((1, 1, 48), "tube", 59, taus, collision, ZG, 200)
+    a = _gpu_grad(e, u, n, tgt, taus, collision, ZG, 200)
+    b = _gpu_grad(e, u, n, tgt, taus, collision, ZG, 200, w_P=-1.0, w_u=-1.0)
+    assert b[0] == -a[0]
+    assert float((a[2] + b[2]).abs().max()) <= 64 * 2.0 ** -53 * float(a[2].abs().max())
