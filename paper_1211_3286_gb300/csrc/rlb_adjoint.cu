@@ -664,10 +664,11 @@ __global__ void __launch_bounds__(64) k_adj_step_ws(const double* __restrict__ g
 // mu = C_h^T lambda depends on the forward state through u alone: with the cotangents of u
 // taken per sigma, every coefficient of the walk back through the collide is dimensionless
 // (r = sigma / sqrt(A) = 2 / (3 - u^2), T00 / sigma = (3 + u^2) / 4).  The walk runs in 64-bit
-// block fixed point on the grid of the node's largest |lambda| (unit 2^-54 to 2^-55 of it),
-// where an addition costs two issue slots instead of the 64 cycles that an FP64 instruction
-// holds its unit.  The omega cotangents, which do multiply g by lambda, leave this chain: the
-// lambda of every step is stored, and k_adj_omega forms them for a whole segment at once.
+// block fixed point on the grid of the node's largest |lambda| (unit 2^-55 to 2^-56 of it; every
+// intermediate stays below 2^62.6 for any u and any admissible rates), where an addition costs
+// two issue slots instead of the 64 cycles that an FP64 instruction holds its unit.  The omega
+// cotangents, which do multiply g by lambda, leave this chain: the lambda of every step is
+// stored, and k_adj_omega forms them for a whole segment at once.
 //
 // A block holds kTubeTile nodes as k_tube_steps does (tiles that overlap by one node per
 // step): warps 0..3 hold lambda, four lanes per node, and warp 4 recovers u of the next
@@ -678,9 +679,9 @@ struct RevU {
   unsigned long long ax[kTubeTile], ay[kTubeTile], az[kTubeTile];
   unsigned sg[kTubeTile];
 };
-// a b / 2^64, to the nearest.  Rounded, the walk's error is 0.64 x 2^-53 of the node's largest
+// a b / 2^64, to the nearest.  Rounded, the walk's error is 0.4 x 2^-53 of the node's largest
 // |lambda| (rms over random lambda and u, MRT; FP64 arithmetic: 1.67) with no bias; products cut
-// off below gave 2.5 with a bias of -1.9, which added up over the steps.
+// off below on a grid half as fine gave 2.5 with a bias of -1.9, which added up over the steps.
 __device__ __forceinline__ long long mul_s(long long a, long long b) {
   const unsigned a0 = (unsigned)a, a1 = (unsigned)((unsigned long long)a >> 32), b0 = (unsigned)b,
                  b1 = (unsigned)((unsigned long long)b >> 32);
@@ -706,11 +707,11 @@ __device__ __forceinline__ void quad_vjp(int lane, double (&v)[6], const RevU& r
   for (int sl = 0; sl < 6; ++sl) me = max(me, (unsigned)__double2hiint(v[sl]) & 0x7fffffffu);
   me = max(me, (unsigned)__shfl_xor_sync(0xffffffffu, (int)me, 1));
   me = max(me, (unsigned)__shfl_xor_sync(0xffffffffu, (int)me, 2));
-  const bool finite = me < 0x7f000000u;   // else (NaN, infinities, above 1e304) the node comes out NaN
-  const int E = finite ? max((int)(me >> 20), 128) : 1023;
+  const bool finite = me < 0x7ff00000u;   // else the node comes out NaN
+  const int E = finite ? max((int)(me >> 20), 64) : 1023;   // tiny weights: see rlb_adjoint
   long long L[6];
 #pragma unroll
-  for (int sl = 0; sl < 6; ++sl) L[sl] = to_fixed(v[sl], E + 9);   // |L| < 2^55
+  for (int sl = 0; sl < 6; ++sl) L[sl] = to_fixed(v[sl], E + 8);   // |L| < 2^56
   const long long l0 = __shfl_sync(0xffffffffu, L[0], base + 3);
   // u_i 2^62 and the pairs' c.u at 2^61
   const unsigned sg = ru.sg[i];
@@ -771,13 +772,22 @@ __device__ __forceinline__ void quad_vjp(int lane, double (&v)[6], const RevU& r
       const long long t = (p == 0 ? Sab : Sdb) + T;
       long long ya = L[2 * p] - om(L[2 * p]) + t, yb = L[2 * p + 1] - om(L[2 * p + 1]) + t;
       asm("" : "+l"(ya), "+l"(yb));   // sums kept apart, as in relax_links_store
-      v[2 * p] = finite ? from_fixed_rn(ya + d[p], E + 2) : nan;
-      v[2 * p + 1] = finite ? from_fixed_rn(yb - d[p], E + 2) : nan;
+      v[2 * p] = finite ? from_fixed_rn(ya + d[p], E + 1) : nan;
+      v[2 * p + 1] = finite ? from_fixed_rn(yb - d[p], E + 1) : nan;
     }
   } else {
-    v[0] = finite ? from_fixed_rn(l0 - om(l0) + T + h0, E + 2) : nan;
+    v[0] = finite ? from_fixed_rn(l0 - om(l0) + T + h0, E + 1) : nan;
 #pragma unroll
     for (int sl = 1; sl < 6; ++sl) v[sl] = v[0];
+  }
+  if (E > 2032) {   // a sum beyond the format: its exponent has passed 0x7ff into the sign bit
+#pragma unroll
+    for (int sl = 0; sl < 6; ++sl) {
+      const unsigned hi = (unsigned)__double2hiint(v[sl]), f = (hi >> 20) & 0x7ffu;
+      const bool past = f < 16u && (hi | (unsigned)__double2loint(v[sl])) != 0;
+      if (finite && (past || f == 0x7ffu))
+        v[sl] = __hiloint2double((int)(((hi ^ (past ? 0x80000000u : 0u)) & 0x80000000u) | 0x7ff00000u), 0);
+    }
   }
 }
 
@@ -971,9 +981,10 @@ __global__ void __launch_bounds__(kThreads) k_adj_loss(const double* __restrict_
 
 // dJ/de0 of an equilibrium initial state: g^0 is linear in e0, so sum_a lambda_a g0_a / e0.
 // dJ/de0 at node (x, y, z): lambda^0 = S^T mu^0 gathered at the node, contracted with
-// dg^eq/de of the initial state (g^eq is homogeneous of degree 1 in e at fixed u).
+// dg^eq/de of the initial state (g^eq is homogeneous of degree 1 in e at fixed u).  unit: a power
+// of two that the misfit weights were divided by.
 __global__ void __launch_bounds__(kThreads) k_adj_e0(const double* __restrict__ g0, const double* __restrict__ mu,
-                                                    double* __restrict__ de0, AGeo geo, int lanes) {
+                                                    double* __restrict__ de0, double unit, AGeo geo, int lanes) {
   const int x = blockIdx.x * lanes + threadIdx.x;
   if ((int)threadIdx.x >= lanes || x >= geo.nx) return;
   const int y = blockIdx.y, z = blockIdx.z;
@@ -989,7 +1000,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_e0(const double* __restrict__ 
   GFwd F;
   StepConst dummy{};
   gforward(h, dummy, false, F);
-  de0[i] = acc / (3.0 * F.P);
+  de0[i] = acc / (3.0 * F.P) * unit;
 }
 
 // Deterministic sums of `rows` arrays of length n (one block per row).
@@ -1095,7 +1106,7 @@ cudaError_t reverse_step(bool quad, bool tube, bool mrt, dim3 grid8, dim3 grid3,
 
 // Enqueue the whole gradient computation on stream st (the handle's, or the plan's stream
 // whose work is being captured).
-cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, bool mrt, cudaStream_t st) {
+cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, double unit, bool mrt, cudaStream_t st) {
   const unsigned long long N = h->nodes;
   const size_t state_bytes = 38 * N * sizeof(double);
   const int T = a->nsteps, K = a->K, th = a->threads;
@@ -1258,7 +1269,7 @@ cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, boo
   ENQ(cudaStreamWaitEvent(st, ev_fork, 0));
   if (many) ENQ(cudaStreamWaitEvent(st, ev_free[0], 0));   // segment 0's omega cotangents, the last of that stream
   ENQ(cudaGetLastError());
-  k_adj_e0<<<grid3, th, 0, st>>>((const double*)a->ckpt[0] + 19 * N, mu_cur, a->dde0, geo, lanes);
+  k_adj_e0<<<grid3, th, 0, st>>>((const double*)a->ckpt[0] + 19 * N, mu_cur, a->dde0, unit, geo, lanes);
   k_rowsum<<<3, 256, 0, st>>>(a->tb, N, a->sums);
   k_rowsum<<<1, 256, 0, st>>>(a->lossn, N, a->sums + 3);
   ENQ(cudaGetLastError());
@@ -1373,9 +1384,16 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
   // lattice per gradient, as the autograd function does, would not use a graph twice: 800
   // nodes x 400 steps 5.1 -> 3.6 ms per call with the plan's buffers in one allocation).
   const bool direct = a->most > 1 || a->runs++ == 0;
+  // The integer walk keeps cotangents down to 2^-959: tiny weights are brought near 1 by a power
+  // of two (the gradient is linear in them) and the results taken back.
+  int up = 0;
+  if (a->most > 1) {
+    const double big = std::max(std::fabs(w_P), std::fabs(w_u));
+    if (big > 0.0 && big < 0x1p-400) up = -std::ilogb(big);
+  }
   const long long steps_before = h->steps;
   if (direct) {
-    const cudaError_t de = enqueue_adjoint(h, a, w_P, w_u, mrt, st);
+    const cudaError_t de = enqueue_adjoint(h, a, std::ldexp(w_P, up), std::ldexp(w_u, up), std::ldexp(1.0, -up), mrt, st);
     if (de != cudaSuccess) {
       h->cur = a->start_cur;
       h->steps = steps_before;
@@ -1388,7 +1406,7 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
     if (a->graph) { cudaGraphDestroy(a->graph); a->graph = nullptr; }
     const long long steps0 = h->steps;
     ACUDA(cudaStreamBeginCapture(a->cap, cudaStreamCaptureModeThreadLocal));
-    cudaError_t ce = enqueue_adjoint(h, a, w_P, w_u, mrt, a->cap);
+    cudaError_t ce = enqueue_adjoint(h, a, w_P, w_u, 1.0, mrt, a->cap);
     cudaGraph_t g = nullptr;
     cudaError_t ee = cudaStreamEndCapture(a->cap, &g);
     h->cur = a->start_cur;   // nothing ran yet
@@ -1424,12 +1442,12 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
   }
   // omega = 1 / tau  =>  dJ/dtau = -omega^2 dJ/domega
   const double wv = 1.0 / h->cfg.tau_v;
-  *loss = hs[3];
-  dtau[0] = -wv * wv * hs[0];
+  *loss = std::ldexp(hs[3], -up);
+  dtau[0] = std::ldexp(-wv * wv * hs[0], -up);
   if (mrt) {
     const double we = 1.0 / h->cfg.tau_e, wp = 1.0 / h->cfg.tau_eps;
-    dtau[1] = -we * we * hs[1];
-    dtau[2] = -wp * wp * hs[2];
+    dtau[1] = std::ldexp(-we * we * hs[1], -up);
+    dtau[2] = std::ldexp(-wp * wp * hs[2], -up);
   } else {
     dtau[1] = 0.0;
     dtau[2] = 0.0;

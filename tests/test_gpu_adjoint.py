@@ -245,3 +245,20 @@ def test_gradient_is_odd_in_the_misfit_weights(collision):
     b = _gpu_grad(e, u, n, tgt, taus, collision, ZG, 200, w_P=-1.0, w_u=-1.0)
     assert b[0] == -a[0]
     assert float((a[2] + b[2]).abs().max()) <= 64 * 2.0 ** -53 * float(a[2].abs().max())
+
+
+@pytest.mark.parametrize("collision", ["mrt", "bgk"])
+def test_gradient_scales_with_the_misfit_weights_over_the_number_range(collision):
+    """The gradient is linear in (w_P, w_u): powers of two that bring its largest component to
+    2^1012, 2^-905 and 2^-1000 scale loss and gradients exactly, but for one rounding of what
+    ends below the normal numbers."""
+    taus = (0.9, 0.55, 0.8) if collision == "mrt" else (0.9, 0.9, 0.9)
+    e, u, n, tgt = _case((1, 1, 40), "tube", 58, taus, collision, ZG, 25)
+    base = _gpu_grad(e, u, n, tgt, taus, collision, ZG, 25)
+    top = math.frexp(float(base[2].abs().max()))[1]
+    for target in (1012, -905, -1000):
+        w = 2.0 ** ((target - top) // 2)   # in two factors, each of them normal
+        v = 2.0 ** ((target - top) - (target - top) // 2)
+        got = _gpu_grad(e, u, n, tgt, taus, collision, ZG, 25, w_P=w * v, w_u=w * v)
+        assert got[0] == base[0] * w * v
+        assert torch.equal(got[1], base[1] * w * v) and torch.equal(got[2], base[2] * w * v), target
