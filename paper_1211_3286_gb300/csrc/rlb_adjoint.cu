@@ -907,10 +907,11 @@ __global__ void __launch_bounds__(32 * (kTubeWarps + 1))
 }
 
 // The omega cotangents of every node and step of a segment (blockIdx.y: the step), from its
-// states and stored lambdas, and their sum over the steps in the order of the sweep.
+// states and stored lambdas, and their sum over the steps in the order of the sweep.  A node's
+// three cotangents take the place of its first three lambdas, which this thread alone reads.
 template <bool MRT>
-__global__ void __launch_bounds__(kThreads) k_adj_omega(const double* __restrict__ g, const double* __restrict__ lam,
-                                                       double* __restrict__ part, int nx, int zg, StepConst k) {
+__global__ void __launch_bounds__(kThreads) k_adj_omega(const double* __restrict__ g, double* __restrict__ lam, int nx,
+                                                       int zg, StepConst k) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= nx) return;
   const unsigned long long n = (unsigned long long)nx, off = blockIdx.y * 19ull * n;
@@ -940,17 +941,17 @@ __global__ void __launch_bounds__(kThreads) k_adj_omega(const double* __restrict
     wpb = F.np * (fma(4.0, KAb, -KDb) - 12.0 * lo[0]) * (1.0 / 252.0);
     wvb -= web + wpb;
   }
-  double* p = part + blockIdx.y * 3ull * n + x;
+  double* p = lam + off + x;
   p[0] = wvb;
   p[n] = web;
   p[2 * n] = wpb;
 }
 __global__ void __launch_bounds__(kThreads) k_adj_omega_sum(const double* __restrict__ part, double* __restrict__ tb,
-                                                           unsigned long long n3, int steps) {
+                                                           unsigned long long n, int steps) {
   const unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-  if (i >= n3) return;
+  if (i >= 3 * n) return;
   double acc = tb[i];
-  for (int s = steps - 1; s >= 0; --s) acc += part[(unsigned long long)s * n3 + i];
+  for (int s = steps - 1; s >= 0; --s) acc += part[(unsigned long long)s * 19ull * n + i];
   tb[i] = acc;
 }
 
@@ -1039,7 +1040,7 @@ struct AdjPlan {
   double *lam = nullptr, *mu = nullptr, *tb = nullptr, *lossn = nullptr, *sums = nullptr, *dde0 = nullptr;
   double* fw[2] = {nullptr, nullptr};         // QFwd of alternate reverse steps (two warp roles)
   double* tgt = nullptr;
-  double *lamseg[2] = {nullptr, nullptr}, *part = nullptr;   // quasi-1D: stored lambdas, omega cotangents per step
+  double* lamseg[2] = {nullptr, nullptr};     // quasi-1D: stored lambdas, then omega cotangents per step
   cudaStream_t cap3 = nullptr;                // the omega cotangents beside the sweep of the next segment
   cudaStream_t cap = nullptr;
   cudaStream_t cap2 = nullptr;                // recompute of segment s - 1 beside the reverse sweep of s
@@ -1220,12 +1221,12 @@ cudaError_t enqueue_adjoint(rlb_handle* h, AdjPlan* a, double wP, double wu, dou
       ENQ(cudaStreamWaitEvent(a->cap3, swept, 0));
       for (int j = 0; j < t1 - t0; j += 65535) {   // steps along the grid's y
         const dim3 go((unsigned)((N + kThreads - 1) / kThreads), (unsigned)std::min(t1 - t0 - j, 65535));
-        const double *gj = g_at(s, j), *lj = a->lamseg[s & 1] + (size_t)j * 19 * N;
-        double* pj = a->part + (size_t)j * 3 * N;
-        if (mrt) k_adj_omega<true><<<go, kThreads, 0, a->cap3>>>(gj, lj, pj, geo.nx, geo.zgx, h->k);
-        else k_adj_omega<false><<<go, kThreads, 0, a->cap3>>>(gj, lj, pj, geo.nx, geo.zgx, h->k);
+        double* lj = a->lamseg[s & 1] + (size_t)j * 19 * N;
+        if (mrt) k_adj_omega<true><<<go, kThreads, 0, a->cap3>>>(g_at(s, j), lj, geo.nx, geo.zgx, h->k);
+        else k_adj_omega<false><<<go, kThreads, 0, a->cap3>>>(g_at(s, j), lj, geo.nx, geo.zgx, h->k);
       }
-      k_adj_omega_sum<<<(unsigned)((3 * N + kThreads - 1) / kThreads), kThreads, 0, a->cap3>>>(a->part, a->tb, 3 * N, t1 - t0);
+      k_adj_omega_sum<<<(unsigned)((3 * N + kThreads - 1) / kThreads), kThreads, 0, a->cap3>>>(a->lamseg[s & 1], a->tb, N,
+                                                                                               t1 - t0);
       ENQ(cudaGetLastError());
       ENQ(cudaEventRecord(ev_free[s & 1], a->cap3));
       continue;
@@ -1349,7 +1350,6 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
     need((void**)&a->sums, 8 * sizeof(double));
     need((void**)&a->dde0, N * sizeof(double));
     need((void**)&a->tgt, 4 * N * sizeof(double));
-    if (a->most > 1) need((void**)&a->part, (size_t)a->K * 3 * N * sizeof(double));
     for (int i = 0; i < 2 && a->quad && a->most == 1; ++i)
       need((void**)&a->fw[i], (kFwdFields + 9 * kPairFields) * N * sizeof(double));
     bool ok = plan_commit(a, want, total);

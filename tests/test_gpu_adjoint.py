@@ -262,3 +262,27 @@ def test_gradient_scales_with_the_misfit_weights_over_the_number_range(collision
         got = _gpu_grad(e, u, n, tgt, taus, collision, ZG, 25, w_P=w * v, w_u=w * v)
         assert got[0] == base[0] * w * v
         assert torch.equal(got[1], base[1] * w * v) and torch.equal(got[2], base[2] * w * v), target
+
+
+def test_gradient_of_a_tube_takes_no_more_memory_than_whole_states():
+    """Device memory of a 2000-node tube's first gradient, 4000 steps in two segments: at most the
+    two checkpoints, two buffers of K + 1 states and one more state, as with one launch per
+    step, the two cotangents and the per-node results (38 + 9 values) and 32 MiB for
+    allocation granularity."""
+    from paper_1211_3286_gb300.adjoint import misfit_gradient
+    from paper_1211_3286_gb300.lattice import Lattice
+    L, T, K = 2000, 4000, 2000
+    e, ux, uy, uz, n = (torch.from_numpy(a).cuda() for a in I.shock_tube(L))
+    lat = Lattice((1, 1, L), collision="mrt", tau_f=0.9, tau_v=0.9, tau_e=0.55, tau_eps=0.8, bc=ZG)
+    lat.set_fields(e, ux, uy, uz, n)
+    lat.step(30)
+    misfit_gradient(lat, 3, e / 3.0, ux, uy, uz)   # the kernels are loaded
+    lat.close()
+    lat = Lattice((1, 1, L), collision="mrt", tau_f=0.9, tau_v=0.9, tau_e=0.55, tau_eps=0.8, bc=ZG)
+    lat.set_fields(e, ux, uy, uz, n)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    misfit_gradient(lat, T, e / 3.0, ux, uy, uz, checkpoint_every=K)
+    used = free - torch.cuda.mem_get_info()[0]
+    lat.close()
+    assert used <= 8 * L * (38 * (2 + 2 * (K + 1) + 1) + 38 + 9) + (32 << 20), used
