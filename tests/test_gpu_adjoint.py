@@ -286,3 +286,41 @@ def test_gradient_of_a_tube_takes_no_more_memory_than_whole_states():
     used = free - torch.cuda.mem_get_info()[0]
     lat.close()
     assert used <= 8 * L * (38 * (2 + 2 * (K + 1) + 1) + 38 + 9) + (32 << 20), used
+
+
+@pytest.mark.parametrize("shape, bc, Ts", [
+    ((3, 4, 7), ("periodic", "zero_gradient", "zero_gradient"), (7, 8)),   # four lanes per node (k_adj_step_ws)
+    ((4, 100, 100), ("periodic",) * 3, (5, 6)),                            # one thread per node (k_adj_step)
+])
+@pytest.mark.parametrize("collision", ["mrt", "bgk"])
+def test_repeated_gradients_on_one_lattice_equal_fresh_ones(shape, bc, Ts, collision):
+    """A lattice's first gradient is enqueued directly, the second captures a graph, later ones
+    replay it, other weights capture it again, and another number of steps makes a new plan.
+    Loss, gradients, the state left behind and the step count equal a fresh lattice's bit for
+    bit, whichever of the handle's two buffers the state starts in."""
+    from paper_1211_3286_gb300.adjoint import misfit_gradient
+    from paper_1211_3286_gb300.lattice import Lattice
+    taus = (0.9, 0.55, 0.8) if collision == "mrt" else (0.9, 0.9, 0.9)
+
+    def lattice():
+        return Lattice(shape, collision=collision, tau_f=taus[0], tau_v=taus[0], tau_e=taus[1], tau_eps=taus[2], bc=bc)
+
+    def gradient(lat, seed, T, w, extra):
+        e, ux, uy, uz, n = (t.cuda() for t in I.periodic_box(None, seed=seed, shape=shape))
+        tgt = [(1.01 * e / 3.0), 0.9 * ux, 1.1 * uy, uz]
+        lat.set_fields(e, 0.5 * ux, 0.5 * uy, 0.5 * uz, n)
+        lat.step(extra)   # 0 or 1: the other buffer
+        loss, dtau, de0 = misfit_gradient(lat, T, *tgt, *w)
+        return torch.tensor([loss]), dtau, de0, lat.state(), torch.tensor([lat.steps_done()])
+
+    kept = lattice()
+    for T in Ts:
+        for i, w in enumerate([(1.0, 1.0)] * 4 + [(2.5, 0.5)] * 2):
+            a = gradient(kept, 90 + i, T, w, i % 2)
+            fresh = lattice()
+            b = gradient(fresh, 90 + i, T, w, i % 2)
+            fresh.close()
+            for p, q in zip(a, b):
+                assert torch.equal(p, q), (T, i)
+            assert int(a[4]) == T + i % 2
+    kept.close()

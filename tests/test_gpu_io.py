@@ -143,3 +143,20 @@ def test_velocity_output_keeps_its_relative_precision_at_any_speed(lattice, prec
         size = float(sum(w * w for w in want).sqrt())
         for k in range(3):
             assert abs(float(Decimal(float(out[k, x])) - want[k])) <= 16 * EPS * size, (x, k, size)
+
+
+def test_fp32_initial_state_is_the_fp64_equilibrium_rounded_once():
+    """The integer form's FP32 state at scale 1 against the FP64 form's (the same fields times
+    2^-70 lie outside the integer form's range), scaled back: equal bit for bit on 2^20 nodes,
+    about one in 2^13 of which has a population next to a rounding tie."""
+    from paper_1211_3286_gb300.lattice import Lattice
+    shape = (64, 128, 128)
+    e, u, n = _node_fields(shape, "d3q19", 1.0)
+    u = 0.8 * u
+    st = []
+    for scale in (1.0, 2.0 ** -70):
+        lat = Lattice(shape, collision="mrt", tau_v=0.9, tau_e=0.55, tau_eps=0.8, precision="fp32")
+        lat.set_fields((e * scale).cuda(), u[0].cuda(), u[1].cuda(), u[2].cuda(), (n * scale).cuda())
+        st.append(lat.state())
+        lat.close()
+    assert torch.equal(st[0], st[1] * 2.0 ** 70)

@@ -677,3 +677,35 @@ def test_eta_over_s_streams_a_frozen_f_unchanged():
         want = torch.roll(f[a], shifts=[200 * c[2], 200 * c[1], 200 * c[0]], dims=[0, 1, 2])
         err = float((s[a] - want).abs().max())
         assert err <= (18 if a == 0 else 1) * 2.0 ** -54 * float(f.max()), (a, err)
+
+
+def test_tube_steps_name_the_node_that_single_steps_name():
+    """A node made non-physical at the ends, at a tile's border and inside: one step names it (at
+    the open right end the node before it, which pulls the same value from the end), and five
+    steps in one call name the node that five calls of one step name."""
+    from paper_1211_3286_gb300 import _lib as L
+    for bcx in ("zero_gradient", "periodic"):
+        lat = _lattice((1, 1, 100), tau_v=0.9, tau_e=0.55, tau_eps=0.8, bc=(bcx, "periodic", "periodic"))
+        e, ux, uy, uz, n = _tube(100)
+        lat.set_fields(*(t.cuda() for t in (e, ux, uy, uz, n)))
+        lat.step(25)
+        lat.check()
+        st0 = lat.state()
+        for x in (0, 9, 10, 59, 99):
+            st = st0.clone()
+            m, p = (max(x - 1, 0), min(x + 1, 99)) if bcx == "zero_gradient" else ((x - 1) % 100, (x + 1) % 100)
+            st[19 + 1, 0, 0, m] = 1.0      # node x pulls +x from m and -x from p
+            st[19 + 2, 0, 0, p] = -0.9
+            said = []
+            for calls in ((1,), (1,) * 5, (5,)):
+                lat.load_state(st)
+                for c in calls:
+                    lat.step(c)
+                with pytest.raises(L.RlbError) as ex:
+                    lat.check()
+                assert ex.value.code == L.RLB_ENONPHYS
+                said.append(str(ex.value))
+            first = 98 if bcx == "zero_gradient" and x == 99 else x
+            assert "node %d " % first in said[0], (x, said)
+            assert said[1] == said[2], (x, said)
+        lat.close()
