@@ -323,12 +323,13 @@ struct TubeLaunch {
 // slots per tube, in powers of two up to 8, and no more threads than the longest tube has nodes.
 TubeLaunch tube_launch(const rlb_batch* b, int threads, int ctas_per_sm) {
   if (threads == 0) {
-    // No shape set: 128 threads where that leaves room for clusters of at least 2 (FP32
-    // storage) or 4 (FP64) CTAs per tube; else the widest CTAs (431 tubes FP32 17.0 -> 11.3 ms per
-    // 200 steps, 1024 26.0 -> 19.8; 160 tubes FP64 22.5 -> 14.2), but 128 again for more than
-    // 600 FP64 tubes (1024: 55.7 against 57.4 ms).
+    // No shape set: 128 threads where that leaves room for clusters of at least 2 CTAs per tube
+    // (ms per 100 steps at 128 / at the widest threads, tubes of 200-3200 nodes: FP64, 152 tubes
+    // 6.7 / 7.0, 154 10.2 / 6.9; FP32, 380 tubes 4.0 / 5.4, 382 8.3 / 5.4); else the widest CTAs, but
+    // 128 again for more than 950 FP64 tubes, whose last round is then better filled (930: 26.1 /
+    // 25.8, 960: 26.7 / 26.8, 990: 27.3 / 27.7, 1024: 28.2 / 28.7).
     const bool f32 = b->esize == 4;
-    const bool narrow = (long long)b->ntubes * (f32 ? 2 : 4) <= max_ctas(b, 128, 0) || (!f32 && b->ntubes > 600);
+    const bool narrow = b->ntubes * 2ll <= max_ctas(b, 128, 0) || (!f32 && b->ntubes > 950);
     threads = narrow ? 128 : (f32 ? RLB_TUBES_F32_THREADS : 256);
     ctas_per_sm = 0;
   }
