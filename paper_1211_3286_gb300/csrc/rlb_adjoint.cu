@@ -771,7 +771,7 @@ __device__ __forceinline__ void quad_vjp(int lane, double (&v)[6], const RevU& r
     for (int p = 0; p < 3; ++p) {
       const long long t = (p == 0 ? Sab : Sdb) + T;
       long long ya = L[2 * p] - om(L[2 * p]) + t, yb = L[2 * p + 1] - om(L[2 * p + 1]) + t;
-      asm("" : "+l"(ya), "+l"(yb));   // sums kept apart, as in relax_links_store
+      asm("" : "+l"(ya), "+l"(yb));   // as fx::relax says
       v[2 * p] = finite ? from_fixed_rn(ya + d[p], E + 1) : nan;
       v[2 * p + 1] = finite ? from_fixed_rn(yb - d[p], E + 1) : nan;
     }

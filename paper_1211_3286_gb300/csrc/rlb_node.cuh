@@ -676,6 +676,13 @@ __device__ __forceinline__ double from_fixed(long long K, int E) {
 
 // One relaxation X - omega (X - X^eq) + c with Om = omega 2^63: the biased product
 // mulhi(2 (X - X^eq) + 2^63, Om) is omega (X - X^eq) + Om / 2, and c carries + Om / 2.
+// Where a correction enters the two links of a pair with opposite signs (c + d and c - d here,
+// L - omega L +- d in the adjoint's walk), the value it is added to or subtracted from has to stay
+// a separate one, through an empty asm: ptxas 13.0 at -O1 and up, not at -O0, has lost a carry
+// between the 32-bit halves of the sum that it folded the three terms into.  Seen with d9_relax
+// (both values), the relaxation without the shift and the three-value form of relax_links_store
+// (c - d).  Every such place has a fence, and the tests compare the kernels with an unoptimised
+// build bit for bit.
 __device__ __forceinline__ long long relax(long long X, long long Xeq, unsigned long long Om, long long c) {
   const unsigned long long y = (unsigned long long)(X - Xeq) << 1;
   return X - (long long)mulhi(y ^ kSignBit, Om) + c;
@@ -740,7 +747,7 @@ __device__ __forceinline__ void relax_links(const long long (&X)[19], const EqPi
     const long long c = p < 3 ? cA : cD;
     const long long d = ODD ? dq[p] : 0;
     long long ca = c + d, cb = c - d;
-    if (ODD) asm("" : "+l"(ca), "+l"(cb));   // as in relax_links_store
+    if (ODD) asm("" : "+l"(ca), "+l"(cb));   // as relax says
     const long long ya = relax(X[2 * p + 1], ev[p] + od[p], Om, ca);
     const long long yb = relax(X[2 * p + 2], ev[p] - od[p], Om, cb);
     // (DP >> p) & 1 is a constant once the loop is unrolled
@@ -786,9 +793,8 @@ __device__ __forceinline__ void relax_links_store(const long long (&X)[19], cons
       d = p < 3 ? 4 * aq[pi[p]] : -((p & 1) ? aq[pi[p]] + aq[pj[p]] : aq[pi[p]] - aq[pj[p]]);
     }
     long long ca = c + d, cb = c - d;
-    // kept a separate value: folded into the relaxation's sum, ptxas 13.0 (-O1 and up, not
-    // -O0) can lose a carry between the 32-bit halves (a tube at rest across x then grew a
-    // transverse velocity of 1e-8)
+    // as relax says (a tube at rest across x grew a transverse velocity of 1e-8); c + d as well costs
+    // 0.7 % of a 150 x 110 x 90 step, and the unoptimised build shows no loss without it
     if (ODD) asm("" : "+l"(cb));
     const long long ya = relax_r<R>(X[2 * p + 1], ev[p] + od[p], Om, ca);
     const long long yb = relax_r<R>(X[2 * p + 2], ev[p] - od[p], Om, cb);
@@ -1836,9 +1842,7 @@ __device__ __forceinline__ void d9_relax(const D9State& s, unsigned long long D,
     if (MRT && QSEP && G) {
       ca += dq[p];
       cb -= dq[p];
-      // Both stay separate values: folded into the relaxation's sum, ptxas 13.0 (-O1 and up,
-      // not -O0) loses a carry between the 32-bit halves (link 6 off by 2^32 units on a
-      // third of all nodes).
+      // as relax says (link 6 was off by 2^32 units on a third of all nodes)
       asm("" : "+l"(ca), "+l"(cb));
     }
     const long long ya = relax(s.X[2 * p + 1], ev[p] + od[p], Om, ca);
