@@ -73,38 +73,18 @@ __device__ __forceinline__ int src_plus(int i, int n, int zg) {   // source of a
   return i < n - 1 ? i + 1 : (zg ? n - 1 : 0);
 }
 
-// Population load.  FP64 populations are streamed past L1 (each value is
-// read once per step from its plane; L2 serves the neighbouring rows' reuse), which
-// leaves L1 to the FP64 step's register spills.
-#ifndef RLB_LD_NOALLOC
-#define RLB_LD_NOALLOC 1
-#endif
+// Population load, coherent: the grid before may still be writing when this one is resident
+// (wait_for_grid).  FP64 populations are streamed past L1 (each value is read once per step
+// from its plane; L2 serves the neighbouring rows' reuse), which leaves L1 to the FP64 step's
+// register spills.  L2 prefetch size 256 B, the row segment a warp reads (512^3 FP32 step
+// 6.763 -> 6.740 ms, 256^3 FP64 step 1.859 -> 1.856 ms).
 template <typename S>
-__device__ __forceinline__ S ldg_nc(const S* p) { return __ldg(p); }
-// L2 prefetch size of the population loads: 256 B, the row segment a warp reads
-// (512^3 FP32 step 6.763 -> 6.740 ms, 256^3 FP64 step 1.859 -> 1.856 ms)
-#ifndef RLB_LD_PF
-#define RLB_LD_PF 256
-#endif
-#if RLB_LD_NOALLOC
-template <>
-__device__ __forceinline__ double ldg_nc<double>(const double* p) {
-  double v;
-  if (RLB_LD_PF == 256) asm("ld.global.L1::no_allocate.L2::256B.f64 %0, [%1];" : "=d"(v) : "l"(p));
-  else if (RLB_LD_PF == 128) asm("ld.global.L1::no_allocate.L2::128B.f64 %0, [%1];" : "=d"(v) : "l"(p));
-  else asm("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
+__device__ __forceinline__ S ld_pop(const S* p) {
+  S v;
+  if constexpr (sizeof(S) == 8) asm("ld.global.L1::no_allocate.L2::256B.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  else asm("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
   return v;
 }
-#endif
-#if RLB_LD_PF
-template <>
-__device__ __forceinline__ float ldg_nc<float>(const float* p) {
-  float v;
-  if (RLB_LD_PF == 256) asm("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  else asm("ld.global.L2::128B.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  return v;
-}
-#endif
 
 // Gather the 19 populations of one distribution arriving at node (x, y, z):
 // link a comes from (x - cx, y - cy, z - cz).
@@ -115,7 +95,7 @@ __device__ __forceinline__ void pull19(const S* __restrict__ base, unsigned long
   for (int a = 0; a < 19; ++a) {
     const int cx = link_cx(a), cy = link_cy(a), cz = link_cz(a);
     const unsigned idx = row[1 - cz][1 - cy] + (unsigned)xs[1 - cx];
-    v[a] = ldg_nc(base + (unsigned long long)a * plane + idx);
+    v[a] = ld_pop(base + (unsigned long long)a * plane + idx);
   }
 }
 
@@ -146,7 +126,7 @@ __device__ __forceinline__ void pull19(const S* __restrict__ base, unsigned long
     const int cx = link_cx(a), cy = link_cy(a), cz = link_cz(a);
     const unsigned idx = i + (unsigned)((cx > 0 ? b.xm : cx < 0 ? b.xp : 0) + (cy > 0 ? b.ym : cy < 0 ? b.yp : 0) +
                                         (cz > 0 ? b.zm : cz < 0 ? b.zp : 0));
-    v[a] = ldg_nc(base + (unsigned long long)a * plane + idx);
+    v[a] = ld_pop(base + (unsigned long long)a * plane + idx);
   }
 }
 
@@ -242,7 +222,7 @@ __device__ __noinline__ void step_eta_general(const double* __restrict__ src, do
   const Nbr3 nb = neighbours3(geo, node);
   pull19<double>(src, geo.plane, node, nb, f);
   pull19<double>(src + 19ull * geo.plane, geo.plane, node, nb, g);
-  if (node_collide_f64<MRT, QSEP, true>(f, g, k)) atomicMin(bad, (unsigned long long)node);
+  if (node_collide_f64<MRT, QSEP>(f, g, k)) atomicMin(bad, (unsigned long long)node);
 #pragma unroll
   for (int a = 0; a < 19; ++a) {
     dst[(unsigned long long)a * geo.plane + node] = f[a];
@@ -640,7 +620,7 @@ __global__ void __launch_bounds__(64, 8) k_step_quad(const double* __restrict__ 
     const int sy = cy > 0 ? ym : (cy < 0 ? yp : y);
     const int sz = cz > 0 ? zm : (cz < 0 ? zp : z);
     const unsigned idx = ((unsigned)sz * (unsigned)geo.ny + (unsigned)sy) * (unsigned)geo.nx + (unsigned)sx;
-    v[sl] = ldg_nc(src + plane0 + (unsigned long long)quad_link(j, sl) * geo.plane + idx);
+    v[sl] = ld_pop(src + plane0 + (unsigned long long)quad_link(j, sl) * geo.plane + idx);
   }
   const bool b = quad_collide<MRT, RV, RF>(is_g, lane, v, k, su, 1);
   const unsigned node = ((unsigned)z * (unsigned)geo.ny + (unsigned)y) * (unsigned)geo.nx + (unsigned)x;
@@ -765,7 +745,7 @@ __device__ __forceinline__ void pull9(const double* __restrict__ base, const Geo
   for (int a = 0; a < 9; ++a) {
     const int cx = d2_cx(a), cy = d2_cy(a);
     const unsigned i = node + (unsigned)((cx > 0 ? b.xm : cx < 0 ? b.xp : 0) + (cy > 0 ? b.ym : cy < 0 ? b.yp : 0));
-    v[a] = ldg_nc(base + (unsigned long long)a * geo.plane + i);
+    v[a] = ld_pop(base + (unsigned long long)a * geo.plane + i);
   }
 }
 
@@ -1098,9 +1078,9 @@ cudaError_t launch_step(rlb_handle* h, const void* src, void* dst, cudaStream_t 
     }
     return cudaGetLastError();
   }
-  // small lattices (a 1600-node tube) spread over more SMs with one warp per block:
-  // the FP64 pipe of an SM serves 2 lanes per clock, so fewer warps per SM means
-  // shorter steps when the lattice cannot fill the GPU anyway
+  // Lattices that cannot fill the GPU go in one-warp blocks (one warp per role), which spread
+  // over more SMs; quasi-1D FP64 ones with constant rates come here for single steps only
+  // (enqueue_tube).
   // FP32 storage: 64-thread blocks, whose finer tail suits every size (64^3 14.9 -> 14.5 us per
   // step, 100^3 52.5 -> 52.3, 256^3 820 -> 815; 96 threads 14.9, 52.7, 839)
   const int bx = h->nodes <= kSmallNodes ? 32 : sizeof(S) == 4 ? kBlockX / 2 : kBlockX;

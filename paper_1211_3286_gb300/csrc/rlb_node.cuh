@@ -37,8 +37,8 @@
 //     populations; sums, recovery (fx_recover) and per-link work in 64-bit
 //     block fixed point on the integer pipes, each output rounded once to FP64
 //     -- the FP64 step with constant relaxation times;
-//   node_collide_f64: the same update in FP64 arithmetic -- the fixed-eta/s
-//     mode, whose relaxation times vary per node;
+//   node_collide_f64: the update of the fixed-eta/s mode in FP64 arithmetic, for nodes
+//     outside the range of its integer form (eta_rates);
 //   node_collide_f32s: FP32 population storage, exact sums, recovery by one FP64
 //     Newton step on sigma's quadratic from an FP32 seed, FP32 per-link work;
 //   d9_load / d9_relax: the D2Q9 model of Sec. V.A, on the same integers;
@@ -325,8 +325,6 @@ __device__ __forceinline__ void pair_cu(C ux, C uy, C uz, C (&cu)[9]) {
   cu[7] = uy + uz; cu[8] = uy - uz;
 }
 
-// FP64 node collide: moments, recovery, equilibria, BGK f, BGK / MRT g.
-// f and g hold the pulled populations on entry and the post-collision ones on exit.
 // x * 2^e for a normal double whose scaled value stays normal (exponent add on the
 // bits); zero stays zero
 __device__ __forceinline__ double scale_pow2(double x, int e) {
@@ -430,7 +428,10 @@ __device__ __forceinline__ double tau_eta_over_s(double eta_s, const NodeMacro& 
   return 0.5 + (eta_s * s) * inv_gamma / ((1.0 / 3.0) * 4.0 * m.P);   // (e + P) = 4 P
 }
 
-template <bool MRT, bool QSEP, bool ETA = false>
+// FP64 node collide with relaxation times from a fixed eta/s: moments, recovery, rates,
+// equilibria, BGK f, BGK / MRT g.  f and g hold the pulled populations on entry and the
+// post-collision ones on exit.
+template <bool MRT, bool QSEP>
 __device__ __forceinline__ bool node_collide_f64(double (&f)[19], double (&g)[19], const StepConst& kc) {
   NodeMacro m;
   const int Eg = max_exp19_f64(g), Ef = max_exp19_f64(f);
@@ -446,12 +447,10 @@ __device__ __forceinline__ bool node_collide_f64(double (&f)[19], double (&g)[19
   const double Sd = MRT ? fixed_to_f64(X.Sd, Eg) : 0.0;
   m.bad |= (Eg == 0x7ff) || (Ef == 0x7ff);
   StepConst k = kc;
-  if (ETA) {
-    const double tv = tau_eta_over_s(kc.eta_s, m);
-    const double omv = 1.0 / tv;
-    set_bgk_coefficients(k, kc.tauf_local ? omv : kc.omf, omv);
-    if (MRT) set_mrt_eta_coefficients(k, tv, 19);
-  }
+  const double tv = tau_eta_over_s(kc.eta_s, m);
+  const double omv = 1.0 / tv;
+  set_bgk_coefficients(k, kc.tauf_local ? omv : kc.omf, omv);
+  if (MRT) set_mrt_eta_coefficients(k, tv, 19);
 
   double cu[9];
   pair_cu<double>(m.ux, m.uy, m.uz, cu);
