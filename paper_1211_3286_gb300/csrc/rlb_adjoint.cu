@@ -673,8 +673,8 @@ __global__ void __launch_bounds__(64) k_adj_step_ws(const double* __restrict__ g
 // A block holds kTubeTile nodes as k_tube_steps does (tiles that overlap by one node per
 // step): warps 0..3 hold lambda, four lanes per node, and warp 4 recovers u of the next
 // step's state, one node per lane, while they walk back through this one.  1600 nodes: 7.8 ->
-// 4.3 us per reverse step, 1600 nodes x 4000 steps 40.7 -> 27 ms per gradient; bound by the
-// dependent integer chains of the two roles.
+// 4.2 us per reverse step, 1600 nodes x 4000 steps 40.7 -> 26.7 ms per gradient; bound by the
+// dependent integer chains of the two roles (issue 25 %, fixed-latency waits).
 struct RevU {
   unsigned long long ax[kTubeTile], ay[kTubeTile], az[kTubeTile];
   unsigned sg[kTubeTile];
@@ -1379,7 +1379,7 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
                             where == RLB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st));
   }
   // Enqueued as it is, without a graph: every gradient with several steps per launch (its
-  // launches are few enough for the host to keep ahead; 1600 nodes x 4000 steps take 27.3 ms
+  // launches are few enough for the host to keep ahead; 1600 nodes x 4000 steps took 27.3 ms
   // so and 27.2 from a graph), and the first gradient of any plan (a program that makes a new
   // lattice per gradient, as the autograd function does, would not use a graph twice: 800
   // nodes x 400 steps 5.1 -> 3.6 ms per call with the plan's buffers in one allocation).

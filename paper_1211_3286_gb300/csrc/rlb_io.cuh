@@ -7,7 +7,7 @@
 // All three kernels run on 64-bit integers.  In FP64 arithmetic they were bound by the
 // FP64 pipe, which retires 2 lanes per clock and SM (ncu: 82-87 % busy, DRAM 14-28 % of
 // its peak); the integer forms leave 6 (fields), 10 (totals) and 19 (initial state)
-// FP64-pipe instructions per node.  FP32 states come out bit for bit as from the FP64
+// FP64-pipe instructions per node (totals hold 38 % of the pipe, the others 10 to 49 %).  FP32 states come out bit for bit as from the FP64
 // form.  Nodes outside the range of the integer forms
 // (exponents near the ends of the format, non-physical or invalid values) take the FP64
 // forms, which define what is accepted and what such a node's output is.
@@ -91,9 +91,11 @@ __device__ __noinline__ void fields_general(const S* __restrict__ lat, unsigned 
 // ---- initial state
 
 // f = f^eq, g = g^eq of the given FP64 fields; flags invalid input nodes.  FP64 storage
-// takes the f conversions on the integer pipe and the g conversions on the FP64 pipe, so
-// that neither holds the kernel above its memory time (256^3: 4.31 -> 1.19 ms per
-// rlb_set_fields, 512^3 with FP32 storage: 43.1 -> 10.3 ms).
+// takes the f conversions on the integer pipe and the g conversions on the FP64 pipe, which
+// shares the work between them (ALU 45 %, FP64 pipe 49 %): 256^3 4.31 -> 1.19 ms per
+// rlb_set_fields, 1.4 times its memory time, the rest fixed-latency waits at 24 % of the
+// warps.  FP32 storage, 512^3: 43.1 -> 10.3 ms, 2.7 times its memory time: bound by the ALU (67 %,
+// issue 56 %), whose work is the single rounding of 38 values with its test for ties.
 template <typename S, int Q = 19>
 __global__ void __launch_bounds__(256, 2) k_init(S* __restrict__ lat, unsigned long long nodes,
                                               const double* __restrict__ e, const double* __restrict__ ux,
@@ -187,8 +189,9 @@ __device__ __forceinline__ bool stored_sums(const S* __restrict__ lat, unsigned 
 }
 
 // Macroscopic fields of the stored state.  One thread per node, bound by the memory it
-// reads: 256^3 FP64 3.21 -> 0.95 ms per rlb_get_fields, 512^3 FP32 storage 34.4 ->
-// 5.6 ms, against the FP64 form's 85 % busy FP64 pipe.
+// reads (FP64: 1.1 times its memory time, 256^3 3.21 -> 0.95 ms per rlb_get_fields) and by issue
+// (FP32 storage: 67 %, 1.4 times, 512^3 34.4 -> 5.6 ms), against the FP64 form's 85 % busy
+// FP64 pipe.
 template <typename S, int Q = 19>
 __global__ void __launch_bounds__(256) k_fields(const S* __restrict__ lat, unsigned long long nodes,
                                                 double* __restrict__ e, double* __restrict__ P,

@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(kBlockX, RLB_F32_BLOCKS_PER_SM) k_step(const S
 // barrier; a node outside that form's range is left to its g lane, which runs the FP64 form
 // for both distributions.  128 x 96 x 80 MRT with its own tau_q: 598 -> 182 us per step (FP64
 // arithmetic held the FP64 pipe 88 % busy with 329 instructions per node, now 46; the limit
-// is the integer instruction stream, issue 58 %).
+// is the integer instruction stream, issue 57 %, of which 400 bytes of spills per thread in
+// the tau_q form are part).
 template <bool MRT, bool QSEP>
 __device__ __noinline__ void step_eta_general(const double* __restrict__ src, double* __restrict__ dst, const Geo& geo,
                                               const StepConst& k, unsigned long long* __restrict__ bad, unsigned node) {
@@ -848,7 +849,9 @@ __global__ void __launch_bounds__(kBlockX) k_macro_d2q9(const double* __restrict
 // f is rounded on the integer pipe and g on the FP64 pipe, 9 FP64-pipe instructions per
 // node (31 with C_7), and f is pulled only when g is stored, which lets 8 blocks per SM
 // hold the launch's latency (64 registers; 5 blocks at 96 registers: 145 us with C_7).
-// 1200 x 900: 295 -> 70 us per step, with C_7 561 -> 128 (of that k_macro_d2q9 138 -> 30).
+// 1200 x 900: 295 -> 70 us per step, with C_7 561 -> 124 (k_macro_d2q9 alone 138 -> 30).  Bound by
+// issue and fixed latencies (issue 65 %, ALU 66 %), with C_7 by the FP64 pipe (71 %) and the
+// waits for the neighbours' fields.
 template <bool MRT, bool QSEP, bool CORR>
 __global__ void __launch_bounds__(kBlockX, 8) k_step_d2q9(const double* __restrict__ src, double* __restrict__ dst,
                                                        const __grid_constant__ Geo geo, const __grid_constant__ StepConst k,
