@@ -324,3 +324,23 @@ def test_repeated_gradients_on_one_lattice_equal_fresh_ones(shape, bc, Ts, colli
                 assert torch.equal(p, q), (T, i)
             assert int(a[4]) == T + i % 2
     kept.close()
+
+
+def test_gradient_past_the_format_is_infinite_with_its_sign():
+    """Weights that take dJ/de0 up to the largest double and past it, a power of two at a time: every
+    component is the exactly scaled one, an infinity of its sign, or NaN (where infinities met
+    on the way), never a finite value that has passed the format's end."""
+    taus = (0.9, 0.55, 0.8)
+    e, u, n, tgt = _case((1, 1, 40), "tube", 58, taus, "mrt", ZG, 3)
+    tgt.P += 100.0
+    base = _gpu_grad(e, u, n, tgt, taus, "mrt", ZG, 3)[2].cpu()
+    top = math.frexp(float(base.abs().max()))[1]
+    assert top > 4
+    kinds = set()
+    for k in range(1012 - top, 1024 - min(top, 3)):
+        got = _gpu_grad(e, u, n, tgt, taus, "mrt", ZG, 3, w_P=2.0 ** k, w_u=2.0 ** k)[2].cpu()
+        fine, inf = torch.isfinite(got), torch.isinf(got)
+        assert torch.equal(got[fine], (base * 2.0 ** (k // 2) * 2.0 ** (k - k // 2))[fine]), k
+        assert torch.equal(got[inf].sign(), base[inf].sign()), k
+        kinds |= {"fine" if bool(fine.all()) else "past"}
+    assert kinds == {"fine", "past"}
