@@ -1371,6 +1371,17 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
     h->adj_plan = a;
     h->adj_free = free_plan;
   }
+  // a refused call (a stream under capture: nothing has run) leaves the state where it was
+  const long long steps_before = h->steps;
+  struct Keep {
+    rlb_handle* h;
+    int cur;
+    long long steps;
+    ~Keep() {
+      h->cur = cur;
+      h->steps = steps;
+    }
+  } keep{h, h->cur, h->steps};
   // the graph's lattice pointers assume the state starts in lat[start_cur]
   if (h->cur != a->start_cur) {
     ACUDA(cudaMemcpyAsync(h->lat[a->start_cur], h->lat[h->cur], state_bytes, cudaMemcpyDeviceToDevice, st));
@@ -1396,14 +1407,9 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
     const double big = std::max(std::fabs(w_P), std::fabs(w_u));
     if (big > 0.0 && big < 0x1p-400) up = -std::ilogb(big);
   }
-  const long long steps_before = h->steps;
   if (direct) {
     const cudaError_t de = enqueue_adjoint(h, a, std::ldexp(w_P, up), std::ldexp(w_u, up), std::ldexp(1.0, -up), mrt, st);
-    if (de != cudaSuccess) {
-      h->cur = a->start_cur;
-      h->steps = steps_before;
-      return afail(h, RLB_ECUDA, std::string("adjoint launch: ") + cudaGetErrorString(de));
-    }
+    if (de != cudaSuccess) return afail(h, RLB_ECUDA, std::string("adjoint launch: ") + cudaGetErrorString(de));
   }
   // capture once per plan (the misfit weights are kernel arguments: recapture if they change)
   if (!direct && (!a->exec || a->wP != w_P || a->wu != w_u)) {
@@ -1432,8 +1438,8 @@ extern "C" int rlb_adjoint(rlb_handle* h, int nsteps, int checkpoint_every, cons
     ACUDA(cudaMemcpyAsync(de0, a->dde0, N * sizeof(double),
                           where == RLB_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, st));
   ACUDA(cudaStreamSynchronize(st));
-  h->cur = a->end_cur;
-  h->steps = steps_before + nsteps;
+  keep.cur = a->end_cur;
+  keep.steps = steps_before + nsteps;
   {
     unsigned long long bad = ~0ull;
     ACUDA(cudaMemcpy(&bad, h->d_bad, sizeof bad, cudaMemcpyDeviceToHost));

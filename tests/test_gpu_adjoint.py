@@ -344,3 +344,43 @@ def test_gradient_past_the_format_is_infinite_with_its_sign():
         assert torch.equal(got[inf].sign(), base[inf].sign()), k
         kinds |= {"fine" if bool(fine.all()) else "past"}
     assert kinds == {"fine", "past"}
+
+
+def test_gradient_refused_under_capture_leaves_the_lattice_as_it_was():
+    """A gradient synchronises, so it is refused on a stream that is being captured.  Nothing has
+    run then: the state, its place and the step count are what they were, and the next gradient
+    equals a fresh lattice's (odd and even numbers of launches)."""
+    import ctypes
+    from paper_1211_3286_gb300 import _lib as L
+    from paper_1211_3286_gb300.adjoint import misfit_gradient
+    from paper_1211_3286_gb300.lattice import Lattice
+    rt = ctypes.CDLL("libcudart.so.13")
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        e, ux, uy, uz, n = (torch.from_numpy(a).cuda() for a in I.shock_tube(60))
+        tgt = [1.01 * e / 3.0, ux + 0.01, uy, uz]
+        for T, sets in ((5, 1), (5, 2), (30, 1), (30, 2)):   # setting the fields changes the buffer
+            lat = Lattice((1, 1, 60), collision="mrt", tau_f=0.9, tau_v=0.9, tau_e=0.55, tau_eps=0.8, bc=ZG)
+            lat.set_fields(e, ux, uy, uz, n)
+            first = misfit_gradient(lat, T, *tgt)   # the plan exists
+            for _ in range(sets):
+                lat.set_fields(e, ux, uy, uz, n)
+            lat.step(3)
+            before, steps = lat.state(), lat.steps_done()
+            stream, graph = ctypes.c_void_p(s.cuda_stream), ctypes.c_void_p()
+            torch.cuda.synchronize()
+            assert rt.cudaStreamBeginCapture(stream, 2) == 0   # relaxed
+            try:
+                with pytest.raises(L.RlbError) as ex:
+                    misfit_gradient(lat, T, *tgt)
+            finally:
+                rt.cudaStreamEndCapture(stream, ctypes.byref(graph))
+                if graph:
+                    rt.cudaGraphDestroy(graph)
+                rt.cudaGetLastError()
+            assert ex.value.code == L.RLB_ECUDA
+            assert lat.steps_done() == steps and torch.equal(lat.state(), before)
+            lat.set_fields(e, ux, uy, uz, n)
+            again = misfit_gradient(lat, T, *tgt)
+            lat.close()
+            assert again[0] == first[0] and torch.equal(again[1], first[1]) and torch.equal(again[2], first[2])
