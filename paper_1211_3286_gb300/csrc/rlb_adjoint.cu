@@ -673,7 +673,7 @@ __global__ void __launch_bounds__(64) k_adj_step_ws(const double* __restrict__ g
 // A block holds kTubeTile nodes as k_tube_steps does (tiles that overlap by one node per
 // step): warps 0..3 hold lambda, four lanes per node, and warp 4 recovers u of the next
 // step's state, one node per lane, while they walk back through this one.  1600 nodes: 7.8 ->
-// 4.2 us per reverse step, 1600 nodes x 4000 steps 40.7 -> 26.7 ms per gradient; bound by the
+// 4.2 us per reverse step, 1600 nodes x 4000 steps 40.7 -> 26.4 ms per gradient; bound by the
 // dependent integer chains of the two roles (issue 25 %, fixed-latency waits).
 struct RevU {
   unsigned long long ax[kTubeTile], ay[kTubeTile], az[kTubeTile];
